@@ -1756,9 +1756,36 @@ struct qf_batch {
   int grid = 0;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
+  // the last step's end: every step of a batch writes the same workspace, so
+  // one issued on another stream waits for it
+  cudaEvent_t done = nullptr;
+  cudaStream_t last = nullptr;
+  bool stepped = false;
 };
 
 namespace {
+
+// Order a step on st after the batch's previous one (on another stream), and
+// mark its end. Steps under capture are ordered by whoever replays them.
+bool batch_capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return cs != cudaStreamCaptureStatusNone;
+}
+cudaError_t batch_begin(qf_batch* b, cudaStream_t st) {
+  if (!b->stepped || b->last == st || batch_capturing(st)) return cudaSuccess;
+  return cudaStreamWaitEvent(st, b->done, 0);
+}
+cudaError_t batch_end(qf_batch* b, cudaStream_t st) {
+  if (batch_capturing(st)) return cudaSuccess;
+  const cudaError_t e = cudaEventRecord(b->done, st);
+  b->last = st;
+  b->stepped = e == cudaSuccess;
+  return e;
+}
 
 template <class T>
 T* rel(size_t off) {  // a workspace-relative pointer (rebased by the kernels)
@@ -1769,6 +1796,8 @@ void batch_free(qf_batch* b) {
   if (b->exec) cudaGraphExecDestroy(b->exec);
   if (b->graph) cudaGraphDestroy(b->graph);
   if (b->d_tables) cudaFree(b->d_tables);
+  if (b->done) cudaEventDestroy(b->done);
+  b->done = nullptr;
   b->exec = nullptr;
   b->graph = nullptr;
   b->d_tables = nullptr;
@@ -1990,10 +2019,11 @@ qf_status qf_batch_create(int32_t n_circuits, qf_circuit* const* circuits, const
     b->prep_total = prep_pref[n_circuits];
     b->n_grad_out = gout_pref[n_circuits];
     b->grid = qf::batch_grid();
-    if (b->grid <= 0) {
+    if (b->grid <= 0 || cudaEventCreateWithFlags(&b->done, cudaEventDisableTiming) != cudaSuccess) {
+      cudaGetLastError();
       batch_free(b);
       delete b;
-      return fail(QF_ERR_CUDA, "cannot query the device's SM count");
+      return fail(QF_ERR_CUDA, "cannot query the device's SM count or make an event");
     }
   } catch (const std::bad_alloc&) {
     if (b) {
@@ -2042,7 +2072,10 @@ qf_status qf_batch_train_step(qf_batch* b, const float* theta_d, const float* x_
   a.loss = loss_d;
   a.lterm = reinterpret_cast<double*>(a.ws + b->lterm_off);
   a.queue = reinterpret_cast<int32_t*>(a.ws + b->queue_off);
-  QF_CU(qf::launch_batch(a, b->grid, b->prep_total, b->n_grad_out, static_cast<cudaStream_t>(stream)));
+  const cudaStream_t st = static_cast<cudaStream_t>(stream);
+  QF_CU(batch_begin(b, st));
+  QF_CU(qf::launch_batch(a, b->grid, b->prep_total, b->n_grad_out, st));
+  QF_CU(batch_end(b, st));
   return QF_OK;
 }
 
@@ -2075,7 +2108,10 @@ qf_status qf_batch_graph_capture(qf_batch* b, const float* theta_d, const float*
 
 qf_status qf_batch_graph_launch(qf_batch* b, void* stream) {
   if (!b || !b->exec) return fail(QF_ERR_INVALID_ARG, "no captured graph (call qf_batch_graph_capture)");
-  QF_CU(cudaGraphLaunch(b->exec, static_cast<cudaStream_t>(stream)));
+  const cudaStream_t st = static_cast<cudaStream_t>(stream);
+  QF_CU(batch_begin(b, st));
+  QF_CU(cudaGraphLaunch(b->exec, st));
+  QF_CU(batch_end(b, st));
   return QF_OK;
 }
 

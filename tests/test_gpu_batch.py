@@ -122,3 +122,22 @@ def test_mixed512_heaviest_circuits_against_oracle():
         assert np.max(np.abs(g[t0:t1] - gr)) < TOL, (c.cid, c.n, c.d)
         total += Er.sum()
     assert abs(lv.item() - total) < TOL * len(heavy)
+
+
+def test_steps_of_a_batch_on_two_streams_are_ordered():
+    """Steps of one batch share its workspace: a step issued on another stream
+    right behind one in flight gives the same bits as alone."""
+    thetas, xs, ys = make(SPECS, 9)
+    bt = Batch(SPECS, loss="mse")
+    th, x, y = cat(thetas), cat(xs), cat(ys)
+    ref = [t.clone() for t in bt.train_step(th, x, y)]
+    torch.cuda.synchronize()
+    a, b = bt.outputs(), bt.outputs()
+    stream = torch.cuda.Stream()
+    for _ in range(5):
+        bt.train_step(th, x, y, out=a)
+        with torch.cuda.stream(stream):
+            bt.train_step(th, x, y, out=b)
+    torch.cuda.synchronize()
+    for r, u, v in zip(ref, a, b):
+        assert torch.equal(r, u) and torch.equal(r, v)

@@ -1994,7 +1994,7 @@ qf_status qf_batch_create(int32_t n_circuits, qf_circuit* const* circuits, const
       r.n_params = c->circ.n_params;
       r.param_off = T.param_off;
       r.param_terms = T.param_terms;
-      prep_pref[i + 1] = prep_pref[i] + p.n_fused + p.n_terms + p.B * p.n_eff + qf::round_par_elems(p);
+      prep_pref[i + 1] = prep_pref[i] + (qf::prep_elems(p) + 31) / 32 * 32;  // whole warps
       gout_pref[i + 1] = gout_pref[i] + c->circ.n_params;
     }
     memcpy(img.data() + circ_off, recs.data(), recs.size() * sizeof(qf::BatchCircuit));

@@ -184,15 +184,17 @@ __device__ __forceinline__ void link_terms(uint32_t L, uint32_t gb, int n, uint3
 // the thread (rgb = gb rotated right by one qubit, lgb = left, g12 = gb &
 // rgb): as rotation distributes over &, u = rotl(L) & lgb ^ L & rgb (the
 // link_terms u), and the constant part is |L & g12|. When the register bits
-// sit on consecutive qubits (contig), A is one shift of u.
+// sit on consecutive qubits (contig), A is one shift of u. Register p holds
+// amplitude p ^ m (the step's bit flips, see rot_T), so the linear part of
+// amplitude j = p ^ m adds the constant |A & m|.
 __device__ __forceinline__ void chain_pending(uint32_t L, uint32_t rgb, uint32_t lgb, uint32_t g12, int n,
-                                                const uint32_t (&p)[4], bool contig, uint32_t& D) {
+                                                const uint32_t (&p)[4], bool contig, uint32_t m, uint32_t& D) {
   const uint32_t nmask = n >= 32 ? ~0u : ((1u << n) - 1u);
   const uint32_t u = ((((L << 1) | (L >> (n - 1))) & nmask) & lgb) ^ (L & rgb);
   const uint32_t A = contig ? (u >> p[0]) & 15u
                             : ((u >> p[0]) & 1u) | (((u >> p[1]) & 1u) << 1) | (((u >> p[2]) & 1u) << 2) |
                                   (((u >> p[3]) & 1u) << 3);
-  D ^= A | ((__popc(L & g12) & 1u) << 4);
+  D ^= A | ((__popc((L & g12) ^ (A & m)) & 1u) << 4);
 }
 
 // Multiply the registers by D (end of a step).
@@ -215,50 +217,53 @@ __device__ __forceinline__ void apply_pending(uint32_t D, float2 (&r)[16], float
   }
 }
 
-// RX(w) applied on register bit R: a rotation by -w/2 of the real pairs
-// (re p0, im p1) and (re p1, im p0), three shears each (x += t y; y -= s x;
-// x += t y). yq: the term's shear parameters (t, s, wrap parity) of the
-// un-apply direction. A pending Z_R turns RX(w) into RX(-w).
-template <int R>
-__device__ __forceinline__ void rx_fwd(float2 (&r)[16], float4 yq, uint32_t a) {
-  const int f = (int)(a << 31);
-  const float t = __int_as_float(__float_as_int(yq.x) ^ f), s = __int_as_float(__float_as_int(yq.y) ^ f);
-#pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    if (j & (1 << R)) continue;
-    const int j1 = j | (1 << R);
-    float2 p0 = r[j], p1 = r[j1];
-    p0.x = fmaf(t, p1.y, p0.x); p1.y = fmaf(-s, p0.x, p1.y); p0.x = fmaf(t, p1.y, p0.x);
-    p1.x = fmaf(t, p0.y, p1.x); p0.y = fmaf(-s, p1.x, p0.y); p1.x = fmaf(t, p0.y, p1.x);
-    r[j] = p0; r[j1] = p1;
-  }
-}
-
-// The rotation of a forward item on register bit R (RY, or RX where rx; rx is
-// uniform over the CTA): applying is the un-apply rotation the other way,
-// (t, s) -> (-t, -s). A pending Z_R turns the rotation by w into one by -w.
-// The rotation by w is u(phi) up to the sign (-1)^k of its wrap; prep folds
-// the round's signs into the round's diagonal (a global sign of the state).
+// One rotation of a round on register bit R, two FMAs per real component:
+//   RY: p0 -= q p1; p1 += q p0      RX: p0 -= i q p1; p1 -= i q p0
+// (old values on the right), i.e. [[1, -q], [q, 1]] or [[1, -iq], [-iq, 1]].
+// A rotation by w with |w| <= pi/2 is cos(w/2) times that with q = tan(w/2);
+// beyond, with k = cot(w/2), RY(w) = sin(w/2) X Z T(-k) and RX(w) =
+// -i sin(w/2) X T(-k), so |q| <= 1 for every angle. The factors of the round's
+// four rotations (scales, signs, Z's and phases) are multiplied into its
+// diagonal's 16 phases, which the kernel applies anyway; the X's are never
+// executed: they flip bits of a mask m (the same for every thread, from the
+// tables), register p of a step holding amplitude p ^ m, and the step's last
+// store puts the registers at their addresses. An RY acts on a flipped pair
+// with -q (folded into the table's q). Against rotations as three shears
+// (3 FMAs per component): forward of n = 16, d = 20, 500 samples 2.86 -> 2.57
+// ms; training step of n = 20, d = 24, 64 samples 28.35 -> 26.32 ms, of n = 12,
+// d = 20, 256 samples 268 -> 251 us.
+// A pending Z_R turns the rotation by w into one by -w, i.e. q into -q (the
+// sign of sin(w/2) moves to the pending constant: it cancels against the flip
+// of the pending sign's own index, chain_pending's |A & m|).
 template <int R, bool RX>
-__device__ __forceinline__ void rot_fwd(float2 (&r)[16], float4 yq, uint32_t a, uint32_t& D, bool rx) {
+__device__ __forceinline__ void rot_T(float2 (&r)[16], float q, bool rx) {
   if (RX && rx) {
-    rx_fwd<R>(r, yq, a);
-  } else {
-    const int f = (int)(a << 31);
-    const float tn = -__int_as_float(__float_as_int(yq.x) ^ f), sp = __int_as_float(__float_as_int(yq.y) ^ f);
-    const float2 t2 = make_float2(tn, tn), ms2 = make_float2(sp, sp);
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
       if (j & (1 << R)) continue;
       const int j1 = j | (1 << R);
-      float2 p0 = r[j], p1 = r[j1];
-      // RY(w) on (p0, p1): rotation by +w/2 as three packed shears
-      p0 = __ffma2_rn(t2, p1, p0);
-      p1 = __ffma2_rn(ms2, p0, p1);
-      p0 = __ffma2_rn(t2, p1, p0);
-      r[j] = p0; r[j1] = p1;
+      const float2 p0 = r[j], p1 = r[j1];
+      r[j] = make_float2(fmaf(q, p1.y, p0.x), fmaf(-q, p1.x, p0.y));
+      r[j1] = make_float2(fmaf(q, p0.y, p1.x), fmaf(-q, p0.x, p1.y));
+    }
+  } else {
+    // RY is real: the same on re and im, one packed FFMA2 each
+    const float2 q2 = make_float2(q, q), n2 = make_float2(-q, -q);
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      if (j & (1 << R)) continue;
+      const int j1 = j | (1 << R);
+      const float2 p0 = r[j];
+      r[j] = __ffma2_rn(n2, r[j1], p0);
+      r[j1] = __ffma2_rn(q2, p0, r[j1]);
     }
   }
+}
+
+// The rotation of a forward item (q of the round's table; a: a pending Z_R).
+template <int R, bool RX>
+__device__ __forceinline__ void rot_fwd(float2 (&r)[16], float q, uint32_t a, bool rx) {
+  rot_T<R, RX>(r, __int_as_float(__float_as_int(q) ^ (int)(a << 31)), rx);
 }
 
 // v *= (c + i s)
@@ -321,62 +326,40 @@ __device__ __forceinline__ void diag_bwd(float2 (&p)[16], float2 (&l)[16], const
   g[3] = (s2[0] + s2[1]) - (s2[2] + s2[3]);
 }
 
-// Un-apply one rotation on register bit R by three shears and return the
-// thread's sum of Im<lambda|P|psi> taken before it. A plane rotation by phi
-// equals x += a y; y += b x; x += a y with a = -tan(phi/2), b = sin(phi)
-// (exact; |a| <= 1 for |phi| <= pi/2), three FMAs per component; t =
-// tan(w/4), s = sin(w/2).
-//   RY: (x, y) <- RY(w)^dagger (x, y) = rotation by -w/2: a = t, b = -s.
-template <int R, int KIND>
-__device__ __forceinline__ float bwd_shear(float2 (&p)[16], float2 (&l)[16], const float t, const float s) {
-  float acc = 0.f;
-  float2 accp = make_float2(0.f, 0.f), accm = make_float2(0.f, 0.f);
-  const float2 t2 = make_float2(t, t), ms2 = make_float2(-s, -s);
-#pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    if (j & (1 << R)) continue;
-    const int j1 = j | (1 << R);
-    float2 p0 = p[j], p1 = p[j1], l0 = l[j], l1 = l[j1];
-    if (KIND == G_RX) {
-      // Im<lambda|X|psi> per pair; RX(w)^dagger rotates (re p0, im p1) and
-      // (re p1, im p0) by +w/2: x -= t y; y += s x; x -= t y
-      acc += l0.x * p1.y - l0.y * p1.x + l1.x * p0.y - l1.y * p0.x;
-      p0.x = fmaf(-t, p1.y, p0.x); p1.y = fmaf(s, p0.x, p1.y); p0.x = fmaf(-t, p1.y, p0.x);
-      p1.x = fmaf(-t, p0.y, p1.x); p0.y = fmaf(s, p1.x, p0.y); p1.x = fmaf(-t, p0.y, p1.x);
-      l0.x = fmaf(-t, l1.y, l0.x); l1.y = fmaf(s, l0.x, l1.y); l0.x = fmaf(-t, l1.y, l0.x);
-      l1.x = fmaf(-t, l0.y, l1.x); l0.y = fmaf(s, l1.x, l0.y); l1.x = fmaf(-t, l0.y, l1.x);
-    } else {
-      // RY is real: the same shear acts on re and im, so each step is one
-      // packed FFMA2 on the (re, im) pair; Im<lambda|Y|psi> per pair is
-      // l1 . p0 - l0 . p1 (component-wise products, two packed accumulators).
-      accp = __ffma2_rn(l1, p0, accp);
-      accm = __ffma2_rn(l0, p1, accm);
-      p0 = __ffma2_rn(t2, p1, p0);
-      p1 = __ffma2_rn(ms2, p0, p1);
-      p0 = __ffma2_rn(t2, p1, p0);
-      l0 = __ffma2_rn(t2, l1, l0);
-      l1 = __ffma2_rn(ms2, l0, l1);
-      l0 = __ffma2_rn(t2, l1, l0);
-    }
-    p[j] = p0; p[j1] = p1; l[j] = l0; l[j1] = l1;
-  }
-  if (KIND == G_RY) acc = (accp.x + accp.y) - (accm.x + accm.y);
-  return acc;
-}
-
-// The rotation of an adjoint item on register bit R (shear parameters (t, s);
-// RX where rx, uniform over the CTA, else RY), un-applied after the round's
-// diagonal; gy: its Im<lambda|P|psi>. With a pending Z_R the rotation
-// un-applies as the one by +w (t, s negated) and gy changes sign. The wrap
-// sign (u(phi) = -u(w) for odd k) is folded into the round's diagonal, which
-// multiplies psi and lambda alike (their gradient terms do not change).
+// The rotation of an adjoint item on register bit R (q un-applies it; RX where
+// rx, uniform over the CTA, else RY), after the round's diagonal; gy: the
+// thread's sum of Im<lambda|P|psi> taken before it. A pending Z_R negates q
+// and gy. The round's scales and flips multiply gy by a factor that is the
+// same for every thread and sample; the owner lane of the reduced sum undoes
+// it (the table's .y).
 template <int R, bool RX = false>
-__device__ __forceinline__ void rot_bwd(float2 (&p)[16], float2 (&l)[16], float4 yq, uint32_t a, uint32_t& D,
-                                        float& gy, bool rx = false) {
+__device__ __forceinline__ void rot_bwd(float2 (&p)[16], float2 (&l)[16], float qt, uint32_t a, float& gy,
+                                        bool rx = false) {
   const int f = (int)(a << 31);
-  const float t = __int_as_float(__float_as_int(yq.x) ^ f);
-  const float s = __int_as_float(__float_as_int(yq.y) ^ f);
-  const float g = RX && rx ? bwd_shear<R, G_RX>(p, l, t, s) : bwd_shear<R, G_RY>(p, l, t, s);
+  const float q = __int_as_float(__float_as_int(qt) ^ f);
+  float g;
+  if (RX && rx) {
+    g = 0.f;
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      if (j & (1 << R)) continue;
+      const int j1 = j | (1 << R);
+      g += l[j].x * p[j1].y - l[j].y * p[j1].x + l[j1].x * p[j].y - l[j1].y * p[j].x;
+    }
+  } else {
+    // l1 . p0 - l0 . p1 per pair (component-wise products, two packed sums)
+    float2 accp = make_float2(0.f, 0.f), accm = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      if (j & (1 << R)) continue;
+      const int j1 = j | (1 << R);
+      accp = __ffma2_rn(l[j1], p[j], accp);
+      accm = __ffma2_rn(l[j], p[j1], accm);
+    }
+    g = (accp.x + accp.y) - (accm.x + accm.y);
+  }
+  rot_T<R, RX>(p, q, rx);
+  rot_T<R, RX>(l, q, rx);
   gy = __int_as_float(__float_as_int(g) ^ f);
 }
 
@@ -434,8 +417,8 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
 // Parameters of one round step, staged from the round-ordered tables: per
-// round kRoundPar float4 (the items' rotation shears, then the round's
-// diagonal) and the round record.
+// round kRoundPar float4 (the items' rotations, then the round's diagonal) and
+// the round record.
 constexpr int kMaxRoundWords = kFwdRoundWords > kBwdRoundWords ? kFwdRoundWords : kBwdRoundWords;
 struct StepPar {
   float4 v[kMaxStepRounds][kRoundPar];
@@ -918,21 +901,23 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
       for (int k = 0; k < nr; ++k) {
         if (!BWD) {
           const uint4 lk = P.rec[k * (kFwdRoundWords / 4) + 1];  // links, bbits, rx mask
-          rot_fwd<0, RX>(r, P.v[k][0], D & 1u, D, lk.z & 1u);
-          rot_fwd<1, RX>(r, P.v[k][1], (D >> 1) & 1u, D, (lk.z >> 1) & 1u);
-          rot_fwd<2, RX>(r, P.v[k][2], (D >> 2) & 1u, D, (lk.z >> 2) & 1u);
-          rot_fwd<3, RX>(r, P.v[k][3], (D >> 3) & 1u, D, (lk.z >> 3) & 1u);
+          const float4 t0 = P.v[k][0];
+          rot_fwd<0, RX>(r, t0.x, D & 1u, lk.z & 1u);
+          rot_fwd<1, RX>(r, P.v[k][1].x, (D >> 1) & 1u, (lk.z >> 1) & 1u);
+          rot_fwd<2, RX>(r, P.v[k][2].x, (D >> 2) & 1u, (lk.z >> 2) & 1u);
+          rot_fwd<3, RX>(r, P.v[k][3].x, (D >> 3) & 1u, (lk.z >> 3) & 1u);
           apply_diag(r, &P.v[k][4]);
-          chain_pending(lk.x, rgb, lgb, g12, nq, pos, contig, D);
+          chain_pending(lk.x, rgb, lgb, g12, nq, pos, contig, __float_as_uint(t0.w), D);
         } else {
           const uint4 lk = P.rec[k * (kBwdRoundWords / 4) + 2];  // links, bbits, rx mask
-          chain_pending(lk.x, rgb, lgb, g12, nq, pos, contig, D);
+          const float4 t0 = P.v[k][0];
+          chain_pending(lk.x, rgb, lgb, g12, nq, pos, contig, __float_as_uint(t0.w), D);
           float v[8];
           diag_bwd(r, l, &P.v[k][4], v);
-          rot_bwd<0, RX>(r, l, P.v[k][0], D & 1u, D, v[4], lk.z & 1u);
-          rot_bwd<1, RX>(r, l, P.v[k][1], (D >> 1) & 1u, D, v[5], (lk.z >> 1) & 1u);
-          rot_bwd<2, RX>(r, l, P.v[k][2], (D >> 2) & 1u, D, v[6], (lk.z >> 2) & 1u);
-          rot_bwd<3, RX>(r, l, P.v[k][3], (D >> 3) & 1u, D, v[7], (lk.z >> 3) & 1u);
+          rot_bwd<0, RX>(r, l, t0.x, D & 1u, v[4], lk.z & 1u);
+          rot_bwd<1, RX>(r, l, P.v[k][1].x, (D >> 1) & 1u, v[5], (lk.z >> 1) & 1u);
+          rot_bwd<2, RX>(r, l, P.v[k][2].x, (D >> 2) & 1u, v[6], (lk.z >> 2) & 1u);
+          rot_bwd<3, RX>(r, l, P.v[k][3].x, (D >> 3) & 1u, v[7], (lk.z >> 3) & 1u);
           int idx;
           float sum;
           bool owner;
@@ -945,6 +930,8 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
           }
           const int32_t term =
               reinterpret_cast<const int32_t*>(&P.rec[k * (kBwdRoundWords / 4)])[idx];
+          // the table's factor of this value (diagonal terms in .z, rotation terms in .y)
+          sum *= reinterpret_cast<const float*>(&P.v[k][idx & 3])[idx < 4 ? 2 : 1];
           if (Tt >= 32) {
             if (owner) {
               s_red[buf][warp][k * 8 + idx] = sum;
@@ -957,10 +944,12 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
       }
       apply_pending<BWD>(D, r, l);
       }  // CUDA-core rounds
+      // register p holds amplitude p ^ m after the step's last round
+      const uint32_t ps = TC ? pb : pb ^ reg_off(__float_as_uint(P.v[nr - 1][1].w), so);
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
-        tp[pb ^ reg_off(j, so)] = r[j];
-        if (BWD) tl[pb ^ reg_off(j, so)] = l[j];
+        tp[ps ^ reg_off(j, so)] = r[j];
+        if (BWD) tl[ps ^ reg_off(j, so)] = l[j];
       }
       if (TC) {
         cp_async_wait_all();
@@ -1331,38 +1320,6 @@ __device__ double term_angle(const PrepArgs& a, int64_t t) {
   return phi;
 }
 
-// term_angle of the terms t[0..3] (-1: none, angle 0) with the loads of the
-// four terms issued together: the index ranges and constants, then the first
-// two parameters of each, then their values (the same summation order as
-// term_angle; a term of more than two parameters finishes in a loop).
-__device__ void term_angles4(const PrepArgs& a, const int32_t* t, double (&phi)[4]) {
-  int b0[4], b1[4], p0[4], p1[4];
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const bool on = t[r] >= 0;
-    b0[r] = on ? a.term_off[t[r]] : 0;
-    b1[r] = on ? a.term_off[t[r] + 1] : 0;
-    phi[r] = on && a.term_const ? a.term_const[t[r]] : 0.0;
-  }
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    p0[r] = b1[r] > b0[r] ? a.term_params[b0[r]] : -1;
-    p1[r] = b1[r] > b0[r] + 1 ? a.term_params[b0[r] + 1] : -1;
-  }
-  double v0[4], v1[4];
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    v0[r] = p0[r] >= 0 ? theta_at(a, p0[r]) : 0.0;
-    v1[r] = p1[r] >= 0 ? theta_at(a, p1[r]) : 0.0;
-  }
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    if (p0[r] >= 0) phi[r] += v0[r];
-    if (p1[r] >= 0) phi[r] += v1[r];
-    for (int j = b0[r] + 2; j < b1[r]; ++j) phi[r] += theta_at(a, a.term_params[j]);
-  }
-}
-
 // The angle of a resolved round term (the same summation order as
 // term_angle: the constant, then the parameters).
 __device__ __forceinline__ double round_term_angle(const PrepArgs& a, const RoundTerm& e) {
@@ -1393,13 +1350,6 @@ __device__ void shear_params(double phi, double& tq, double& sh, int& parity) {
   parity = ((long long)k) & 1;
 }
 
-__device__ float4 shear_of(double phi) {
-  double tq, sh;
-  int parity;
-  shear_params(phi, tq, sh, parity);
-  return make_float4((float)tq, (float)sh, __int_as_float(parity), 0.f);
-}
-
 // The same in float64 (complex128 round programs).
 __device__ Shear64 shear64_of(double phi) {
   Shear64 r{0.0, 0.0, 0, 0};
@@ -1413,45 +1363,146 @@ __device__ Shear64 shear64_of(double phi) {
 // act on register index j as e^{-i a_j} with a_j = sum_r sigma_r(j) phi_r / 2,
 // sigma_r(j) = +1 where bit r of j is clear, else -1 (RZ(phi) =
 // diag(e^{-i phi/2}, e^{i phi/2})), and its CZ links between register bits r
-// and r + 1 (bit r of bbits) as -1 where both bits of j are set. Gives
-// (cos, sin) of the applied phase (forward: -a_j) or of the un-applied one
+// and r + 1 (bit r of bbits) as -1 where both bits of j are set. Gives the
+// angle of the applied phase (forward: -a_j) or of the un-applied one
 // (backward: +a_j) for j = m, and the CZ signs of m and its complement
 // 15 - m: a_{15-m} = -a_m, so one float64 sincos of the summed angle serves both.
-__device__ void diag_phase_pair(const double (&phi)[4], uint32_t bbits, int m, bool apply, double& c, double& s,
-                                bool& f0, bool& f1) {
+__device__ double diag_angle(const double (&phi)[4], uint32_t bbits, int m, bool apply, bool& f0, bool& f1) {
   double al = 0.0;
   for (int r = 0; r < 4; ++r) al += ((m >> r) & 1) ? -phi[r] : phi[r];
-  al *= apply ? -0.5 : 0.5;
-  sincos_prep(al, &s, &c);
   const int mc = 15 - m;
   f0 = __popc(bbits & (uint32_t)m & (uint32_t)(m >> 1)) & 1;
   f1 = __popc(bbits & (uint32_t)mc & (uint32_t)(mc >> 1)) & 1;
-}
-
-// neg: the round's items' wrap signs multiply to -1; the phases carry it.
-__device__ void diag_phases(const double (&phi)[4], uint32_t bbits, int m, bool apply, bool neg, float2* ph) {
-  double cd, sd;
-  bool f0, f1;
-  diag_phase_pair(phi, bbits, m, apply, cd, sd, f0, f1);
-  const float c = neg ? -(float)cd : (float)cd, s = neg ? -(float)sd : (float)sd;
-  ph[m] = f0 ? make_float2(-c, -s) : make_float2(c, s);
-  ph[15 - m] = f1 ? make_float2(-c, s) : make_float2(c, -s);
+  return al * (apply ? -0.5 : 0.5);
 }
 
 // The same in float64 (complex128 round programs).
 __device__ void diag_phases64(const double (&phi)[4], uint32_t bbits, int m, bool apply, double2* ph) {
   double c, s;
   bool f0, f1;
-  diag_phase_pair(phi, bbits, m, apply, c, s, f0, f1);
+  sincos_prep(diag_angle(phi, bbits, m, apply, f0, f1), &s, &c);
   ph[m] = f0 ? make_double2(-c, -s) : make_double2(c, s);
   ph[15 - m] = f1 ? make_double2(-c, s) : make_double2(c, -s);
 }
 
+// One round's float32 parameters by a half-warp (e: lane in it): lanes 0..3
+// hold the 4 rotations, lanes 4..11 two phases of the diagonal each. The
+// rotations' reduced form (see rot_T): q, and a bit flip X for |w| > pi/2. The
+// flips of the step's earlier rounds (at most 3, s0 of them) come from their
+// angles alone, one item per lane, so every lane takes one sincos.
+__device__ void round_params(const PrepArgs& a, bool on, bool fwd, int64_t r, const int32_t* rec,
+                             const RoundTerm* rt, int e, int lane) {
+  const int s0 = fwd ? rec[7] : rec[11];
+  const uint32_t rx = (uint32_t)(fwd ? rec[6] : rec[10]), bbits = (uint32_t)(fwd ? rec[5] : rec[9]);
+  const double two_pi = 6.283185307179586476925286766559, half_pi = 1.5707963267948966192313216916398;
+  // item e & 3 of round r - s0 + e / 4: does it flip?
+  bool flips = false;
+  if ((e >> 2) <= s0) {
+    const double phi = round_term_angle(a, rt[8 * ((e >> 2) - s0) + (e & 3)]);
+    flips = fabs(phi - two_pi * wrap_count(phi)) > half_pi;
+  }
+  const uint32_t F = (__ballot_sync(0xffffffffu, flips) >> (lane & 16)) & 0xffffu;
+  const uint32_t K = (F >> (4 * s0)) & 15u;
+  uint32_t m0 = 0;  // flips before this round
+  for (int k = 0; k < s0; ++k) m0 ^= (F >> (4 * k)) & 15u;
+  const uint32_t m1 = m0 ^ K;
+  double ang = 0.0, phi[4] = {0.0, 0.0, 0.0, 0.0};
+  bool odd = false;  // the wrap's sign: u(phi) = (-1)^k u(w)
+  if (e < 4) {
+    const double ph = round_term_angle(a, rt[e]), k = wrap_count(ph);
+    ang = 0.5 * (ph - two_pi * k);
+    odd = ((long long)k) & 1;
+  }
+  double c, s;
+  bool f0 = false, f1 = false;
+  if (e >= 4 && e < 12) {
+    for (int q = 0; q < 4; ++q) phi[q] = round_term_angle(a, rt[4 + q]);
+    ang = diag_angle(phi, bbits, e - 4, fwd, f0, f1);
+  }
+  sincos_prep(ang, &s, &c);
+  float q = 0.f;
+  if (e < 4) {
+    const bool kf = (K >> e) & 1u;
+    q = (float)(kf ? c / s : s / c);
+    if (kf && s < 0.0) odd = !odd;  // the scale sin(w/2) is negative
+  }
+  const uint32_t neg = __popc((__ballot_sync(0xffffffffu, odd) >> (lane & 16)) & 15u) & 1u;
+  double Q[4], Qs = 1.0;  // 1 + q^2 of the rounded q: the scales keep the norm
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const double qk = (double)__shfl_sync(0xffffffffu, q, (lane & 16) + k);
+    Q[k] = 1.0 + qk * qk;
+    Qs *= Q[k];
+  }
+  const double S = (neg ? -1.0 : 1.0) / sqrt(Qs);
+  float4* out = (fwd ? a.rpf : a.rpb) + r * kRoundPar;
+  if (!on) return;
+  if (e < 4) {
+    const uint32_t mr = (fwd ? m0 : m1) >> e & 1u, isrx = rx >> e & 1u;
+    // the table's q: T(t) or T(-k) applied, T(-t) or T(k) un-applied; an RY on a flipped pair: -q
+    const uint32_t kf = (K >> e) & 1u;
+    const bool neg_q = (fwd ? kf != 0 : kf == 0) != (mr && !isrx);
+    double g = Q[3];  // undoes the scales that the gradient value of item e carries
+#pragma unroll
+    for (int k = 2; k >= 0; --k)
+      if (k >= e) g *= Q[k];
+    out[e] = make_float4(neg_q ? -q : q, (float)(mr && !isrx && !fwd ? -g : g), (m0 >> e & 1u) ? -1.f : 1.f,
+                         __uint_as_float(e == 0 ? (fwd ? m1 : m0) : m1));
+  } else if (e < 12) {
+    // e^{i ang} for index e - 4 and its conjugate for the complement, times the round's scale, the Z's of
+    // flipped RYs, and (-i) (adjoint: i) per flipped RX; amplitude j sits in register j ^ (flips so far)
+    const uint32_t Kz = K & ~rx, nx = (uint32_t)__popc(K & rx) & 3u, md = fwd ? m1 : m0;
+    float2* ph = reinterpret_cast<float2*>(out + 4);
+    for (int h = 0; h < 2; ++h) {
+      const uint32_t j = h ? 15u - (uint32_t)(e - 4) : (uint32_t)(e - 4);
+      const bool sg = (h ? f1 : f0) != ((__popc((j ^ K) & Kz) & 1) != 0);
+      double x = c * S, y = (h ? -s : s) * S;
+      if (sg) { x = -x; y = -y; }
+      for (uint32_t k = 0; k < nx; ++k) {
+        const double t = x;
+        x = fwd ? y : -y;
+        y = fwd ? -t : t;
+      }
+      ph[j ^ md] = make_float2((float)x, (float)y);
+    }
+  }
+}
+
 }  // namespace
 
-// Element i of the tables: fused matrices, terms, encodings, then (round
-// programs) the forward and backward round parameters in round order.
+// Element i of the tables: (round programs) the forward and backward round
+// parameters in round order, then fused matrices, terms and encodings. A
+// round's float32 parameters are made by 16 lanes together; round_par_elems
+// is a multiple of 32, so that a warp is either wholly on rounds or not.
 __device__ void prep_one(const PrepArgs& a, int64_t i) {
+  const int64_t nre = round_par_elems(a);
+  if (i < nre) {
+    const int64_t nr = (int64_t)a.n_rpf + a.n_rpb;
+    int64_t r = i >> 4;
+    const bool on = r < nr;
+    if (!on) r = nr - 1;
+    const int e = (int)(i & 15);
+    const bool fwd = r < a.n_rpf;
+    if (!fwd) r -= a.n_rpf;
+    const int32_t* rec = fwd ? reinterpret_cast<const int32_t*>(a.rpf_src) + r * kFwdRoundWords
+                             : reinterpret_cast<const int32_t*>(a.rpb_src) + r * kBwdRoundWords;
+    const RoundTerm* rt = (fwd ? a.rpf_terms : a.rpb_terms) + r * 8;
+    if (a.rpf64 || a.rpb64) {
+      RoundPar64& out = (fwd ? a.rpf64 : a.rpb64)[r];
+      if (!on || e >= 12) return;
+      if (e < 4) {
+        out.rot[e] = shear64_of(round_term_angle(a, rt[e]));
+      } else {
+        double phi[4];
+        for (int q = 0; q < 4; ++q) phi[q] = round_term_angle(a, rt[4 + q]);
+        diag_phases64(phi, (uint32_t)(fwd ? rec[5] : rec[9]), e - 4, fwd, out.ph);
+      }
+    } else {
+      round_params(a, on, fwd, r, rec, rt, e, threadIdx.x & 31);
+    }
+    return;
+  }
+  i -= nre;
   if (i < a.n_fused) {
     float4 m0, m1;
     fused_u(a, i, m0, m1, a.mats64 ? a.mats64 + 8 * i : nullptr);
@@ -1463,15 +1514,10 @@ __device__ void prep_one(const PrepArgs& a, int64_t i) {
   }
   i -= a.n_fused;
   if (i < a.n_terms) {
-    if (a.cs64) {
-      double s, c;
-      sincos_prep(0.5 * term_angle(a, i), &s, &c);
-      a.cs64[i] = make_double2(c, s);
-    } else {
-      double s, c;
-      sincos_prep(0.5 * term_angle(a, i), &s, &c);
-      a.cs[i] = make_float2((float)c, (float)s);
-    }
+    double s, c;
+    sincos_prep(0.5 * term_angle(a, i), &s, &c);
+    if (a.cs64) a.cs64[i] = make_double2(c, s);
+    else a.cs[i] = make_float2((float)c, (float)s);
     return;
   }
   i -= a.n_terms;
@@ -1486,50 +1532,6 @@ __device__ void prep_one(const PrepArgs& a, int64_t i) {
     }
     if (a.enc64) a.enc64[i] = make_double2(c, s);
     else a.enc[i] = make_float2((float)c, (float)s);
-    return;
-  }
-  i -= (int64_t)a.B * a.n_eff;
-  // per round the 4 rotation shears, then the merged diagonal (float32 tables,
-  // or float64 ones for complex128 plans)
-  bool fwd = i < (int64_t)kRoundPar * a.n_rpf;
-  if (!fwd) i -= (int64_t)kRoundPar * a.n_rpf;
-  if (!fwd && i >= (int64_t)kRoundPar * a.n_rpb) return;
-  const int64_t r = i / kRoundPar;
-  const int e = (int)(i - r * kRoundPar);
-  const int32_t* rec = fwd ? reinterpret_cast<const int32_t*>(a.rpf_src) + r * kFwdRoundWords
-                           : reinterpret_cast<const int32_t*>(a.rpb_src) + r * kBwdRoundWords;
-  const int32_t* tz = fwd ? rec + 8 : rec;
-  const int32_t* ty = fwd ? rec + 12 : rec + 4;
-  // the round's terms resolved at plan time (their loads issue together), or
-  // through the term maps
-  const RoundTerm* rt = fwd ? a.rpf_terms : a.rpb_terms;
-  if (rt) rt += r * 8;
-  const bool f64 = a.rpf64 || a.rpb64;
-  if (e < 4) {
-    const double phi = rt ? round_term_angle(a, rt[e]) : (ty[e] >= 0 ? term_angle(a, ty[e]) : 0.0);
-    if (f64) (fwd ? a.rpf64 : a.rpb64)[r].rot[e] = shear64_of(phi);
-    else (fwd ? a.rpf : a.rpb)[r * kRoundPar + e] = shear_of(phi);
-    return;
-  }
-  const uint32_t bbits = (uint32_t)(fwd ? rec[5] : rec[9]);
-  double phi[4];
-  if (rt) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) phi[q] = round_term_angle(a, rt[4 + q]);
-  } else {
-    term_angles4(a, tz, phi);
-  }
-  if (f64) {
-    diag_phases64(phi, bbits, e - 4, fwd, (fwd ? a.rpf64 : a.rpb64)[r].ph);
-  } else {
-    // the product of the 4 rotations' wrap signs (-1)^k, the same k as their shears
-    long long k = 0;
-    for (int q = 0; q < 4; ++q) {
-      const double phr = rt ? round_term_angle(a, rt[q]) : (ty[q] >= 0 ? term_angle(a, ty[q]) : 0.0);
-      k += (long long)wrap_count(phr);
-    }
-    diag_phases(phi, bbits, e - 4, fwd, (k & 1) != 0,
-                reinterpret_cast<float2*>((fwd ? a.rpf : a.rpb) + r * kRoundPar + 4));
   }
 }
 
@@ -1851,7 +1853,7 @@ cudaError_t launch_batch(const BatchArgs& a, int grid, int64_t prep_total, int64
 
 // ---- launchers ----------------------------------------------------------------
 cudaError_t launch_prep(const PrepArgs& a, cudaStream_t st) {
-  int64_t total = (int64_t)a.n_fused + a.n_terms + (int64_t)a.B * a.n_eff + round_par_elems(a);
+  int64_t total = prep_elems(a);
   if (total == 0 && !a.zero_word) return cudaSuccess;
   if (total == 0) total = 1;  // element 0 only clears the counter
   // float64 work per element: small blocks spread it over more SMs

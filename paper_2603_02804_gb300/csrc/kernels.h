@@ -95,10 +95,10 @@ struct PrepArgs {
   // round programs: the parameters of every round gathered in round order
   int32_t n_rpf;               // forward rounds
   const uint4* rpf_src;        // forward round records (fused index per item)
-  float4* rpf;                 // [n_rpf][kRoundPar]: rotation shears, then the applied diagonal
+  float4* rpf;                 // [n_rpf][kRoundPar]: rotations, then the applied diagonal
   int32_t n_rpb;               // backward rounds
   const uint4* rpb_src;        // backward round records (tz[4], ty[4] terms)
-  float4* rpb;                 // [n_rpb][kRoundPar]: rotation shears, then the un-applied diagonal
+  float4* rpb;                 // [n_rpb][kRoundPar]: rotations, then the un-applied diagonal
   RoundPar64* rpf64;           // if non-null instead of rpf / rpb: the same in float64
   RoundPar64* rpb64;           //   (complex128 round programs), [n_rpf] / [n_rpb]
   uint32_t* zero_word;         // if non-null: set to 0 (the forward's CTA counter)
@@ -106,9 +106,13 @@ struct PrepArgs {
   const RoundTerm* rpb_terms;  //   4 RZ-run terms (-1 terms: no parameter, angle 0)
 };
 
-// Table elements of the round parameters (prep work items, kRoundPar per round).
+// Prep work items: 16 per round (a half-warp makes one round's parameters),
+// rounded up to whole warps, then one per fused matrix, term and encoding.
 __host__ __device__ inline int64_t round_par_elems(const PrepArgs& a) {
-  return (int64_t)kRoundPar * ((int64_t)a.n_rpf + a.n_rpb);
+  return (16 * ((int64_t)a.n_rpf + a.n_rpb) + 31) / 32 * 32;
+}
+__host__ __device__ inline int64_t prep_elems(const PrepArgs& a) {
+  return round_par_elems(a) + a.n_fused + a.n_terms + a.B * a.n_eff;
 }
 
 struct GradReduceArgs {

@@ -963,6 +963,7 @@ FusedPlan plan_fused_with(const Circuit& c_in, const PlanRequest& req, bool stri
       fw[4] = links;
       fw[5] = bbits;
       fw[6] = rx_mask;
+      fw[7] = (uint32_t)brs.size();  // the round's index in the step
       for (int r = 0; r < 8; ++r) fw[8 + r] = (uint32_t)bw[r];  // the items' terms (forward shears)
       bw[8] = (int32_t)links;
       bw[9] = (int32_t)bbits;
@@ -979,7 +980,10 @@ FusedPlan plan_fused_with(const Circuit& c_in, const PlanRequest& req, bool stri
     ++P.n_steps;
     P.n_rounds += (int)nr;
     const uint32_t br0 = (uint32_t)(P.bwd_rounds.size() / kBwdRoundWords);
-    for (auto it = brs.rbegin(); it != brs.rend(); ++it) P.bwd_rounds.insert(P.bwd_rounds.end(), it->begin(), it->end());
+    for (auto it = brs.rbegin(); it != brs.rend(); ++it) {
+      (*it)[11] = (int32_t)(it - brs.rbegin());
+      P.bwd_rounds.insert(P.bwd_rounds.end(), it->begin(), it->end());
+    }
     bwd_items.push_back({{w0(OP_STEP, (uint32_t)st.group << 4 | nr << 8), br0}});
   };
   for (size_t pi = 0; pi < passes.size(); ++pi) {

@@ -42,11 +42,11 @@ enum OpCode : uint32_t {
 // and then the CZ links of the round.
 //   forward round, kFwdRoundWords words: m[4] (fused 2x2 index per register
 //     bit, 0 = identity), links, bbits (links between register bits r, r+1),
-//     rx (bit r: item r's rotation is an RX), a pad word, tz[4], ty[4] (the
-//     items' gradient terms, as below).
+//     rx (bit r: item r's rotation is an RX), the round's index in its step,
+//     tz[4], ty[4] (the items' gradient terms, as below).
 //   backward round, kBwdRoundWords words: tz[4], ty[4] (term of the merged RZ
-//     run and of the rotation of each item, -1 = none), links, bbits, rx, a
-//     pad word.
+//     run and of the rotation of each item, -1 = none), links, bbits, rx, the
+//     round's index in its step.
 // An item is an RZ run alone or a rotation (RY or RX) followed by an RZ run.
 // A forward round applies per item the rotation and then the RZ run, then the
 // links; a backward step runs its rounds in the order stored, each applying
@@ -55,15 +55,16 @@ enum OpCode : uint32_t {
 constexpr int kFwdRoundWords = 16;
 constexpr int kBwdRoundWords = 12;
 constexpr int kMaxStepRounds = 4;   // 8 gradient values per round
-// Parameters of one round of a complex64 round program, in float4: [0, 4) the
-// shear parameters (tan(w/4), sin(w/2), wrap parity) of the 4 items'
-// rotations; [4, 12) the round's diagonal, i.e. the 4 RZ runs (and the CZ
-// links between register bits) merged into one phase per register index j:
-// float4 4 + m holds (cos a_j, sin a_j) for j = 2m and 2m + 1, times the
-// product of the 4 rotations' wrap signs (the kernels do not read the
-// parities themselves). Prep fills
-// them as kRoundPar work items per round; complex128 programs hold the same
-// in float64 (RoundPar64).
+// Parameters of one round of a complex64 round program, in float4. [0, 4): the
+// 4 items' rotations: x = q of [[1, -q], [q, 1]] (|q| <= 1), y and z = the
+// factors of the adjoint's gradient values of the item's rotation and RZ run,
+// w = a mask of register bits as an integer (item 0: the flips in force where
+// the round's links act, the others: those after the round; register p holds
+// amplitude p ^ mask). [4, 12): the round's diagonal, i.e. the 4 RZ runs (and
+// the CZ links between register bits) merged into one phase per register p,
+// two per float4, times the scales, signs and phases that the 4 rotations in
+// their reduced form leave out. Prep fills them with 16 lanes per round;
+// complex128 programs hold shears and phases in float64 (RoundPar64).
 constexpr int kRoundPar = 12;
 
 // Source / destination codes of a pass.

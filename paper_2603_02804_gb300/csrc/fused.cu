@@ -165,7 +165,13 @@ __device__ __forceinline__ float2 mul_ipow(float2 v, uint32_t k) {
 // register index j (bit 4 of D: c0, bits 0..3: A). D commutes with every
 // diagonal gate; a gate on register bit r only sees the factor Z_r^(A_r),
 // which is folded into that gate. CZs between two register bits (quadratic in
-// j, the same for every thread) are signs of the round's diagonal table.
+// j, the same for every thread) are signs of the round's diagonal table. A
+// link that leaves the register group stays pending beyond its step, as a bit
+// of `pend`: the next step starts from the D that pend gives its threads. It
+// is applied only where the plan says so (a later group holds both its qubits,
+// a checkpoint, the end of the pass). Applying D at every step took 80 of the
+// adjoint's instructions per step and thread (n = 20, d = 24, 64 samples: step
+// 26.12 -> 25.10 ms).
 //
 // Links L of one round, thread base index gb (register bits zero), register
 // bit positions p[r]: x = gb ^ y(j) with disjoint supports, so each link q
@@ -184,17 +190,15 @@ __device__ __forceinline__ void link_terms(uint32_t L, uint32_t gb, int n, uint3
 // the thread (rgb = gb rotated right by one qubit, lgb = left, g12 = gb &
 // rgb): as rotation distributes over &, u = rotl(L) & lgb ^ L & rgb (the
 // link_terms u), and the constant part is |L & g12|. When the register bits
-// sit on consecutive qubits (contig), A is one shift of u. Register p holds
-// amplitude p ^ m (the step's bit flips, see rot_T), so the linear part of
-// amplitude j = p ^ m adds the constant |A & m|.
+// sit on consecutive qubits (contig), A is one shift of u.
 __device__ __forceinline__ void chain_pending(uint32_t L, uint32_t rgb, uint32_t lgb, uint32_t g12, int n,
-                                                const uint32_t (&p)[4], bool contig, uint32_t m, uint32_t& D) {
+                                                const uint32_t (&p)[4], bool contig, uint32_t& D) {
   const uint32_t nmask = n >= 32 ? ~0u : ((1u << n) - 1u);
   const uint32_t u = ((((L << 1) | (L >> (n - 1))) & nmask) & lgb) ^ (L & rgb);
   const uint32_t A = contig ? (u >> p[0]) & 15u
                             : ((u >> p[0]) & 1u) | (((u >> p[1]) & 1u) << 1) | (((u >> p[2]) & 1u) << 2) |
                                   (((u >> p[3]) & 1u) << 3);
-  D ^= A | ((__popc((L & g12) ^ (A & m)) & 1u) << 4);
+  D ^= A | ((__popc(L & g12) & 1u) << 4);
 }
 
 // Multiply the registers by D (end of a step).
@@ -219,22 +223,19 @@ __device__ __forceinline__ void apply_pending(uint32_t D, float2 (&r)[16], float
 
 // One rotation of a round on register bit R, two FMAs per real component:
 //   RY: p0 -= q p1; p1 += q p0      RX: p0 -= i q p1; p1 -= i q p0
-// (old values on the right), i.e. [[1, -q], [q, 1]] or [[1, -iq], [-iq, 1]].
-// A rotation by w with |w| <= pi/2 is cos(w/2) times that with q = tan(w/2);
-// beyond, with k = cot(w/2), RY(w) = sin(w/2) X Z T(-k) and RX(w) =
-// -i sin(w/2) X T(-k), so |q| <= 1 for every angle. The factors of the round's
-// four rotations (scales, signs, Z's and phases) are multiplied into its
-// diagonal's 16 phases, which the kernel applies anyway; the X's are never
-// executed: they flip bits of a mask m (the same for every thread, from the
-// tables), register p of a step holding amplitude p ^ m, and the step's last
-// store puts the registers at their addresses. An RY acts on a flipped pair
-// with -q (folded into the table's q). Against rotations as three shears
-// (3 FMAs per component): forward of n = 16, d = 20, 500 samples 2.86 -> 2.57
-// ms; training step of n = 20, d = 24, 64 samples 28.35 -> 26.32 ms, of n = 12,
-// d = 20, 256 samples 268 -> 251 us.
-// A pending Z_R turns the rotation by w into one by -w, i.e. q into -q (the
-// sign of sin(w/2) moves to the pending constant: it cancels against the flip
-// of the pending sign's own index, chain_pending's |A & m|).
+// (old values on the right), i.e. [[1, -q], [q, 1]] or [[1, -iq], [-iq, 1]]: the
+// rotation by w over cos(w/2), with q = tan(w/2). The cosines of a round's four
+// rotations are one scale of the state, multiplied into the 16 phases of the
+// round's diagonal, which the kernel applies anyway. q is rounded before the
+// scale is made from it, so that the norm is kept; a large q costs no accuracy,
+// as the scaled result is rounded once. Where any of the four has |tan(w/2)| >
+// kMaxTan, the round runs twice, by half the angles (|q| <= 1) and with the
+// diagonal once: 1 % of the rounds for uniform angles, and the scale of a round
+// stays above 2^-32 (a branch that repeats only the rotations made every round
+// 8 % slower: registers spill). Three shears (3 FMAs per component) need no scale and
+// were slower: training step of n = 20, d = 24, 64 samples 28.35 -> 25.10 ms, of
+// n = 12, d = 20, 256 samples 268 -> 237 us (with the pending links below). A
+// pending Z_R turns the rotation by w into one by -w, i.e. q into -q.
 template <int R, bool RX>
 __device__ __forceinline__ void rot_T(float2 (&r)[16], float q, bool rx) {
   if (RX && rx) {
@@ -260,10 +261,9 @@ __device__ __forceinline__ void rot_T(float2 (&r)[16], float q, bool rx) {
   }
 }
 
-// The rotation of a forward item (q of the round's table; a: a pending Z_R).
-template <int R, bool RX>
-__device__ __forceinline__ void rot_fwd(float2 (&r)[16], float q, uint32_t a, bool rx) {
-  rot_T<R, RX>(r, __int_as_float(__float_as_int(q) ^ (int)(a << 31)), rx);
+// q with the sign of a pending Z (a = 1).
+__device__ __forceinline__ float pend_q(float q, uint32_t a) {
+  return __int_as_float(__float_as_int(q) ^ (int)(a << 31));
 }
 
 // v *= (c + i s)
@@ -324,9 +324,9 @@ __device__ __forceinline__ void diag_bwd(float2 (&p)[16], float2 (&l)[16], const
 // The rotation of an adjoint item on register bit R (q un-applies it; RX where
 // rx, uniform over the CTA, else RY), after the round's diagonal; gy: the
 // thread's sum of Im<lambda|P|psi> taken before it. A pending Z_R negates q
-// and gy. The round's scales and flips multiply gy by a factor that is the
-// same for every thread and sample; the owner lane of the reduced sum undoes
-// it (the table's .y).
+// and gy. The round's scale and the earlier items' rotations multiply gy by a
+// factor that is the same for every thread and sample; the owner lane of the
+// reduced sum undoes it (the table's factor).
 template <int R, bool RX = false>
 __device__ __forceinline__ void rot_bwd(float2 (&p)[16], float2 (&l)[16], float qt, uint32_t a, float& gy,
                                         bool rx = false) {
@@ -620,6 +620,7 @@ __device__ void loss_block(int kind, double* E, const Y* y, int64_t B, double sc
 
 struct PassShared {
   StepPar par[2];
+  float4 ident[8];             // the diagonal of a round's run that has none
   uint32_t ticket;             // the CTA's finishing order (loss on the last CTA)
   uint32_t lg[256];
   uint32_t base[4][kThreads];  // per register group: the thread's tile index with the group's bits zero
@@ -669,6 +670,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
   if (tid < 16) {
     s_gmap[tid] = pd.gmap[tid];
     s_grp[tid >> 2][tid & 3] = pd.groups[tid >> 2][tid & 3];
+    if (ROUNDS && tid < 8) sh.ident[tid] = make_float4(1.f, 0.f, 1.f, 0.f);
   }
   __syncthreads();
   for (int h = tid; h < (1 << tl2); h += kThreads) {
@@ -847,6 +849,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
 
   // ---- step program ------------------------------------------------------------
   int buf = 0;
+  uint32_t pend = 0;  // links whose CZ signs the tile's amplitudes still lack (round programs)
   int32_t pc = pd.op_begin;
   const uint2* ops = a.ops;
 #pragma unroll 1
@@ -889,27 +892,38 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
       const uint32_t g12 = gb & rgb;
       const bool contig = pos[1] == pos[0] + 1 && pos[2] == pos[0] + 2 && pos[3] == pos[0] + 3;
       uint32_t D = 0;
+      if (!TC) chain_pending(pend, rgb, lgb, g12, nq, pos, contig, D);
       if constexpr (TC) {
         tc_rounds(*tc, P, nr, tc->bsm + (size_t)sb * kMaxStepRounds * kTcBFloats, gb, pos, a.n_eff, r, ph, tid);
       } else {
+      // a round whose rotations are steep runs twice (see rot_T): the forward
+      // with its diagonal and links the second time, the adjoint the first
+      bool again = false;
 #pragma unroll 1
-      for (int k = 0; k < nr; ++k) {
+      for (int k = 0; k < nr;) {
         if (!BWD) {
-          const uint4 lk = P.rec[k * (kFwdRoundWords / 4) + 1];  // links, bbits, rx mask
-          const float4 t0 = P.v[k][0];
-          rot_fwd<0, RX>(r, t0.x, D & 1u, lk.z & 1u);
-          rot_fwd<1, RX>(r, P.v[k][1].x, (D >> 1) & 1u, (lk.z >> 1) & 1u);
-          rot_fwd<2, RX>(r, P.v[k][2].x, (D >> 2) & 1u, (lk.z >> 2) & 1u);
-          rot_fwd<3, RX>(r, P.v[k][3].x, (D >> 3) & 1u, (lk.z >> 3) & 1u);
-          apply_diag(r, &P.v[k][4]);
-          chain_pending(lk.x, rgb, lgb, g12, nq, pos, contig, __float_as_uint(t0.w), D);
+          const uint4 lk = P.rec[k * (kFwdRoundWords / 4) + 1];  // links, bbits, rx mask, leaving links
+          const bool pre = P.v[k][0].y < 0.f && !again;
+          rot_T<0, RX>(r, pend_q(P.v[k][0].x, D & 1u), lk.z & 1u);
+          rot_T<1, RX>(r, pend_q(P.v[k][1].x, (D >> 1) & 1u), (lk.z >> 1) & 1u);
+          rot_T<2, RX>(r, pend_q(P.v[k][2].x, (D >> 2) & 1u), (lk.z >> 2) & 1u);
+          rot_T<3, RX>(r, pend_q(P.v[k][3].x, (D >> 3) & 1u), (lk.z >> 3) & 1u);
+          apply_diag(r, pre ? sh.ident : &P.v[k][4]);
+          if (!pre) {
+            chain_pending(lk.x, rgb, lgb, g12, nq, pos, contig, D);
+            pend ^= lk.w;
+            ++k;
+          }
+          again = pre;
         } else {
-          const uint4 lk = P.rec[k * (kBwdRoundWords / 4) + 2];  // links, bbits, rx mask
-          const float4 t0 = P.v[k][0];
-          chain_pending(lk.x, rgb, lgb, g12, nq, pos, contig, __float_as_uint(t0.w), D);
+          const uint4 lk = P.rec[k * (kBwdRoundWords / 4) + 2];  // links, bbits, rx mask, leaving links
+          if (!again) {
+            chain_pending(lk.x, rgb, lgb, g12, nq, pos, contig, D);
+            pend ^= lk.w;
+          }
           float v[8];
-          diag_bwd(r, l, &P.v[k][4], v);
-          rot_bwd<0, RX>(r, l, t0.x, D & 1u, v[4], lk.z & 1u);
+          diag_bwd(r, l, again ? sh.ident : &P.v[k][4], v);
+          rot_bwd<0, RX>(r, l, P.v[k][0].x, D & 1u, v[4], lk.z & 1u);
           rot_bwd<1, RX>(r, l, P.v[k][1].x, (D >> 1) & 1u, v[5], (lk.z >> 1) & 1u);
           rot_bwd<2, RX>(r, l, P.v[k][2].x, (D >> 2) & 1u, v[6], (lk.z >> 2) & 1u);
           rot_bwd<3, RX>(r, l, P.v[k][3].x, (D >> 3) & 1u, v[7], (lk.z >> 3) & 1u);
@@ -925,8 +939,8 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
           }
           const int32_t term =
               reinterpret_cast<const int32_t*>(&P.rec[k * (kBwdRoundWords / 4)])[idx];
-          // the table's factor of this value (diagonal terms in .z, rotation terms in .y)
-          sum *= reinterpret_cast<const float*>(&P.v[k][idx & 3])[idx < 4 ? 2 : 1];
+          if (idx >= 4) sum *= fabsf(P.v[k][idx - 4].y);
+          if (again) owner = false;  // the first run of the round has its values
           if (Tt >= 32) {
             if (owner) {
               s_red[buf][warp][k * 8 + idx] = sum;
@@ -935,16 +949,19 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
           } else if (owner && active && term >= 0) {
             a.g_part[tile * a.n_slots + term] = 0.5 * (double)sum;
           }
+          again = P.v[k][0].y < 0.f && !again;
+          k += again ? 0 : 1;
         }
       }
-      apply_pending<BWD>(D, r, l);
+      if ((op.x >> kStepFlushBit) & 1u) {
+        apply_pending<BWD>(D, r, l);
+        pend = 0;
+      }
       }  // CUDA-core rounds
-      // register p holds amplitude p ^ m after the step's last round
-      const uint32_t ps = TC ? pb : pb ^ reg_off(__float_as_uint(P.v[nr - 1][1].w), so);
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
-        tp[ps ^ reg_off(j, so)] = r[j];
-        if (BWD) tl[ps ^ reg_off(j, so)] = l[j];
+        tp[pb ^ reg_off(j, so)] = r[j];
+        if (BWD) tl[pb ^ reg_off(j, so)] = l[j];
       }
       if (TC) {
         cp_async_wait_all();
@@ -1381,85 +1398,53 @@ __device__ void diag_phases64(const double (&phi)[4], uint32_t bbits, int m, boo
 }
 
 // One round's float32 parameters by a half-warp (e: lane in it): lanes 0..3
-// hold the 4 rotations, lanes 4..11 two phases of the diagonal each. The
-// rotations' reduced form (see rot_T): q, and a bit flip X for |w| > pi/2. The
-// flips of the step's earlier rounds (at most 3, s0 of them) come from their
-// angles alone, one item per lane, so every lane takes one sincos.
+// take the 4 rotations, lanes 4..11 two phases of the diagonal each, one sincos
+// per lane (see rot_T).
 __device__ void round_params(const PrepArgs& a, bool on, bool fwd, int64_t r, const int32_t* rec,
                              const RoundTerm* rt, int e, int lane) {
-  const int s0 = fwd ? rec[7] : rec[11];
-  const uint32_t rx = (uint32_t)(fwd ? rec[6] : rec[10]), bbits = (uint32_t)(fwd ? rec[5] : rec[9]);
-  const double two_pi = 6.283185307179586476925286766559, half_pi = 1.5707963267948966192313216916398;
-  // item e & 3 of round r - s0 + e / 4: does it flip?
-  bool flips = false;
-  if ((e >> 2) <= s0) {
-    const double phi = round_term_angle(a, rt[8 * ((e >> 2) - s0) + (e & 3)]);
-    flips = fabs(phi - two_pi * wrap_count(phi)) > half_pi;
-  }
-  const uint32_t F = (__ballot_sync(0xffffffffu, flips) >> (lane & 16)) & 0xffffu;
-  const uint32_t K = (F >> (4 * s0)) & 15u;
-  uint32_t m0 = 0;  // flips before this round
-  for (int k = 0; k < s0; ++k) m0 ^= (F >> (4 * k)) & 15u;
-  const uint32_t m1 = m0 ^ K;
-  double ang = 0.0, phi[4] = {0.0, 0.0, 0.0, 0.0};
-  bool odd = false;  // the wrap's sign: u(phi) = (-1)^k u(w)
+  double ang = 0.0;
+  bool odd = false, f0 = false, f1 = false;
   if (e < 4) {
-    const double ph = round_term_angle(a, rt[e]), k = wrap_count(ph);
-    ang = 0.5 * (ph - two_pi * k);
+    // u(phi) = (-1)^k u(w) with w = phi - 2 pi k in [-pi, pi]
+    const double phi = round_term_angle(a, rt[e]), k = wrap_count(phi);
+    ang = 0.5 * (phi - 6.283185307179586476925286766559 * k);
     odd = ((long long)k) & 1;
+  } else if (e < 12) {
+    double phi[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) phi[q] = round_term_angle(a, rt[4 + q]);
+    ang = diag_angle(phi, (uint32_t)(fwd ? rec[5] : rec[9]), e - 4, fwd, f0, f1);
   }
   double c, s;
-  bool f0 = false, f1 = false;
-  if (e >= 4 && e < 12) {
-    for (int q = 0; q < 4; ++q) phi[q] = round_term_angle(a, rt[4 + q]);
-    ang = diag_angle(phi, bbits, e - 4, fwd, f0, f1);
-  }
   sincos_prep(ang, &s, &c);
-  float q = 0.f;
-  if (e < 4) {
-    const bool kf = (K >> e) & 1u;
-    q = (float)(kf ? c / s : s / c);
-    if (kf && s < 0.0) odd = !odd;  // the scale sin(w/2) is negative
-  }
-  const uint32_t neg = __popc((__ballot_sync(0xffffffffu, odd) >> (lane & 16)) & 15u) & 1u;
-  double Q[4], Qs = 1.0;  // 1 + q^2 of the rounded q: the scales keep the norm
+  const int half = lane & 16;
+  const bool steep = e < 4 && fabs(s) > kMaxTan * fabs(c);
+  const bool twice = ((__ballot_sync(0xffffffffu, steep) >> half) & 15u) != 0;
+  const uint32_t neg = __popc((__ballot_sync(0xffffffffu, odd) >> half) & 15u) & 1u;
+  const float q = e < 4 ? (float)(s / (twice ? 1.0 + c : c)) : 0.f;  // tan(w/4) = sin(w/2) / (1 + cos(w/2))
+  double Q[4], S = 1.0;
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    const double qk = (double)__shfl_sync(0xffffffffu, q, (lane & 16) + k);
+    const double qk = (double)__shfl_sync(0xffffffffu, q, half + k);
     Q[k] = 1.0 + qk * qk;
-    Qs *= Q[k];
+    S *= Q[k];
   }
-  const double S = (neg ? -1.0 : 1.0) / sqrt(Qs);
-  float4* out = (fwd ? a.rpf : a.rpb) + r * kRoundPar;
   if (!on) return;
+  float4* out = (fwd ? a.rpf : a.rpb) + r * kRoundPar;
   if (e < 4) {
-    const uint32_t mr = (fwd ? m0 : m1) >> e & 1u, isrx = rx >> e & 1u;
-    // the table's q: T(t) or T(-k) applied, T(-t) or T(k) un-applied; an RY on a flipped pair: -q
-    const uint32_t kf = (K >> e) & 1u;
-    const bool neg_q = (fwd ? kf != 0 : kf == 0) != (mr && !isrx);
-    double g = Q[3];  // undoes the scales that the gradient value of item e carries
+    // the factor of rotation e's gradient value: 1 / (scale^2), less the rotations before it
+    double g = Q[3];
 #pragma unroll
     for (int k = 2; k >= 0; --k)
       if (k >= e) g *= Q[k];
-    out[e] = make_float4(neg_q ? -q : q, (float)(mr && !isrx && !fwd ? -g : g), (m0 >> e & 1u) ? -1.f : 1.f,
-                         __uint_as_float(e == 0 ? (fwd ? m1 : m0) : m1));
+    if (twice) g *= S;
+    out[e] = make_float4(fwd ? q : -q, (float)(twice ? -g : g), 0.f, 0.f);
   } else if (e < 12) {
-    // e^{i ang} for index e - 4 and its conjugate for the complement, times the round's scale, the Z's of
-    // flipped RYs, and (-i) (adjoint: i) per flipped RX; amplitude j sits in register j ^ (flips so far)
-    const uint32_t Kz = K & ~rx, nx = (uint32_t)__popc(K & rx) & 3u, md = fwd ? m1 : m0;
+    const double sc = (neg ? -1.0 : 1.0) * (twice ? 1.0 / S : rsqrt(S));
+    const float x0 = (float)(c * sc), y0 = (float)(s * sc);
     float2* ph = reinterpret_cast<float2*>(out + 4);
-    for (int h = 0; h < 2; ++h) {
-      const uint32_t j = h ? 15u - (uint32_t)(e - 4) : (uint32_t)(e - 4);
-      const bool sg = (h ? f1 : f0) != ((__popc((j ^ K) & Kz) & 1) != 0);
-      double x = c * S, y = (h ? -s : s) * S;
-      if (sg) { x = -x; y = -y; }
-      for (uint32_t k = 0; k < nx; ++k) {
-        const double t = x;
-        x = fwd ? y : -y;
-        y = fwd ? -t : t;
-      }
-      ph[j ^ md] = make_float2((float)x, (float)y);
-    }
+    ph[e - 4] = f0 ? make_float2(-x0, -y0) : make_float2(x0, y0);
+    ph[15 - (e - 4)] = f1 ? make_float2(-x0, y0) : make_float2(x0, -y0);
   }
 }
 

@@ -926,6 +926,7 @@ FusedPlan plan_fused_with(const Circuit& c_in, const PlanRequest& req, bool stri
     P.term_const.push_back(cst);
     return id;
   };
+  std::vector<std::pair<uint32_t, uint32_t>> step_links;  // of this pass: links inside the group, toggled links that leave it
   // A round step: forward rounds in order; the backward step runs the same
   // rounds in reverse, each one links first, then per item the RZ run and the RY.
   auto emit_round_step = [&](const Tile& tile, const StepRec& st, std::vector<Item>& bwd_items) {
@@ -934,6 +935,7 @@ FusedPlan plan_fused_with(const Circuit& c_in, const PlanRequest& req, bool stri
     for (int r = 0; r < 4; ++r) gq[r] = tile.local_to_global[gl[r]];
     const uint32_t fr0 = (uint32_t)(P.fwd_rounds.size() / kFwdRoundWords);
     std::vector<std::vector<int32_t>> brs;
+    uint32_t step_ext = 0;
     for (const RoundRec& rr : st.rounds) {
       uint32_t links = 0;
       for (int g : rr.czs) {
@@ -963,12 +965,17 @@ FusedPlan plan_fused_with(const Circuit& c_in, const PlanRequest& req, bool stri
       fw[4] = links;
       fw[5] = bbits;
       fw[6] = rx_mask;
-      fw[7] = (uint32_t)brs.size();  // the round's index in the step
+      // the links that leave the register group
+      uint32_t ext = links;
+      for (int r = 0; r < 3; ++r)
+        if ((bbits >> r) & 1u) ext &= ~(1u << gq[r]);
+      step_ext ^= ext;
+      fw[7] = ext;
       for (int r = 0; r < 8; ++r) fw[8 + r] = (uint32_t)bw[r];  // the items' terms (forward shears)
       bw[8] = (int32_t)links;
       bw[9] = (int32_t)bbits;
       bw[10] = (int32_t)rx_mask;
-      bw[11] = 0;
+      bw[11] = (int32_t)ext;
       P.has_rx |= rx_mask != 0;
       P.fwd_rounds.insert(P.fwd_rounds.end(), fw.begin(), fw.end());
       brs.push_back(std::move(bw));
@@ -980,11 +987,32 @@ FusedPlan plan_fused_with(const Circuit& c_in, const PlanRequest& req, bool stri
     ++P.n_steps;
     P.n_rounds += (int)nr;
     const uint32_t br0 = (uint32_t)(P.bwd_rounds.size() / kBwdRoundWords);
-    for (auto it = brs.rbegin(); it != brs.rend(); ++it) {
-      (*it)[11] = (int32_t)(it - brs.rbegin());
-      P.bwd_rounds.insert(P.bwd_rounds.end(), it->begin(), it->end());
-    }
+    for (auto it = brs.rbegin(); it != brs.rend(); ++it) P.bwd_rounds.insert(P.bwd_rounds.end(), it->begin(), it->end());
     bwd_items.push_back({{w0(OP_STEP, (uint32_t)st.group << 4 | nr << 8), br0}});
+    uint32_t inner = 0;
+    for (int r = 0; r < 3; ++r)
+      if (gq[r + 1] == gq[r] + 1) inner |= 1u << gq[r];
+    step_links.push_back({inner, step_ext});
+  };
+  // Pending CZ signs. A link that leaves the register group is a sign linear
+  // in the group's bits, and a rotation meets it by a sign of its own, so it
+  // need not be applied at the end of its step: it stays pending, on the next
+  // steps too, until a step whose group holds both its qubits, a checkpoint or
+  // the end of the pass. Marks the steps of [op0, end) that apply what is
+  // pending (bit kStepFlushBit). at: index into step_links, walked by dir.
+  auto mark_flushes = [&](std::vector<uint32_t>& ops, size_t op0, int at, int dir) {
+    uint32_t pend = 0;
+    const size_t end = ops.size() / 2;
+    for (size_t o = op0; o < end; ++o) {
+      if ((ops[2 * o] & 15u) != OP_STEP) continue;
+      pend ^= step_links[at].second;
+      at += dir;
+      const bool last = o + 1 == end || (ops[2 * (o + 1)] & 15u) != OP_STEP;
+      if (last || (pend & step_links[at].first)) {
+        ops[2 * o] |= 1u << kStepFlushBit;
+        pend = 0;
+      }
+    }
   };
   for (size_t pi = 0; pi < passes.size(); ++pi) {
     const PassRec& pr = passes[pi];
@@ -1008,6 +1036,7 @@ FusedPlan plan_fused_with(const Circuit& c_in, const PlanRequest& req, bool stri
     std::vector<std::vector<std::pair<uint32_t, uint32_t>>> bwd_items;
 
     const int n_steps = (int)pr.steps.size();
+    step_links.clear();
     int trailing_ckpt = -1;
     for (int si = 0; si < n_steps; ++si) {
       const StepRec& st = pr.steps[si];
@@ -1153,6 +1182,7 @@ FusedPlan plan_fused_with(const Circuit& c_in, const PlanRequest& req, bool stri
       }
     }
     fd.op_end = (int32_t)(P.fwd_ops.size() / 2);
+    if (P.rounds) mark_flushes(P.fwd_ops, (size_t)fd.op_begin, 0, 1);
     const bool last = pi + 1 == passes.size();
     fd.psi_src = pi == 0 ? SRC_GENERATE : (P.fwd.back().psi_dst >= 0 ? P.fwd.back().psi_dst : BUF_WORK);
     fd.psi_dst = last ? final_slot : (trailing_ckpt >= 0 ? trailing_ckpt : BUF_WORK);
@@ -1171,6 +1201,7 @@ FusedPlan plan_fused_with(const Circuit& c_in, const PlanRequest& req, bool stri
         P.bwd_ops.push_back(o.second);
       }
     bd.op_end = (int32_t)(P.bwd_ops.size() / 2);
+    if (P.rounds) mark_flushes(P.bwd_ops, (size_t)bd.op_begin, n_steps - 1, -1);
     P.bwd.push_back(bd);
   }
   // backward pass order is the reverse of the forward one

@@ -37,35 +37,37 @@ enum OpCode : uint32_t {
                   // or the control's global qubit index (a bit of the thread's base index)
 };
 
-// Round programs: a step is OP_STEP {w0: group (bits 4-5) | rounds << 8,
-// w1: first round}; every round applies one item per register bit r = 0..3
+// Round programs: a step is OP_STEP {w0: group (bits 4-5) | rounds << 8 |
+// flush << kStepFlushBit, w1: first round}; flush: the complex64 kernels apply
+// the CZ signs pending after this step (elsewhere they stay pending); every round applies one item per register bit r = 0..3
 // and then the CZ links of the round.
 //   forward round, kFwdRoundWords words: m[4] (fused 2x2 index per register
 //     bit, 0 = identity), links, bbits (links between register bits r, r+1),
-//     rx (bit r: item r's rotation is an RX), the round's index in its step,
-//     tz[4], ty[4] (the items' gradient terms, as below).
+//     rx (bit r: item r's rotation is an RX), the links that leave the
+//     register group, tz[4], ty[4] (the items' gradient terms, as below).
 //   backward round, kBwdRoundWords words: tz[4], ty[4] (term of the merged RZ
 //     run and of the rotation of each item, -1 = none), links, bbits, rx, the
-//     round's index in its step.
+//     links that leave the group.
 // An item is an RZ run alone or a rotation (RY or RX) followed by an RZ run.
 // A forward round applies per item the rotation and then the RZ run, then the
 // links; a backward step runs its rounds in the order stored, each applying
 // the links first, then per item the RZ run and then the rotation (the exact
 // reverse).
+constexpr int kStepFlushBit = 24;
 constexpr int kFwdRoundWords = 16;
 constexpr int kBwdRoundWords = 12;
 constexpr int kMaxStepRounds = 4;   // 8 gradient values per round
-// Parameters of one round of a complex64 round program, in float4. [0, 4): the
-// 4 items' rotations: x = q of [[1, -q], [q, 1]] (|q| <= 1), y and z = the
-// factors of the adjoint's gradient values of the item's rotation and RZ run,
-// w = a mask of register bits as an integer (item 0: the flips in force where
-// the round's links act, the others: those after the round; register p holds
-// amplitude p ^ mask). [4, 12): the round's diagonal, i.e. the 4 RZ runs (and
-// the CZ links between register bits) merged into one phase per register p,
-// two per float4, times the scales, signs and phases that the 4 rotations in
-// their reduced form leave out. Prep fills them with 16 lanes per round;
-// complex128 programs hold shears and phases in float64 (RoundPar64).
+// Parameters of one round of a complex64 round program, in float4: [0, 4) the 4
+// items' rotations, x = q and y = the factor of the adjoint's gradient value of
+// the rotation (negative: the round runs twice); [4, 12) the round's diagonal,
+// i.e. the 4 RZ runs (and the CZ links between register bits) merged into one
+// phase per register index, two per float4, times the scale and sign that the
+// rotations leave out. (The four q's in one float4 would be loaded together,
+// and the adjoint has no registers for that: it spilled, 3 % slower.) Prep
+// fills them with 16 lanes per round; complex128 programs hold shears and
+// phases in float64 (RoundPar64).
 constexpr int kRoundPar = 12;
+constexpr double kMaxTan = 256.0;   // largest |tan(w/2)| of a round that runs its rotations once
 
 // Source / destination codes of a pass.
 enum : int32_t {

@@ -6,9 +6,13 @@
 // pass's step program on them in shared memory and registers, and stores them
 // once: the forward and backward gate fusion of Secs. 3.2-3.3.
 //
-// Shared-memory layout: amplitude with local index i lives at i ^ ((i>>4)&15)
-// (XOR swizzle on 8-byte words). Register groups are local nibbles, so the 16
-// lanes of a half-warp always hit 16 distinct bank pairs.
+// Shared-memory layout: amplitude with local index i lives at i + (i >> 4), one
+// 8-byte word of padding per 16, so that the 16 lanes of a half-warp hit 16
+// distinct bank pairs for every register group (4 consecutive local bits b ..
+// b + 3). The place of register j is then the thread's base plus a constant of
+// (b, j): loads and stores of a step carry it as their immediate offset, one
+// code copy per b. An XOR swizzle (i ^ ((i >> 4) & 15)) needed an instruction
+// or two per address, about 70 a step and thread.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -25,7 +29,8 @@ __device__ int g_qf_device_status = 0;
 
 namespace {
 
-__device__ __forceinline__ uint32_t swz(uint32_t i) { return i ^ ((i >> 4) & 15u); }
+__device__ __forceinline__ constexpr uint32_t loc(uint32_t i) { return i + (i >> 4); }
+constexpr int kTilePad = kTileAmps + kTileAmps / 16;  // words of a CTA's share of one state
 
 // Scatter the low bits of src into the set bits of mask (ascending).
 __device__ __forceinline__ uint32_t pdep32(uint32_t src, uint32_t mask) {
@@ -42,19 +47,74 @@ __device__ __forceinline__ float flip(float v, uint32_t s) {
   return __int_as_float(__float_as_int(v) ^ (int)(s << 31));
 }
 
-// Pair (i, i+1), i even, to/from the swizzled tile.
-__device__ __forceinline__ void st_pair(float2* sm, uint32_t i, float4 v) {
-  const uint32_t p = swz(i);
-  if (p & 1u) *reinterpret_cast<float4*>(sm + (p ^ 1u)) = make_float4(v.z, v.w, v.x, v.y);
-  else *reinterpret_cast<float4*>(sm + p) = v;
+// Pair (i, i+1), i even, to/from the padded tile (two 8-byte accesses, free of
+// bank conflicts as the pairs of 16 consecutive lanes are).
+__device__ __forceinline__ void st_pair(float2* sm, uint32_t p, float4 v) {
+  sm[p] = make_float2(v.x, v.y);
+  sm[p + 1] = make_float2(v.z, v.w);
 }
-__device__ __forceinline__ float4 ld_pair(const float2* sm, uint32_t i) {
-  const uint32_t p = swz(i);
-  if (p & 1u) {
-    const float4 v = *reinterpret_cast<const float4*>(sm + (p ^ 1u));
-    return make_float4(v.z, v.w, v.x, v.y);
+__device__ __forceinline__ float4 ld_pair(const float2* sm, uint32_t p) {
+  const float2 a = sm[p], b = sm[p + 1];
+  return make_float4(a.x, a.y, b.x, b.y);
+}
+
+// The 16 registers of a group on local bits B .. B + 3, at the thread's base.
+template <int B>
+__device__ __forceinline__ constexpr int group_off(int j) {
+  int o = 0;
+  for (int r = 0; r < 4; ++r)
+    if ((j >> r) & 1) o += (int)loc(1u << (B + r));
+  return o;
+}
+template <int B>
+__device__ __forceinline__ void ld16(const float2* at, float2 (&r)[16]) {
+#pragma unroll
+  for (int j = 0; j < 16; ++j) r[j] = at[group_off<B>(j)];
+}
+template <int B>
+__device__ __forceinline__ void st16(float2* at, const float2 (&r)[16]) {
+#pragma unroll
+  for (int j = 0; j < 16; ++j) at[group_off<B>(j)] = r[j];
+}
+// The group's lowest local bit b is one of these in round programs (K = 7 .. 12:
+// 0, 4, 8 and K - 4; KC = 12: 0, 4, 8). at2: lambda's place (adjoint).
+template <int KC, bool BWD>
+__device__ __forceinline__ void ld_group(uint32_t b, const float2* at, const float2* at2, float2 (&r)[16],
+                                         float2 (&l)[16]) {
+#define QF_LD(B) { ld16<B>(at, r); if (BWD) ld16<B>(at2, l); }
+  if (KC == 12) {
+    if (b == 0) QF_LD(0) else if (b == 4) QF_LD(4) else QF_LD(8)
+  } else {
+    switch (b) {
+      case 0: QF_LD(0) break;
+      case 3: QF_LD(3) break;
+      case 4: QF_LD(4) break;
+      case 5: QF_LD(5) break;
+      case 6: QF_LD(6) break;
+      case 7: QF_LD(7) break;
+      default: QF_LD(8) break;
+    }
   }
-  return *reinterpret_cast<const float4*>(sm + p);
+#undef QF_LD
+}
+template <int KC, bool BWD>
+__device__ __forceinline__ void st_group(uint32_t b, float2* at, float2* at2, const float2 (&r)[16],
+                                         const float2 (&l)[16]) {
+#define QF_ST(B) { st16<B>(at, r); if (BWD) st16<B>(at2, l); }
+  if (KC == 12) {
+    if (b == 0) QF_ST(0) else if (b == 4) QF_ST(4) else QF_ST(8)
+  } else {
+    switch (b) {
+      case 0: QF_ST(0) break;
+      case 3: QF_ST(3) break;
+      case 4: QF_ST(4) break;
+      case 5: QF_ST(5) break;
+      case 6: QF_ST(6) break;
+      case 7: QF_ST(7) break;
+      default: QF_ST(8) break;
+    }
+  }
+#undef QF_ST
 }
 
 // ---- forward: fused 2x2 on register bit R -----------------------------------
@@ -145,8 +205,7 @@ __device__ __forceinline__ void cnot_regs(float2 (&r)[16], float2 (&l)[16], bool
 }
 
 __device__ __forceinline__ uint32_t reg_off(uint32_t j, const uint32_t (&o)[4]) {
-  return ((j & 1u) ? o[0] : 0u) ^ ((j & 2u) ? o[1] : 0u) ^ ((j & 4u) ? o[2] : 0u) ^
-         ((j & 8u) ? o[3] : 0u);
+  return ((j & 1u) ? o[0] : 0u) + ((j & 2u) ? o[1] : 0u) + ((j & 4u) ? o[2] : 0u) + ((j & 8u) ? o[3] : 0u);
 }
 
 // phase i^k times v
@@ -623,19 +682,25 @@ struct PassShared {
   float4 ident[8];             // the diagonal of a round's run that has none
   uint32_t ticket;             // the CTA's finishing order (loss on the last CTA)
   uint32_t lg[256];
-  uint32_t base[4][kThreads];  // per register group: the thread's tile index with the group's bits zero
   float red[2][kThreads / 32][kMaxStepSlots];
   int32_t slot[2][kMaxStepSlots];
   double dred[kThreads / 32];
   uint32_t gmap[16];
-  uint32_t grp[4][4];
+  uint32_t gb[4];              // per register group: its lowest local bit
+  uint4 gpos[4];               // and its qubits
 };
 
 // One CTA's share of a pass: tiles first_tile .. first_tile + tiles_per_cta-1
 // (tile = sample * tiles_per_sample + tile within the sample). Ends with a
 // barrier, so a CTA may call it again for another pass or tile range. LOADS:
 // tile loads in flight per thread and state (8 = the whole tile at once).
-template <bool BWD, bool ROUNDS, int LOADS = 8, bool TC = false, bool RX = false>
+// KC: the tile's qubits where they are known when compiled (12: one tile per
+// CTA of 256 threads, every tile active), else 0. The constant lets the tile
+// loads, the group bases and the reductions drop their index arithmetic: with
+// the padded layout, 366 -> 291 instructions per warp and round forward and 786
+// -> 659 adjoint; step of n = 20, d = 24, 64 samples 25.10 -> 23.00 ms, of n =
+// 12, d = 20, 256 samples 237 -> 222 us.
+template <bool BWD, bool ROUNDS, int LOADS = 8, bool TC = false, bool RX = false, int KC = 0>
 __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_tile, float2* smem, PassShared& sh,
                                          const TcCtx* tc = nullptr) {
   uint32_t (&s_lg)[256] = sh.lg;
@@ -643,33 +708,36 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
   int32_t (&s_slot)[2][kMaxStepSlots] = sh.slot;
   double (&s_dred)[kThreads / 32] = sh.dred;
   uint32_t (&s_gmap)[16] = sh.gmap;
-  uint32_t (&s_grp)[4][4] = sh.grp;
 
   const PassDesc& pd = a.pd;
-  const int K = pd.K;
+  const int K = KC ? KC : pd.K;
   const int tl2 = K - kRegBits;            // log2 threads per tile
   const int Tt = 1 << tl2;
   const int tid = threadIdx.x;
   const int lane = tid & 31, warp = tid >> 5;
-  const int tile_in_cta = tid >> tl2;
-  const uint32_t tau = (uint32_t)(tid & (Tt - 1));
-  const int tiles_per_cta = kThreads >> tl2;
+  const int tile_in_cta = KC ? 0 : tid >> tl2;
+  const uint32_t tau = KC ? (uint32_t)tid : (uint32_t)(tid & (Tt - 1));
+  const int tiles_per_cta = KC ? 1 : kThreads >> tl2;
   const int64_t total_tiles = (int64_t)a.B << a.tps_log2;
   const int64_t tile = first_tile + tile_in_cta;
-  const bool active = tile < total_tiles;
+  const bool active = KC || tile < total_tiles;
   const int64_t b = active ? (tile >> a.tps_log2) : 0;
   const uint32_t t_in = active ? (uint32_t)(tile & ((1ll << a.tps_log2) - 1)) : 0u;
   const uint32_t outer = pdep32(t_in, pd.outer_mask);
   const int64_t dim = 1ll << a.n_eff;
   const int64_t sbase = b * dim;  // sample offset inside one state buffer
-  float2* tp = smem + (tile_in_cta << K);
-  float2* tl = smem + kTileAmps + (tile_in_cta << K);
+  float2* tp = smem + (tile_in_cta << K) + (tile_in_cta << tl2);  // loc(tile_in_cta << K)
+  float2* tl = tp + kTilePad;
   const int wpt = Tt >= 32 ? Tt / 32 : 1;  // warps per tile
   const int lanes = Tt < 32 ? Tt : 32;
 
   if (tid < 16) {
     s_gmap[tid] = pd.gmap[tid];
-    s_grp[tid >> 2][tid & 3] = pd.groups[tid >> 2][tid & 3];
+    if (tid < 4) {
+      sh.gb[tid] = pd.groups[tid][0];
+      sh.gpos[tid] = make_uint4(pd.gmap[pd.groups[tid][0] & 15], pd.gmap[pd.groups[tid][1] & 15],
+                                pd.gmap[pd.groups[tid][2] & 15], pd.gmap[pd.groups[tid][3] & 15]);
+    }
     if (ROUNDS && tid < 8) sh.ident[tid] = make_float4(1.f, 0.f, 1.f, 0.f);
   }
   __syncthreads();
@@ -680,34 +748,22 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
     s_lg[h] = g;
   }
   __syncthreads();
-  // each thread's base index per register group, once per pass (read back by
-  // only the same thread, at every step of that group): computed while the
-  // tile loads are in flight where the pass loads its tiles
-  bool bases = false;
-  auto set_bases = [&]() {
-    for (int g = 0; g < 4; ++g) {
-      // tau's bits scattered into the tile bits outside the group (pdep32 of
-      // tau into the complement of the group's bits): a zero inserted at each
-      // of the 4 group bits, lowest first, so that 4 steps replace K - 4
-      uint32_t m = (1u << s_grp[g][0]) | (1u << s_grp[g][1]) | (1u << s_grp[g][2]) | (1u << s_grp[g][3]);
-      uint32_t x = tau;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const uint32_t low = m & (0u - m);
-        const uint32_t hi = x & ~(low - 1u);
-        x = (x ^ hi) | (hi << 1);
-        m ^= low;
-      }
-      sh.base[g][tid] = x;
-    }
-    bases = true;
-  };
-  // (the persistent batch kernel and the RX instances keep the bases ahead
-  // of the loads: their registers are tighter)
-  constexpr bool kBasesInLoads = LOADS == 8 && !RX && !TC;
-  if (!kBasesInLoads) set_bases();
 
   auto gidx = [&](uint32_t i) -> uint32_t { return outer | (i & 15u) | s_lg[i >> 4]; };
+  // A thread's share of the tile is the pairs i = 2 (it Tt + tau), it = 0..7:
+  // it is the local bits K-3 .. K-1, so the global index splits into the
+  // thread's part and `it_bits` (uniform), and the place in shared memory into
+  // the thread's part and it * loc(2 Tt) (for Tt >= 8, where 2 Tt is a
+  // multiple of 16)
+  const uint32_t g_tau = gidx(2u * tau), p_tau = loc(2u * tau);
+  auto it_bits = [&](int it) -> uint32_t {
+    return ((it & 1) ? 1u << pd.gmap[K - 3] : 0u) | ((it & 2) ? 1u << pd.gmap[K - 2] : 0u) |
+           ((it & 4) ? 1u << pd.gmap[K - 1] : 0u);
+  };
+  auto g_it = [&](int it) -> uint32_t { return g_tau | it_bits(it); };
+  auto p_it = [&](int it) -> uint32_t {
+    return KC ? p_tau + (uint32_t)it * loc(2u * 256u) : loc(2u * ((uint32_t)it * Tt + tau));
+  };
   auto state_ptr = [&](int32_t code) -> float2* {
     if (code >= 0) return a.slots + (int64_t)code * a.slot_stride + sbase;
     return a.work + sbase;
@@ -753,8 +809,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
     const float2* src = a.psi_in + b * din;
 #pragma unroll
     for (int it = 0; it < 8; ++it) {
-      const uint32_t i = 2u * ((uint32_t)it * Tt + tau);
-      const uint32_t g = gidx(i);
+      const uint32_t g = g_it(it);
       float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
       if (a.n_in == a.n_eff) {
         v = __ldcg(reinterpret_cast<const float4*>(src + g));
@@ -762,22 +817,28 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
         const float2 u0 = src[g], u1 = (int64_t)g + 1 < din ? src[g + 1] : make_float2(0.f, 0.f);
         v = make_float4(u0.x, u0.y, u1.x, u1.y);
       }
-      if (active) st_pair(tp, i, v);
+      if (active) st_pair(tp, p_it(it), v);
     }
   } else if (psrc == SRC_GENERATE) {
-    // psi_0 = (x) RY(x_q)|0>: a_x = prod_q (bit q of x ? sin(x_q/2) : cos(x_q/2))
+    // psi_0 = (x) RY(x_q)|0>: a_x = prod_q (bit q of x ? sin(x_q/2) : cos(x_q/2));
+    // the thread's pairs share every factor but those of qubit 0 and the
+    // three local bits K-3 .. K-1
     const float2* e = a.enc + b * a.n_eff;
-#pragma unroll 1
-    for (int it = 0; it < 8; ++it) {
-      const uint32_t i = 2u * ((uint32_t)it * Tt + tau);
-      const uint32_t g = gidx(i);
-      float pr = 1.f;
-      for (int q = 1; q < a.n_eff; ++q) {
-        const float2 f = __ldg(e + q);
-        pr *= ((g >> q) & 1u) ? f.y : f.x;
+    const uint32_t vary = it_bits(7);
+    float pr = 1.f;
+    for (int q = 1; q < a.n_eff; ++q) {
+      if ((vary >> q) & 1u) continue;
+      const float2 f = __ldg(e + q);
+      pr *= ((g_tau >> q) & 1u) ? f.y : f.x;
+    }
+    const float2 f0 = __ldg(e), e0 = __ldg(e + pd.gmap[K - 3]), e1 = __ldg(e + pd.gmap[K - 2]),
+                 e2 = __ldg(e + pd.gmap[K - 1]);
+    if (active) {
+#pragma unroll
+      for (int it = 0; it < 8; ++it) {
+        const float v = pr * ((it & 1) ? e0.y : e0.x) * ((it & 2) ? e1.y : e1.x) * ((it & 4) ? e2.y : e2.x);
+        st_pair(tp, p_it(it), make_float4(v * f0.x, 0.f, v * f0.y, 0.f));
       }
-      const float2 f0 = __ldg(e);
-      if (active) st_pair(tp, i, make_float4(pr * f0.x, 0.f, pr * f0.y, 0.f));
     }
   } else if (active) {
     // issue every load of the tile (psi, and lambda) before the first store
@@ -792,28 +853,22 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
       float4 vp[LOADS], vl[LOADS];
 #pragma unroll
       for (int it = 0; it < LOADS; ++it) {
-        const uint32_t g = gidx(2u * ((uint32_t)(i0 + it) * Tt + tau));
+        const uint32_t g = g_it(i0 + it);
         if (half) vp[it] = bf16x4_to_f4(__ldcg(reinterpret_cast<const uint2*>(hsrc + g)));
         else vp[it] = __ldcg(reinterpret_cast<const float4*>(src + g));
         if (two) vl[it] = __ldcg(reinterpret_cast<const float4*>(lsrc + g));
       }
-      if (kBasesInLoads && i0 == 0) set_bases();
 #pragma unroll
       for (int it = 0; it < LOADS; ++it) {
-        const uint32_t i = 2u * ((uint32_t)(i0 + it) * Tt + tau);
-        st_pair(tp, i, vp[it]);
-        if (two) st_pair(tl, i, vl[it]);
+        st_pair(tp, p_it(i0 + it), vp[it]);
+        if (two) st_pair(tl, p_it(i0 + it), vl[it]);
       }
     }
   }
-  if (!bases) set_bases();
   if (BWD && pd.lam_src == LAM_BUF && psrc == SRC_GENERATE && active) {
     const float2* src = a.lam + sbase;
 #pragma unroll
-    for (int it = 0; it < 8; ++it) {
-      const uint32_t i = 2u * ((uint32_t)it * Tt + tau);
-      st_pair(tl, i, __ldcg(reinterpret_cast<const float4*>(src + gidx(i))));
-    }
+    for (int it = 0; it < 8; ++it) st_pair(tl, p_it(it), __ldcg(reinterpret_cast<const float4*>(src + g_it(it))));
   }
   // round programs: stage the first step's parameters
   int sb = 0;
@@ -839,10 +894,10 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
       const uint32_t i = (uint32_t)it * Tt + tau;  // single amplitudes here
       const uint32_t ip = i ^ pd.xm_local;
       const uint32_t gp = gidx(ip);
-      float2 v = tp[swz(ip)];
+      float2 v = tp[loc(ip)];
       v = mul_ipow(v, a.y_count);
       const uint32_t sg = __popc(gp & a.z_mask) & 1u;
-      tl[swz(i)] = make_float2(flip(v.x, sg) * scale, flip(v.y, sg) * scale);
+      tl[loc(i)] = make_float2(flip(v.x, sg) * scale, flip(v.y, sg) * scale);
     }
     __syncthreads();
   }
@@ -872,19 +927,16 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
         if (next_step(pc, rb, nr2)) stage_b(sb ^ 1, rb, nr2);
       }
       const StepPar& P = sh.par[sb];
-      const uint32_t lb0 = s_grp[g][0], lb1 = s_grp[g][1], lb2 = s_grp[g][2], lb3 = s_grp[g][3];
-      const uint32_t base = sh.base[g][tid];
-      const uint32_t pb = swz(base);
-      const uint32_t so[4] = {swz(1u << lb0), swz(1u << lb1), swz(1u << lb2), swz(1u << lb3)};
+      const uint32_t lb = KC ? 4u * (uint32_t)g : sh.gb[g];
+      // tau's bits around the group's (a zero in each of its four)
+      const uint32_t base = (tau & ((1u << lb) - 1u)) | ((tau >> lb) << (lb + 4u));
+      float2* const at = tp + loc(base);
       const uint32_t gb = gidx(base);
-      const uint32_t pos[4] = {s_gmap[lb0], s_gmap[lb1], s_gmap[lb2], s_gmap[lb3]};
+      const uint4 gp = sh.gpos[g];
+      const uint32_t pos[4] = {gp.x, gp.y, gp.z, gp.w};
       float2 r[16];
       float2 l[16];
-#pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        r[j] = tp[pb ^ reg_off(j, so)];
-        if (BWD) l[j] = tl[pb ^ reg_off(j, so)];
-      }
+      ld_group<KC, BWD>(lb, at, at + kTilePad, r, l);
       const int nq = a.n_eff;
       const uint32_t nmask = nq >= 32 ? ~0u : ((1u << nq) - 1u);
       const uint32_t rgb = ((gb >> 1) | ((gb & 1u) << (nq - 1))) & nmask;
@@ -958,11 +1010,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
         pend = 0;
       }
       }  // CUDA-core rounds
-#pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        tp[pb ^ reg_off(j, so)] = r[j];
-        if (BWD) tl[pb ^ reg_off(j, so)] = l[j];
-      }
+      st_group<KC, BWD>(lb, at, at + kTilePad, r, l);
       if (TC) {
         cp_async_wait_all();
         fence_proxy_async();
@@ -1012,19 +1060,19 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
       const int g = (op.x >> 4) & 3;
       const int nops = (op.x >> 8) & 0xffff;
       const int nk = (int)op.y;
-      const uint32_t lb0 = s_grp[g][0], lb1 = s_grp[g][1], lb2 = s_grp[g][2], lb3 = s_grp[g][3];
-      const uint32_t base = sh.base[g][tid];
-      const uint32_t pb = swz(base);
-      const uint32_t so[4] = {swz(1u << lb0), swz(1u << lb1), swz(1u << lb2), swz(1u << lb3)};
+      const uint32_t lb = sh.gb[g];
+      const uint32_t base = (tau & ((1u << lb) - 1u)) | ((tau >> lb) << (lb + 4u));
+      float2* const at = tp + loc(base);
+      const uint32_t so[4] = {loc(1u << lb), loc(2u << lb), loc(4u << lb), loc(8u << lb)};
       const uint32_t gb = gidx(base);
-      const uint32_t go[4] = {1u << s_gmap[lb0], 1u << s_gmap[lb1], 1u << s_gmap[lb2],
-                              1u << s_gmap[lb3]};
+      const uint4 gp = sh.gpos[g];
+      const uint32_t go[4] = {1u << gp.x, 1u << gp.y, 1u << gp.z, 1u << gp.w};
       float2 r[16];
       float2 l[16];
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
-        r[j] = tp[pb ^ reg_off(j, so)];
-        if (BWD) l[j] = tl[pb ^ reg_off(j, so)];
+        r[j] = at[reg_off(j, so)];
+        if (BWD) l[j] = at[kTilePad + reg_off(j, so)];
       }
 #pragma unroll 1
       for (int k = 0; k < nops; ++k) {
@@ -1080,8 +1128,8 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
       }
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
-        tp[pb ^ reg_off(j, so)] = r[j];
-        if (BWD) tl[pb ^ reg_off(j, so)] = l[j];
+        at[reg_off(j, so)] = r[j];
+        if (BWD) at[kTilePad + reg_off(j, so)] = l[j];
       }
       __syncthreads();
       if (BWD && Tt >= 32) {
@@ -1100,10 +1148,9 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
       float2* sp = a.slots + (int64_t)op.y * a.slot_stride + sbase;
 #pragma unroll
       for (int it = 0; it < 8; ++it) {
-        const uint32_t i = 2u * ((uint32_t)it * Tt + tau);
         if (!active) continue;
-        if (code == OP_CKPT) *reinterpret_cast<float4*>(sp + gidx(i)) = ld_pair(tp, i);
-        else st_pair(tp, i, *reinterpret_cast<const float4*>(sp + gidx(i)));
+        if (code == OP_CKPT) *reinterpret_cast<float4*>(sp + g_it(it)) = ld_pair(tp, p_it(it));
+        else st_pair(tp, p_it(it), *reinterpret_cast<const float4*>(sp + g_it(it)));
       }
       __syncthreads();
     }
@@ -1115,23 +1162,20 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
     __nv_bfloat162* dst = reinterpret_cast<__nv_bfloat162*>(a.hslots) + (int64_t)pd.psi_dst * a.slot_stride + sbase;
 #pragma unroll
     for (int it = 0; it < 8; ++it) {
-      const uint32_t i = 2u * ((uint32_t)it * Tt + tau);
-      if (active) *reinterpret_cast<uint2*>(dst + gidx(i)) = f4_to_bf16x4(ld_pair(tp, i));
+      if (active) *reinterpret_cast<uint2*>(dst + g_it(it)) = f4_to_bf16x4(ld_pair(tp, p_it(it)));
     }
   } else if (pd.psi_dst != BUF_NONE) {
     float2* dst = state_ptr(pd.psi_dst);
 #pragma unroll
     for (int it = 0; it < 8; ++it) {
-      const uint32_t i = 2u * ((uint32_t)it * Tt + tau);
-      if (active) *reinterpret_cast<float4*>(dst + gidx(i)) = ld_pair(tp, i);
+      if (active) *reinterpret_cast<float4*>(dst + g_it(it)) = ld_pair(tp, p_it(it));
     }
   }
   if (BWD && pd.lam_dst == LAM_BUF) {
     float2* dst = a.lam + sbase;
 #pragma unroll
     for (int it = 0; it < 8; ++it) {
-      const uint32_t i = 2u * ((uint32_t)it * Tt + tau);
-      if (active) *reinterpret_cast<float4*>(dst + gidx(i)) = ld_pair(tl, i);
+      if (active) *reinterpret_cast<float4*>(dst + g_it(it)) = ld_pair(tl, p_it(it));
     }
   }
   if (!BWD && (pd.flags & PF_EXPECT)) {
@@ -1141,8 +1185,8 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
     for (int it = 0; it < 16; ++it) {
       const uint32_t i = (uint32_t)it * Tt + tau;
       const uint32_t ip = i ^ pd.xm_local;
-      const float2 v = tp[swz(i)];
-      float2 w = mul_ipow(tp[swz(ip)], a.y_count);
+      const float2 v = tp[loc(i)];
+      float2 w = mul_ipow(tp[loc(ip)], a.y_count);
       const uint32_t sg = __popc(gidx(ip) & a.z_mask) & 1u;
       acc += flip(v.x * w.x + v.y * w.y, sg);  // Re(conj(v) w) with the Z signs
     }
@@ -1185,11 +1229,12 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
 // of RZ / RY items keep the plain code). MINB: CTAs per SM the registers are
 // budgeted for; a forward pass (one 32 KiB state per CTA) of more tiles than
 // two CTAs per SM hold runs with three per SM.
-template <bool BWD, bool ROUNDS, bool RX = false, int MINB = 2>
+template <bool BWD, bool ROUNDS, bool RX = false, int MINB = 2, int KC = 0>
 __global__ void __launch_bounds__(kThreads, MINB) pass_kernel(const PassArgs a) {
   extern __shared__ __align__(16) float2 smem[];
   __shared__ PassShared sh;
-  pass_cta<BWD, ROUNDS, 8, false, RX>(a, (int64_t)blockIdx.x * (kThreads >> (a.pd.K - kRegBits)), smem, sh);
+  const int64_t first = KC ? (int64_t)blockIdx.x : (int64_t)blockIdx.x * (kThreads >> (a.pd.K - kRegBits));
+  pass_cta<BWD, ROUNDS, 8, false, RX, KC>(a, first, smem, sh);
 }
 
 // Forward pass with the rounds on the tensor cores: one 12-qubit tile per
@@ -1215,8 +1260,8 @@ __global__ void __launch_bounds__(kThreads, 2) tc_pass_kernel(const PassArgs a) 
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  TcCtx ctx{tmem_slot, mbar, reinterpret_cast<float*>(smem + kTileAmps)};
-  pass_cta<false, true, 8, true>(a, (int64_t)blockIdx.x, smem, sh, &ctx);
+  TcCtx ctx{tmem_slot, mbar, reinterpret_cast<float*>(smem + kTilePad)};
+  pass_cta<false, true, 8, true, false, 12>(a, (int64_t)blockIdx.x, smem, sh, &ctx);
   // pass_cta ends with a barrier; every tensor-memory access is complete
   tc_fence_after();
   if (warp == 0)
@@ -1814,7 +1859,7 @@ int batch_grid() { return 2 * device_sms(); }
 
 cudaError_t launch_batch(const BatchArgs& a, int grid, int64_t prep_total, int64_t n_grad_out, cudaStream_t st) {
   static OptIn once;
-  const size_t smem = 2 * (size_t)kTileAmps * sizeof(float2);
+  const size_t smem = 2 * (size_t)kTilePad * sizeof(float2);
   cudaError_t e = opt_in(reinterpret_cast<const void*>(batch_kernel), smem, once);
   if (e != cudaSuccess) return e;
   if (prep_total > 0) batch_prep_kernel<<<(unsigned)((prep_total + 63) / 64), 64, 0, st>>>(a, prep_total);
@@ -1847,31 +1892,40 @@ cudaError_t launch_pass(bool bwd, const PassArgs& a, cudaStream_t st, int fwd_ct
   const int64_t total_tiles = (int64_t)a.B << a.tps_log2;
   const int64_t grid = (total_tiles + tiles_per_cta - 1) / tiles_per_cta;
   if (grid == 0) return cudaSuccess;
-  const size_t smem = (size_t)(bwd ? 2 : 1) * kTileAmps * sizeof(float2);
+  const size_t smem = (size_t)(bwd ? 2 : 1) * kTilePad * sizeof(float2);
   const bool rounds = a.rounds != nullptr, rx = rounds && a.rx_items;
+  // 12-qubit tiles run the instances compiled for them; a single-wave forward
+  // keeps the 128-register instance, more tiles than two CTAs per SM hold run
+  // with three per SM (fewer registers, more warps to hide latency across waves)
+  const int n_sm = device_sms();
+  if (n_sm == 0) return cudaErrorInvalidDevice;
+  const bool k12 = a.pd.K == kMaxTileBits;
+  const bool three = rounds && !bwd && (fwd_ctas == 3 || (fwd_ctas == 0 && grid > 2ll * n_sm));
+#define QF_RUN(...)                                                                          \
+  do {                                                                                       \
+    static OptIn once;                                                                       \
+    const cudaError_t e_ = opt_in(reinterpret_cast<const void*>(__VA_ARGS__), smem, once);   \
+    if (e_ != cudaSuccess) return e_;                                                        \
+    __VA_ARGS__<<<(unsigned)grid, kThreads, smem, st>>>(a);                                  \
+    return cudaGetLastError();                                                               \
+  } while (0)
   if (bwd) {
-    // 64 KiB of dynamic shared memory needs the opt-in
-    static OptIn once_generic, once_rounds, once_rx;
-    cudaError_t e = rx       ? opt_in(reinterpret_cast<const void*>(pass_kernel<true, true, true>), smem, once_rx)
-                    : rounds ? opt_in(reinterpret_cast<const void*>(pass_kernel<true, true>), smem, once_rounds)
-                             : opt_in(reinterpret_cast<const void*>(pass_kernel<true, false>), smem, once_generic);
-    if (e != cudaSuccess) return e;
-    if (rx) pass_kernel<true, true, true><<<(unsigned)grid, kThreads, smem, st>>>(a);
-    else if (rounds) pass_kernel<true, true><<<(unsigned)grid, kThreads, smem, st>>>(a);
-    else pass_kernel<true, false><<<(unsigned)grid, kThreads, smem, st>>>(a);
-  } else {
-    // more tiles than two CTAs per SM hold: the three-CTA round instances
-    // (fewer registers, more warps to hide latency across the waves)
-    const int n_sm = device_sms();
-    if (n_sm == 0) return cudaErrorInvalidDevice;
-    const bool three = rounds && (fwd_ctas == 3 || (fwd_ctas == 0 && grid > 2ll * n_sm));
-    if (rx && three) pass_kernel<false, true, true, 3><<<(unsigned)grid, kThreads, smem, st>>>(a);
-    else if (rx) pass_kernel<false, true, true><<<(unsigned)grid, kThreads, smem, st>>>(a);
-    else if (three) pass_kernel<false, true, false, 3><<<(unsigned)grid, kThreads, smem, st>>>(a);
-    else if (rounds) pass_kernel<false, true><<<(unsigned)grid, kThreads, smem, st>>>(a);
-    else pass_kernel<false, false><<<(unsigned)grid, kThreads, smem, st>>>(a);
+    if (!rounds) QF_RUN(pass_kernel<true, false>);
+    if (rx && k12) QF_RUN(pass_kernel<true, true, true, 2, 12>);
+    if (rx) QF_RUN(pass_kernel<true, true, true>);
+    if (k12) QF_RUN(pass_kernel<true, true, false, 2, 12>);
+    QF_RUN(pass_kernel<true, true>);
   }
-  return cudaGetLastError();
+  if (!rounds) QF_RUN(pass_kernel<false, false>);
+  if (rx && k12 && three) QF_RUN(pass_kernel<false, true, true, 3, 12>);
+  if (rx && k12) QF_RUN(pass_kernel<false, true, true, 2, 12>);
+  if (rx && three) QF_RUN(pass_kernel<false, true, true, 3>);
+  if (rx) QF_RUN(pass_kernel<false, true, true>);
+  if (k12 && three) QF_RUN(pass_kernel<false, true, false, 3, 12>);
+  if (k12) QF_RUN(pass_kernel<false, true, false, 2, 12>);
+  if (three) QF_RUN(pass_kernel<false, true, false, 3>);
+  QF_RUN(pass_kernel<false, true>);
+#undef QF_RUN
 }
 
 // ---- observables whose X/Y qubits lie outside the tile (App. B.2) ---------------
@@ -1940,7 +1994,7 @@ cudaError_t launch_pass_tc(const PassArgs& a, cudaStream_t st) {
   if (a.pd.K != kMaxTileBits || a.rounds == nullptr || a.tcb == nullptr) return cudaErrorInvalidValue;
   const int64_t grid = (int64_t)a.B << a.tps_log2;
   if (grid == 0) return cudaSuccess;
-  const size_t smem = (size_t)kTileAmps * sizeof(float2) + (size_t)2 * kMaxStepRounds * kTcBFloats * sizeof(float);
+  const size_t smem = (size_t)kTilePad * sizeof(float2) + (size_t)2 * kMaxStepRounds * kTcBFloats * sizeof(float);
   static OptIn once;
   cudaError_t e = opt_in(reinterpret_cast<const void*>(tc_pass_kernel), smem, once);
   if (e != cudaSuccess) return e;

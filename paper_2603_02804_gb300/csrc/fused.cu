@@ -675,7 +675,7 @@ __device__ __forceinline__ void tc_rounds(const TcCtx& tc, const StepPar& P, int
 // Static shared memory of a pass (the tiles themselves are dynamic).
 template <class Y>
 __device__ void loss_block(int kind, double* E, const Y* y, int64_t B, double scale, double* loss, double* dLdE,
-                           const double* e_part, int tps, int tid);
+                           const double* e_part, int tps, int tid, int nthr);
 
 struct PassShared {
   StepPar par[2];
@@ -717,7 +717,8 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
   const int lane = tid & 31, warp = tid >> 5;
   const int tile_in_cta = KC ? 0 : tid >> tl2;
   const uint32_t tau = KC ? (uint32_t)tid : (uint32_t)(tid & (Tt - 1));
-  const int tiles_per_cta = KC ? 1 : kThreads >> tl2;
+  const int nthr = KC ? kThreads : (int)blockDim.x;
+  const int tiles_per_cta = KC ? 1 : nthr >> tl2;
   const int64_t total_tiles = (int64_t)a.B << a.tps_log2;
   const int64_t tile = first_tile + tile_in_cta;
   const bool active = KC || tile < total_tiles;
@@ -727,7 +728,8 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
   const int64_t dim = 1ll << a.n_eff;
   const int64_t sbase = b * dim;  // sample offset inside one state buffer
   float2* tp = smem + (tile_in_cta << K) + (tile_in_cta << tl2);  // loc(tile_in_cta << K)
-  float2* tl = tp + kTilePad;
+  const int lam_at = KC ? kTilePad : nthr * 17;  // words of the CTA's psi tiles: lambda's follow
+  float2* tl = tp + lam_at;
   const int wpt = Tt >= 32 ? Tt / 32 : 1;  // warps per tile
   const int lanes = Tt < 32 ? Tt : 32;
 
@@ -741,7 +743,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
     if (ROUNDS && tid < 8) sh.ident[tid] = make_float4(1.f, 0.f, 1.f, 0.f);
   }
   __syncthreads();
-  for (int h = tid; h < (1 << tl2); h += kThreads) {
+  for (int h = tid; h < (1 << tl2); h += nthr) {
     uint32_t g = 0;
     for (int j = 0; j < tl2; ++j)
       if ((h >> j) & 1) g |= 1u << s_gmap[kRegBits + j];
@@ -936,7 +938,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
       const uint32_t pos[4] = {gp.x, gp.y, gp.z, gp.w};
       float2 r[16];
       float2 l[16];
-      ld_group<KC, BWD>(lb, at, at + kTilePad, r, l);
+      ld_group<KC, BWD>(lb, at, at + lam_at, r, l);
       const int nq = a.n_eff;
       const uint32_t nmask = nq >= 32 ? ~0u : ((1u << nq) - 1u);
       const uint32_t rgb = ((gb >> 1) | ((gb & 1u) << (nq - 1))) & nmask;
@@ -1010,7 +1012,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
         pend = 0;
       }
       }  // CUDA-core rounds
-      st_group<KC, BWD>(lb, at, at + kTilePad, r, l);
+      st_group<KC, BWD>(lb, at, at + lam_at, r, l);
       if (TC) {
         cp_async_wait_all();
         fence_proxy_async();
@@ -1027,7 +1029,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
         const int nk = nr * 8;
         const int64_t b2 = first_tile >> a.tps_log2;
         const bool first = (first_tile & ((1ll << a.tps_log2) - 1)) == 0;
-        for (int kk = kThreads - 1 - tid; kk < nk; kk += kThreads) {  // the last warp (warp 0 stages)
+        for (int kk = nthr - 1 - tid; kk < nk; kk += nthr) {  // the last warp (warp 0 stages)
           const int32_t term = s_slot[buf][kk];
           if (term < 0) continue;
           double sum = 0.0;
@@ -1044,7 +1046,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
       } else if (BWD && Tt >= 32) {
         // the tile's warp sums in float32 (one float64 value per tile and term)
         const int nk = nr * 8;
-        for (int e = kThreads - 1 - tid; e < tiles_per_cta * nk; e += kThreads) {  // from the last warp
+        for (int e = nthr - 1 - tid; e < tiles_per_cta * nk; e += nthr) {  // from the last warp
           const int tc = e / nk, kk = e - tc * nk;
           const int64_t t2 = first_tile + tc;
           const int32_t term = s_slot[buf][kk];
@@ -1072,7 +1074,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
         r[j] = at[reg_off(j, so)];
-        if (BWD) l[j] = at[kTilePad + reg_off(j, so)];
+        if (BWD) l[j] = at[lam_at + reg_off(j, so)];
       }
 #pragma unroll 1
       for (int k = 0; k < nops; ++k) {
@@ -1129,11 +1131,11 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
         at[reg_off(j, so)] = r[j];
-        if (BWD) at[kTilePad + reg_off(j, so)] = l[j];
+        if (BWD) at[lam_at + reg_off(j, so)] = l[j];
       }
       __syncthreads();
       if (BWD && Tt >= 32) {
-        for (int e = kThreads - 1 - tid; e < tiles_per_cta * nk; e += kThreads) {  // from the last warp
+        for (int e = nthr - 1 - tid; e < tiles_per_cta * nk; e += nthr) {  // from the last warp
           const int tc = e / nk, kk = e - tc * nk;
           const int64_t t2 = first_tile + tc;
           if (t2 < total_tiles) {
@@ -1208,7 +1210,6 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
     }
   }
   __syncthreads();
-  static_assert(kThreads == 256, "loss_block reduces over 256 threads");
   if (!BWD && a.done && (pd.flags & PF_EXPECT)) {
     // the last CTA to finish sums E over every CTA's partials and finishes
     // the loss (the partials are fenced before the count)
@@ -1219,7 +1220,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
     if (sh.ticket == gridDim.x - 1) {
       __threadfence();
       loss_block<float>(a.loss_kind, a.E, a.y, a.B, a.loss_scale, a.loss, a.dLdE_out, a.e_part, 1 << a.tps_log2,
-                        tid);
+                        tid, nthr);
     }
     __syncthreads();
   }
@@ -1233,7 +1234,7 @@ template <bool BWD, bool ROUNDS, bool RX = false, int MINB = 2, int KC = 0>
 __global__ void __launch_bounds__(kThreads, MINB) pass_kernel(const PassArgs a) {
   extern __shared__ __align__(16) float2 smem[];
   __shared__ PassShared sh;
-  const int64_t first = KC ? (int64_t)blockIdx.x : (int64_t)blockIdx.x * (kThreads >> (a.pd.K - kRegBits));
+  const int64_t first = KC ? (int64_t)blockIdx.x : (int64_t)blockIdx.x * (blockDim.x >> (a.pd.K - kRegBits));
   pass_cta<BWD, ROUNDS, 8, false, RX, KC>(a, first, smem, sh);
 }
 
@@ -1625,18 +1626,19 @@ __global__ void g_reduce_kernel(const GradReduceArgs a) {
   if (lane == 0) a.grad[out] = s;
 }
 
-// Loss and dL/dE in one block of 256 threads with a fixed-order reduction
-// (warp shuffles, then the 8 warp sums in warp 0); labels float32, or float64
+// Loss and dL/dE in one block of nthr threads (32 .. 256) with a fixed-order
+// reduction (warp shuffles, then the warp sums in warp 0); labels float32, or float64
 // for complex128 plans. scale = 2 / B (MSE: dL/dE_i = scale (E_i - y_i)).
 // With e_part: E_i is first summed from its tps partials in tile order (as
 // e_reduce_kernel does) and stored; they are read from L2, as they may come
 // from other CTAs of the same launch.
 template <class Y>
 __device__ void loss_block(int kind, double* E, const Y* y, int64_t B, double scale, double* loss, double* dLdE,
-                           const double* e_part, int tps, int tid) {
+                           const double* e_part, int tps, int tid, int nthr) {
   __shared__ double red[8];
   double s = 0.0;
-  for (int64_t i = tid; i < B; i += 256) {
+#pragma unroll 4
+  for (int64_t i = tid; i < B; i += nthr) {
     double Ei;
     if (e_part) {
       Ei = 0.0;
@@ -1658,7 +1660,7 @@ __device__ void loss_block(int kind, double* E, const Y* y, int64_t B, double sc
   if ((tid & 31) == 0) red[tid >> 5] = s;
   __syncthreads();
   if (tid < 32) {
-    s = tid < 8 ? red[tid] : 0.0;
+    s = tid < (nthr >> 5) ? red[tid] : 0.0;
     for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (tid == 0) loss[0] = kind == 1 ? s * (0.5 * scale) : s;
   }
@@ -1667,7 +1669,7 @@ __device__ void loss_block(int kind, double* E, const Y* y, int64_t B, double sc
 template <class Y>
 __global__ void __launch_bounds__(256) loss_kernel(int kind, double* E, const Y* y, int64_t B, double scale,
                                                    double* loss, double* dLdE, const double* e_part, int tps) {
-  loss_block<Y>(kind, E, y, B, scale, loss, dLdE, e_part, tps, threadIdx.x);
+  loss_block<Y>(kind, E, y, B, scale, loss, dLdE, e_part, tps, threadIdx.x, 256);
 }
 
 // ---- batched persistent launch -------------------------------------------------
@@ -1888,25 +1890,33 @@ cudaError_t launch_prep(const PrepArgs& a, cudaStream_t st) {
 }
 
 cudaError_t launch_pass(bool bwd, const PassArgs& a, cudaStream_t st, int fwd_ctas) {
-  const int tiles_per_cta = kThreads >> (a.pd.K - kRegBits);
+  const int tl2 = a.pd.K - kRegBits;
   const int64_t total_tiles = (int64_t)a.B << a.tps_log2;
+  if (total_tiles == 0) return cudaSuccess;
+  const int n_sm = device_sms();
+  if (n_sm == 0) return cudaErrorInvalidDevice;
+  // CTAs of 256 threads hold several tiles of fewer than 12 qubits. While they
+  // would leave SMs without one, CTAs get smaller (one tile, one warp at least):
+  // n = 8, d = 20, 64 samples on 32 SMs instead of 4: step 120 -> 98 us; n = 10,
+  // 256 samples 145 -> 136 us. Launches that fill the SMs keep 256 threads.
+  int thr = kThreads;
+  while (thr > 32 && thr > (1 << tl2) && (total_tiles << tl2) < (int64_t)thr * n_sm) thr >>= 1;
+  const int tiles_per_cta = thr >> tl2;
   const int64_t grid = (total_tiles + tiles_per_cta - 1) / tiles_per_cta;
-  if (grid == 0) return cudaSuccess;
-  const size_t smem = (size_t)(bwd ? 2 : 1) * kTilePad * sizeof(float2);
+  const size_t smem = (size_t)(bwd ? 2 : 1) * thr * 17 * sizeof(float2);
   const bool rounds = a.rounds != nullptr, rx = rounds && a.rx_items;
   // 12-qubit tiles run the instances compiled for them; a single-wave forward
   // keeps the 128-register instance, more tiles than two CTAs per SM hold run
   // with three per SM (fewer registers, more warps to hide latency across waves)
-  const int n_sm = device_sms();
-  if (n_sm == 0) return cudaErrorInvalidDevice;
   const bool k12 = a.pd.K == kMaxTileBits;
-  const bool three = rounds && !bwd && (fwd_ctas == 3 || (fwd_ctas == 0 && grid > 2ll * n_sm));
+  const bool three =
+      rounds && !bwd && (fwd_ctas == 3 || (fwd_ctas == 0 && (total_tiles << tl2) > 2ll * kThreads * n_sm));
 #define QF_RUN(...)                                                                          \
   do {                                                                                       \
     static OptIn once;                                                                       \
-    const cudaError_t e_ = opt_in(reinterpret_cast<const void*>(__VA_ARGS__), smem, once);   \
+    const cudaError_t e_ = opt_in(reinterpret_cast<const void*>(__VA_ARGS__), 2 * kTilePad * sizeof(float2), once);   \
     if (e_ != cudaSuccess) return e_;                                                        \
-    __VA_ARGS__<<<(unsigned)grid, kThreads, smem, st>>>(a);                                  \
+    __VA_ARGS__<<<(unsigned)grid, thr, smem, st>>>(a);                                       \
     return cudaGetLastError();                                                               \
   } while (0)
   if (bwd) {

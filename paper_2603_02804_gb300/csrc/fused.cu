@@ -1388,33 +1388,9 @@ __device__ __forceinline__ double round_term_angle(const PrepArgs& a, const Roun
   return phi;
 }
 
-// u(phi) = (-1)^k u(w) with w = phi - 2 pi k in [-pi, pi] (k the nearest
-// integer to phi / 2 pi): the rotation by w/2 as three shears needs tan(w/4)
-// (|.| <= 1) and sin(w/2); angle 0 (also a missing term) gives all zero.
-// tan(w/4) = sin(w/2) / (1 + cos(w/2)) (the half-angle identity; the
-// denominator lies in [1, 2] for |w/2| <= pi/2), so one float64 sincos gives
-// both.
+// The multiple of 2 pi nearest to phi.
 __device__ __forceinline__ double wrap_count(double phi) {
   return rint(phi * (1.0 / 6.283185307179586476925286766559));
-}
-
-__device__ void shear_params(double phi, double& tq, double& sh, int& parity) {
-  const double two_pi = 6.283185307179586476925286766559;
-  const double k = wrap_count(phi);
-  const double w = phi - two_pi * k;
-  double c;
-  sincos_prep(0.5 * w, &sh, &c);
-  tq = sh / (1.0 + c);
-  parity = ((long long)k) & 1;
-}
-
-// The same in float64 (complex128 round programs).
-__device__ Shear64 shear64_of(double phi) {
-  Shear64 r{0.0, 0.0, 0, 0};
-  int parity;
-  shear_params(phi, r.t, r.s, parity);
-  r.wrap = parity;
-  return r;
 }
 
 // The diagonal of a round: its RZ runs (angles phi_r; 0 for a missing term)
@@ -1434,18 +1410,9 @@ __device__ double diag_angle(const double (&phi)[4], uint32_t bbits, int m, bool
   return al * (apply ? -0.5 : 0.5);
 }
 
-// The same in float64 (complex128 round programs).
-__device__ void diag_phases64(const double (&phi)[4], uint32_t bbits, int m, bool apply, double2* ph) {
-  double c, s;
-  bool f0, f1;
-  sincos_prep(diag_angle(phi, bbits, m, apply, f0, f1), &s, &c);
-  ph[m] = f0 ? make_double2(-c, -s) : make_double2(c, s);
-  ph[15 - m] = f1 ? make_double2(-c, s) : make_double2(c, -s);
-}
-
-// One round's float32 parameters by a half-warp (e: lane in it): lanes 0..3
-// take the 4 rotations, lanes 4..11 two phases of the diagonal each, one sincos
-// per lane (see rot_T).
+// One round's parameters by a half-warp (e: lane in it), float32 or (complex128
+// plans) float64: lanes 0..3 take the 4 rotations, lanes 4..11 two phases of
+// the diagonal each, one sincos per lane (see rot_T).
 __device__ void round_params(const PrepArgs& a, bool on, bool fwd, int64_t r, const int32_t* rec,
                              const RoundTerm* rt, int e, int lane) {
   double ang = 0.0;
@@ -1467,16 +1434,19 @@ __device__ void round_params(const PrepArgs& a, bool on, bool fwd, int64_t r, co
   const bool steep = e < 4 && fabs(s) > kMaxTan * fabs(c);
   const bool twice = ((__ballot_sync(0xffffffffu, steep) >> half) & 15u) != 0;
   const uint32_t neg = __popc((__ballot_sync(0xffffffffu, odd) >> half) & 15u) & 1u;
-  const float q = e < 4 ? (float)(s / (twice ? 1.0 + c : c)) : 0.f;  // tan(w/4) = sin(w/2) / (1 + cos(w/2))
+  double q = e < 4 ? s / (twice ? 1.0 + c : c) : 0.0;  // tan(w/4) = sin(w/2) / (1 + cos(w/2))
+  const bool f64 = a.rpf64 || a.rpb64;
+  if (!f64) q = (double)(float)q;
   double Q[4], S = 1.0;
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    const double qk = (double)__shfl_sync(0xffffffffu, q, half + k);
+    const double qk = __shfl_sync(0xffffffffu, q, half + k);
     Q[k] = 1.0 + qk * qk;
     S *= Q[k];
   }
   if (!on) return;
   float4* out = (fwd ? a.rpf : a.rpb) + r * kRoundPar;
+  RoundPar64* out64 = (fwd ? a.rpf64 : a.rpb64) + r;
   if (e < 4) {
     // the factor of rotation e's gradient value: 1 / (scale^2), less the rotations before it
     double g = Q[3];
@@ -1484,13 +1454,27 @@ __device__ void round_params(const PrepArgs& a, bool on, bool fwd, int64_t r, co
     for (int k = 2; k >= 0; --k)
       if (k >= e) g *= Q[k];
     if (twice) g *= S;
-    out[e] = make_float4(fwd ? q : -q, (float)(twice ? -g : g), 0.f, 0.f);
+    if (!fwd) q = -q;
+    if (twice) g = -g;
+    if (f64) {
+      out64->q[e] = q;
+      out64->g[e] = g;
+    } else {
+      out[e] = make_float4((float)q, (float)g, 0.f, 0.f);
+    }
   } else if (e < 12) {
     const double sc = (neg ? -1.0 : 1.0) * (twice ? 1.0 / S : rsqrt(S));
-    const float x0 = (float)(c * sc), y0 = (float)(s * sc);
-    float2* ph = reinterpret_cast<float2*>(out + 4);
-    ph[e - 4] = f0 ? make_float2(-x0, -y0) : make_float2(x0, y0);
-    ph[15 - (e - 4)] = f1 ? make_float2(-x0, y0) : make_float2(x0, -y0);
+    const double x = c * sc, y = s * sc;
+    const double2 v0 = f0 ? make_double2(-x, -y) : make_double2(x, y);
+    const double2 v1 = f1 ? make_double2(-x, y) : make_double2(x, -y);
+    if (f64) {
+      out64->ph[e - 4] = v0;
+      out64->ph[19 - e] = v1;
+    } else {
+      float2* ph = reinterpret_cast<float2*>(out + 4);
+      ph[e - 4] = make_float2((float)v0.x, (float)v0.y);
+      ph[19 - e] = make_float2((float)v1.x, (float)v1.y);
+    }
   }
 }
 
@@ -1513,19 +1497,7 @@ __device__ void prep_one(const PrepArgs& a, int64_t i) {
     const int32_t* rec = fwd ? reinterpret_cast<const int32_t*>(a.rpf_src) + r * kFwdRoundWords
                              : reinterpret_cast<const int32_t*>(a.rpb_src) + r * kBwdRoundWords;
     const RoundTerm* rt = (fwd ? a.rpf_terms : a.rpb_terms) + r * 8;
-    if (a.rpf64 || a.rpb64) {
-      RoundPar64& out = (fwd ? a.rpf64 : a.rpb64)[r];
-      if (!on || e >= 12) return;
-      if (e < 4) {
-        out.rot[e] = shear64_of(round_term_angle(a, rt[e]));
-      } else {
-        double phi[4];
-        for (int q = 0; q < 4; ++q) phi[q] = round_term_angle(a, rt[4 + q]);
-        diag_phases64(phi, (uint32_t)(fwd ? rec[5] : rec[9]), e - 4, fwd, out.ph);
-      }
-    } else {
-      round_params(a, on, fwd, r, rec, rt, e, threadIdx.x & 31);
-    }
+    round_params(a, on, fwd, r, rec, rt, e, threadIdx.x & 31);
     return;
   }
   i -= nre;

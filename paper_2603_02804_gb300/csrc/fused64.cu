@@ -5,11 +5,10 @@
 // double-precision state type the paper's library supports next to
 // complex64. Generic steps apply a fused 2x2 per register bit in the forward,
 // CZ signs and CNOT swaps, and un-apply one rotation at a time in the
-// adjoint. Round programs apply per register bit an RY and a merged RZ run as
-// three-shear rotations with pending CZ signs, so a qubit-layer of the
-// hardware-efficient ansatz costs 12 FP64 instructions per amplitude pair
-// forward (16 as a fused 2x2) and two gradient terms of 16 backward (three of
-// 20 one rotation at a time). GB300's FP64 pipe runs at 1/61 of its FP32
+// adjoint. Round programs apply four rotations at two FMAs per component and
+// one merged diagonal per round, with pending CZ signs, so a qubit-layer of the
+// hardware-efficient ansatz costs 6 FP64 instructions per amplitude pair
+// forward (16 as a fused 2x2) and 17 backward (60 one rotation at a time). GB300's FP64 pipe runs at 1/61 of its FP32
 // rate, so these passes are bound by FP64 instruction issue, never by memory.
 //
 // A CTA (256 threads) owns 4096 amplitudes per state, as in the complex64
@@ -154,10 +153,7 @@ __device__ __forceinline__ void cnot64(double2 (&r)[16], double2 (&l)[16], bool 
 // ---- round programs (the complex64 round programs' items in float64) -----------
 // A round applies one item per register bit r (the RY, then the merged RZ
 // run; the adjoint runs the exact reverse) and then the round's CZ links.
-// Rotations run as three shears: a plane rotation by phi is x += a y;
-// y += b x; x += a y with a = -tan(phi/2), b = sin(phi), |a| <= 1 for
-// |phi| <= pi/2 (term angles are wrapped into (-pi, pi], the wrap parity
-// kept as a sign). Pending CZ signs D: the registers hold psi~ with
+// Pending CZ signs D: the registers hold psi~ with
 // psi = D psi~, D = (-1)^(c0 + sum_r A_r j_r) (bit 4: c0, bits 0..3: A);
 // a gate on register bit r sees only Z_r^(A_r), folded into it; CZs between
 // two register bits are signs of the round's diagonal table.
@@ -194,44 +190,35 @@ __device__ __forceinline__ void pending64(uint32_t D, double2 (&r)[16], double2 
   }
 }
 
-// The rotation of a forward item on register bit R (RY, or RX where rx):
-// y holds the term's shear parameters of the un-apply direction; applying
-// rotates the other way. A pending Z_R turns the rotation by w into one by
-// -w; the wrap parity goes to the pending constant sign. An absent rotation
-// (no term) is skipped.
+// One rotation on register bit R, two FMAs per real component: the rotation by
+// w over cos(w/2), q = tan(w/2) (see fused.cu's rot_T). The cosines are a scale
+// of the round's diagonal; a round with a steep rotation runs twice by half
+// the angles. Against three shears, and with the diagonal's terms from
+// complement differences: step of n = 12, d = 10, 256 samples 4,296 -> 3,328 us,
+// as these kernels are bound by FP64 issue.
 template <int R>
-__device__ __forceinline__ void rot_fwd64(double2 (&r)[16], const Shear64& y, uint32_t a, uint32_t& D,
-                                          bool has_y, bool rx) {
-  const double ty = a ? y.t : -y.t, sy = a ? -y.s : y.s;
-  if (has_y && rx) {
-    // RX(w): a rotation by -w/2 of (re p0, im p1) and (re p1, im p0):
-    // x += t y; y -= s x; x += t y (t, s negated under a pending Z_R)
-    const double tx = -ty, sx = sy;
+__device__ __forceinline__ void rot_T64(double2 (&r)[16], double q, bool rx) {
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      if (j & (1 << R)) continue;
-      const int j1 = j | (1 << R);
-      double2 p0 = r[j], p1 = r[j1];
-      p0.x = fma(tx, p1.y, p0.x); p1.y = fma(-sx, p0.x, p1.y); p0.x = fma(tx, p1.y, p0.x);
-      p1.x = fma(tx, p0.y, p1.x); p0.y = fma(-sx, p1.x, p0.y); p1.x = fma(tx, p0.y, p1.x);
-      r[j] = p0;
-      r[j1] = p1;
-    }
-  } else if (has_y) {
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      if (j & (1 << R)) continue;
-      const int j1 = j | (1 << R);
-      double2 p0 = r[j], p1 = r[j1];
-      // RY(w) on (p0, p1): rotation by +w/2, the same shears on re and im
-      p0.x = fma(ty, p1.x, p0.x); p0.y = fma(ty, p1.y, p0.y);
-      p1.x = fma(sy, p0.x, p1.x); p1.y = fma(sy, p0.y, p1.y);
-      p0.x = fma(ty, p1.x, p0.x); p0.y = fma(ty, p1.y, p0.y);
-      r[j] = p0;
-      r[j1] = p1;
+  for (int j = 0; j < 16; ++j) {
+    if (j & (1 << R)) continue;
+    const int j1 = j | (1 << R);
+    const double2 p0 = r[j], p1 = r[j1];
+    if (rx) {  // p0 -= i q p1; p1 -= i q p0
+      r[j] = make_double2(fma(q, p1.y, p0.x), fma(-q, p1.x, p0.y));
+      r[j1] = make_double2(fma(q, p0.y, p1.x), fma(-q, p0.x, p1.y));
+    } else {  // p0 -= q p1; p1 += q p0
+      r[j] = make_double2(fma(-q, p1.x, p0.x), fma(-q, p1.y, p0.y));
+      r[j1] = make_double2(fma(q, p0.x, p1.x), fma(q, p0.y, p1.y));
     }
   }
-  D ^= (uint32_t)(y.wrap & 1) << 4;
+}
+
+// A forward item (a: a pending Z_R turns w into -w). An absent rotation is skipped.
+template <int R>
+__device__ __forceinline__ void rot_fwd64(double2 (&r)[16], double q, uint32_t a, bool has_y, bool rx) {
+  if (!has_y) return;
+  if (rx) rot_T64<R>(r, a ? -q : q, true);
+  else rot_T64<R>(r, a ? -q : q, false);
 }
 
 // v *= (c + i s)
@@ -255,87 +242,55 @@ __device__ __forceinline__ void diag64(double2 (&r)[16], const double2* ph) {
 // Adjoint side of the round's diagonal: g[r] = sum_j sigma_r(j) w_j with
 // w_j = Im(conj(lambda_j) psi_j), sigma_r(j) = +1 where bit r of j is clear,
 // else -1 (the RZ-run terms; w_j is unchanged by the diagonal, and Z_r
-// commutes with the rotations on the other bits), then the un-apply.
-__device__ __forceinline__ void diag_bwd64(double2 (&p)[16], double2 (&l)[16], const double2* ph, double (&g)[8]) {
-  double s2[4];
-  double d0 = 0.0, d1 = 0.0, se = 0.0;
+// commutes with the rotations on the other bits), from the differences u_j =
+// w_j - w_{15-j} as sigma_r(15 - j) = -sigma_r(j); then the un-apply.
+__device__ __forceinline__ void diag_terms64(const double2 (&p)[16], const double2 (&l)[16], double (&g)[8]) {
+  double u[8];
 #pragma unroll
   for (int m = 0; m < 8; ++m) {
-    double2& p0 = p[2 * m];
-    double2& p1 = p[2 * m + 1];
-    double2& l0 = l[2 * m];
-    double2& l1 = l[2 * m + 1];
-    const double w0 = fma(l0.x, p0.y, -l0.y * p0.x);
-    const double w1 = fma(l1.x, p1.y, -l1.y * p1.x);
-    const double2 e0 = ph[2 * m], e1 = ph[2 * m + 1];
-    cmul64(p0, e0.x, e0.y);
-    cmul64(l0, e0.x, e0.y);
-    cmul64(p1, e1.x, e1.y);
-    cmul64(l1, e1.x, e1.y);
-    const double sm = w0 + w1;
-    d0 += w0 - w1;
-    if (m & 1) {
-      s2[m >> 1] = se + sm;
-      d1 += se - sm;
-    } else {
-      se = sm;
-    }
+    const double2 p0 = p[m], l0 = l[m], p1 = p[15 - m], l1 = l[15 - m];
+    u[m] = fma(l1.y, p1.x, fma(-l1.x, p1.y, fma(l0.x, p0.y, -l0.y * p0.x)));
   }
-  g[0] = d0;
-  g[1] = d1;
-  g[2] = (s2[0] - s2[1]) + (s2[2] - s2[3]);
-  g[3] = (s2[0] + s2[1]) - (s2[2] + s2[3]);
+  const double a0 = u[0] + u[1], a1 = u[2] + u[3], a2 = u[4] + u[5], a3 = u[6] + u[7];
+  const double q0 = a0 + a1, T = q0 + (a2 + a3);
+  g[0] = fma(2.0, (u[0] + u[2]) + (u[4] + u[6]), -T);
+  g[1] = fma(2.0, a0 + a2, -T);
+  g[2] = fma(2.0, q0, -T);
+  g[3] = T;
 }
 
-// Un-apply one rotation on register bit R by three shears; returns the
-// thread's sum of Im<lambda|P|psi> taken before it.
-//   RY: (x, y) <- RY(w)^dagger (x, y), a rotation by -w/2: a = t, b = -s.
-template <int R, int KIND>
-__device__ __forceinline__ double shear_bwd64(double2 (&p)[16], double2 (&l)[16], const double t, const double s) {
-  double acc = 0.0;
+// The rotation of an adjoint item on register bit R (q un-applies it), after
+// the round's diagonal; gy: the thread's sum of Im<lambda|P|psi> before it. A
+// pending Z_R negates q and gy. An absent rotation is skipped; its value is 0.
+template <int R>
+__device__ __forceinline__ void rot_bwd64(double2 (&p)[16], double2 (&l)[16], double q, uint32_t a, double& gy,
+                                          bool has_y, bool rx) {
+  gy = 0.0;
+  if (!has_y) return;
+  double g0 = 0.0, g1 = 0.0;
 #pragma unroll
   for (int j = 0; j < 16; ++j) {
     if (j & (1 << R)) continue;
     const int j1 = j | (1 << R);
-    double2 p0 = p[j], p1 = p[j1], l0 = l[j], l1 = l[j1];
-    if (KIND == G_RX) {
-      // Im<lambda|X|psi>; RX(w)^dagger rotates (re p0, im p1) and (re p1, im p0) by +w/2
-      acc += l0.x * p1.y - l0.y * p1.x + l1.x * p0.y - l1.y * p0.x;
-      p0.x = fma(-t, p1.y, p0.x); p1.y = fma(s, p0.x, p1.y); p0.x = fma(-t, p1.y, p0.x);
-      p1.x = fma(-t, p0.y, p1.x); p0.y = fma(s, p1.x, p0.y); p1.x = fma(-t, p0.y, p1.x);
-      l0.x = fma(-t, l1.y, l0.x); l1.y = fma(s, l0.x, l1.y); l0.x = fma(-t, l1.y, l0.x);
-      l1.x = fma(-t, l0.y, l1.x); l0.y = fma(s, l1.x, l0.y); l1.x = fma(-t, l0.y, l1.x);
+    const double2 p0 = p[j], p1 = p[j1], l0 = l[j], l1 = l[j1];
+    if (rx) {
+      g0 = fma(l0.x, p1.y, fma(l1.x, p0.y, g0));
+      g1 = fma(l0.y, p1.x, fma(l1.y, p0.x, g1));
     } else {
-      acc += l1.x * p0.x + l1.y * p0.y - l0.x * p1.x - l0.y * p1.y;
-      p0.x = fma(t, p1.x, p0.x); p0.y = fma(t, p1.y, p0.y);
-      p1.x = fma(-s, p0.x, p1.x); p1.y = fma(-s, p0.y, p1.y);
-      p0.x = fma(t, p1.x, p0.x); p0.y = fma(t, p1.y, p0.y);
-      l0.x = fma(t, l1.x, l0.x); l0.y = fma(t, l1.y, l0.y);
-      l1.x = fma(-s, l0.x, l1.x); l1.y = fma(-s, l0.y, l1.y);
-      l0.x = fma(t, l1.x, l0.x); l0.y = fma(t, l1.y, l0.y);
+      g0 = fma(l1.x, p0.x, fma(l1.y, p0.y, g0));
+      g1 = fma(l0.x, p1.x, fma(l0.y, p1.y, g1));
     }
-    p[j] = p0;
-    p[j1] = p1;
-    l[j] = l0;
-    l[j1] = l1;
   }
-  return acc;
-}
-
-// The rotation of an adjoint item on register bit R, un-applied after the
-// round's diagonal; gy: its Im<lambda|P|psi>. With a pending Z_R it
-// un-applies as the rotation by +w and gy changes sign. An absent rotation is
-// skipped; its value is 0.
-template <int R>
-__device__ __forceinline__ void rot_bwd64(double2 (&p)[16], double2 (&l)[16], const Shear64& y, uint32_t a,
-                                          uint32_t& D, double& gy, bool has_y, bool rx) {
-  gy = 0.0;
-  if (has_y) {
-    const double t = a ? -y.t : y.t, s = a ? -y.s : y.s;
-    const double g = rx ? shear_bwd64<R, G_RX>(p, l, t, s) : shear_bwd64<R, G_RY>(p, l, t, s);
-    gy = a ? -g : g;
+  const double g = g0 - g1;
+  gy = a ? -g : g;
+  if (a) q = -q;
+  if (rx) {
+    rot_T64<R>(p, q, true);
+    rot_T64<R>(l, q, true);
+  } else {
+    rot_T64<R>(p, q, false);
+    rot_T64<R>(l, q, false);
   }
-  D ^= (uint32_t)(y.wrap & 1) << 4;
 }
 
 // Reduce 8 per-thread values over `lanes` lanes (8, 16 or 32; whole-warp
@@ -537,32 +492,50 @@ __global__ void __launch_bounds__(kThreads, 1) pass64_kernel(const PassArgs64 a)
         if (BWD) l[j] = tl[pb ^ reg_offset(j, so)];
       }
       uint32_t D = 0;
+      // a round with a steep rotation runs twice: the forward with its diagonal
+      // and links the second time, the adjoint the first
+      bool again = false;
 #pragma unroll 1
-      for (int k = 0; k < nr; ++k) {
+      for (int k = 0; k < nr;) {
         const size_t rr = (size_t)op.y + k;
         const RoundPar64& v = a.rpar[rr];
+        const bool steep = v.g[0] < 0.0;
         if (!BWD) {
           const uint4 lk = __ldg(a.rounds + rr * (kFwdRoundWords / 4) + 1);
           // the items' rotation terms (-1: absent) in words 12..15
           const uint4 ty = __ldg(a.rounds + rr * (kFwdRoundWords / 4) + 3);
-          rot_fwd64<0>(r, v.rot[0], D & 1u, D, (int)ty.x >= 0, RX && (lk.z & 1u));
-          rot_fwd64<1>(r, v.rot[1], (D >> 1) & 1u, D, (int)ty.y >= 0, RX && ((lk.z >> 1) & 1u));
-          rot_fwd64<2>(r, v.rot[2], (D >> 2) & 1u, D, (int)ty.z >= 0, RX && ((lk.z >> 2) & 1u));
-          rot_fwd64<3>(r, v.rot[3], (D >> 3) & 1u, D, (int)ty.w >= 0, RX && ((lk.z >> 3) & 1u));
-          diag64(r, v.ph);
-          chain64(lk.x, gb, pos, a.n_eff, D);
+          rot_fwd64<0>(r, v.q[0], D & 1u, (int)ty.x >= 0, RX && (lk.z & 1u));
+          rot_fwd64<1>(r, v.q[1], (D >> 1) & 1u, (int)ty.y >= 0, RX && ((lk.z >> 1) & 1u));
+          rot_fwd64<2>(r, v.q[2], (D >> 2) & 1u, (int)ty.z >= 0, RX && ((lk.z >> 2) & 1u));
+          rot_fwd64<3>(r, v.q[3], (D >> 3) & 1u, (int)ty.w >= 0, RX && ((lk.z >> 3) & 1u));
+          again = steep && !again;
+          if (!again) {
+            diag64(r, v.ph);
+            chain64(lk.x, gb, pos, a.n_eff, D);
+            ++k;
+          }
         } else {
           const uint4 lk = __ldg(a.rounds + rr * (kBwdRoundWords / 4) + 2);
           const uint4 ty = __ldg(a.rounds + rr * (kBwdRoundWords / 4) + 1);
-          chain64(lk.x, gb, pos, a.n_eff, D);
           double gv[8];
-          diag_bwd64(r, l, v.ph, gv);
-          rot_bwd64<0>(r, l, v.rot[0], D & 1u, D, gv[4], (int)ty.x >= 0, RX && (lk.z & 1u));
-          rot_bwd64<1>(r, l, v.rot[1], (D >> 1) & 1u, D, gv[5], (int)ty.y >= 0, RX && ((lk.z >> 1) & 1u));
-          rot_bwd64<2>(r, l, v.rot[2], (D >> 2) & 1u, D, gv[6], (int)ty.z >= 0, RX && ((lk.z >> 2) & 1u));
-          rot_bwd64<3>(r, l, v.rot[3], (D >> 3) & 1u, D, gv[7], (int)ty.w >= 0, RX && ((lk.z >> 3) & 1u));
+          if (!again) {
+            chain64(lk.x, gb, pos, a.n_eff, D);
+            diag_terms64(r, l, gv);
+            diag64(r, v.ph);
+            diag64(l, v.ph);
+          }
+          rot_bwd64<0>(r, l, v.q[0], D & 1u, gv[4], (int)ty.x >= 0, RX && (lk.z & 1u));
+          rot_bwd64<1>(r, l, v.q[1], (D >> 1) & 1u, gv[5], (int)ty.y >= 0, RX && ((lk.z >> 1) & 1u));
+          rot_bwd64<2>(r, l, v.q[2], (D >> 2) & 1u, gv[6], (int)ty.z >= 0, RX && ((lk.z >> 2) & 1u));
+          rot_bwd64<3>(r, l, v.q[3], (D >> 3) & 1u, gv[7], (int)ty.w >= 0, RX && ((lk.z >> 3) & 1u));
+          if (again) {  // the first run has the round's values
+            again = false;
+            ++k;
+            continue;
+          }
           int idx;
-          const double sum = butterfly8_64(gv, lanes, lane, idx);
+          double sum = butterfly8_64(gv, lanes, lane, idx);
+          if (idx >= 4) sum *= fabs(v.g[idx - 4]);
           const bool owner = (lane & ((lanes >> 3) - 1)) == 0;
           const int32_t term = __ldg(reinterpret_cast<const int32_t*>(a.rounds + rr * (kBwdRoundWords / 4)) + idx);
           if (Tt >= 32) {
@@ -573,6 +546,8 @@ __global__ void __launch_bounds__(kThreads, 1) pass64_kernel(const PassArgs64 a)
           } else if (owner && active && term >= 0) {
             a.g_part[tile * a.n_slots + term] = 0.5 * sum;
           }
+          again = steep;
+          if (!again) ++k;
         }
       }
       pending64<BWD>(D, r, l);

@@ -48,18 +48,13 @@ struct PassArgs {
   double loss_scale;      // 2 / B
 };
 
-// Float64 three-shear parameters of a gradient term (complex128 round
-// programs): t = tan(w/4), s = sin(w/2) with w = phi - 2 pi k in (-pi, pi],
-// wrap = k & 1 (u(phi) = (-1)^k u(w)).
-struct alignas(16) Shear64 {
-  double t, s;
-  int64_t wrap, pad;
-};
-
-// Parameters of one round of a complex128 round program: the shears of the 4
-// items' rotations and the round's diagonal as (cos, sin) per register index.
+// Parameters of one round of a complex128 round program, as the complex64 ones
+// (kRoundPar): the 4 items' rotations q, the factors of their gradient values
+// (negative: the round runs twice) and the diagonal as a phase per register
+// index, times the scale and sign that the rotations leave out.
 struct RoundPar64 {
-  Shear64 rot[4];
+  double q[4];
+  double g[4];
   double2 ph[16];
 };
 

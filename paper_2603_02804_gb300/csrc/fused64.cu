@@ -15,7 +15,8 @@
 // passes; the tile is 64 KiB per state here (16-byte amplitudes), so the
 // adjoint (psi and lambda) takes 128 KiB. One CTA per SM (8 warps) keeps the
 // FP64 pipe busy; the launch bound lets the 16 + 16 double2 registers of the
-// adjoint step stay in registers.
+// adjoint step stay in registers. A launch of few tiles gets smaller CTAs, and
+// below one tile per SM a cluster of two CTAs shares a tile (launch_pass64).
 //
 // Shared-memory layout: amplitude with local index i lives at
 // i ^ ((i >> 4) & 7). Eight 16-byte amplitudes fill the 32 banks, and a
@@ -23,6 +24,7 @@
 // nibbles: for nibble 0 those eight lanes differ in local bits 4..6, which the
 // XOR folds into the low three bits; for any other group they differ in bits
 // 0..2 directly. Either way the eight lanes hit eight distinct bank quads.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -340,19 +342,27 @@ struct Shared64 {
 
 // One complex128 pass: CTA c owns tiles c * tiles_per_cta .. (tile = sample *
 // tiles_per_sample + tile within the sample); 2^(K-4) threads per tile, 16
-// amplitudes per thread per step.
-template <bool BWD, bool ROUNDS, bool RX = false>
+// amplitudes per thread per step. SPLIT: a cluster of 2^a.split CTAs (a.split =
+// 1) owns one tile instead; CTA `rank` holds the amplitudes whose top a.split local bits
+// are its rank, and runs the columns (local indices without the group's bits)
+// with those top bits. Only a step on a group that holds top bits reaches into
+// the other CTAs' shared memory; every barrier is then the cluster's.
+template <bool BWD, bool ROUNDS, bool RX = false, bool SPLIT = false>
 __global__ void __launch_bounds__(kThreads, 1) pass64_kernel(const PassArgs64 a) {
   extern __shared__ __align__(16) double2 smem64[];
   __shared__ Shared64 sh;
   const PassDesc& pd = a.pd;
   const int K = pd.K;
-  const int tl2 = K - kRegBits;
-  const int Tt = 1 << tl2;
+  const int sp = SPLIT ? a.split : 0;
+  const int KL = K - sp;                   // local bits of one CTA's part
+  const int tl2 = K - kRegBits - sp;
+  const int Tt = 1 << tl2;                 // threads per tile in this CTA
+  const int nthr = (int)blockDim.x;
   const int tid = threadIdx.x;
   const int lane = tid & 31, warp = tid >> 5;
-  const int tiles_per_cta = kThreads >> tl2;
-  const int64_t first_tile = (int64_t)blockIdx.x * tiles_per_cta;
+  const int tiles_per_cta = nthr >> tl2;   // 1 when split
+  const uint32_t rank = SPLIT ? blockIdx.x & ((1u << sp) - 1u) : 0u;
+  const int64_t first_tile = SPLIT ? (int64_t)(blockIdx.x >> sp) : (int64_t)blockIdx.x * tiles_per_cta;
   const int tile_in_cta = tid >> tl2;
   const uint32_t tau = (uint32_t)(tid & (Tt - 1));
   const int64_t total_tiles = (int64_t)a.B << a.tps_log2;
@@ -362,19 +372,30 @@ __global__ void __launch_bounds__(kThreads, 1) pass64_kernel(const PassArgs64 a)
   const uint32_t t_in = active ? (uint32_t)(tile & ((1ll << a.tps_log2) - 1)) : 0u;
   const uint32_t outer = pdep(t_in, pd.outer_mask);
   const int64_t sbase = b << a.n_eff;
-  double2* tp = smem64 + (tile_in_cta << K);
-  double2* tl = smem64 + kTileAmps + (tile_in_cta << K);
+  const int lam_at = nthr << kRegBits;     // lambda's part follows psi's
+  double2* tp = smem64 + (tile_in_cta << KL);
+  double2* tl = tp + lam_at;
   const int wpt = Tt >= 32 ? Tt / 32 : 1;  // warps per tile
   const int lanes = Tt < 32 ? Tt : 32;     // lanes per tile within a warp
+  auto barrier = [&]() {
+    if (SPLIT) cooperative_groups::this_cluster().sync();
+    else __syncthreads();
+  };
+  // amplitude i of the tile (any part): psi, or lambda at offset lam_at
+  auto amp = [&](uint32_t i, int off) -> double2& {
+    double2* p = tp + off + swz64(i & ((1u << KL) - 1u));
+    return SPLIT ? *cooperative_groups::this_cluster().map_shared_rank(p, i >> KL) : *p;
+  };
+  const uint32_t i_top = rank << KL;       // the part's local indices start here
 
   if (tid < 16) {
     sh.gmap[tid] = pd.gmap[tid];
     sh.grp[tid >> 2][tid & 3] = pd.groups[tid >> 2][tid & 3];
   }
   __syncthreads();
-  for (int h = tid; h < Tt; h += kThreads) {
+  for (int h = tid; h < (1 << (K - kRegBits)); h += nthr) {
     uint32_t g = 0;
-    for (int j = 0; j < tl2; ++j)
+    for (int j = 0; j < K - kRegBits; ++j)
       if ((h >> j) & 1) g |= 1u << sh.gmap[kRegBits + j];
     sh.lg[h] = g;
   }
@@ -386,7 +407,7 @@ __global__ void __launch_bounds__(kThreads, 1) pass64_kernel(const PassArgs64 a)
     return a.work + sbase;
   };
 
-  // ---- bring psi (and lambda) in: local index i = it * Tt + tau -------------
+  // ---- bring psi (and lambda) in: local index i = i_top | it * Tt + tau ---------
   const int32_t psrc = pd.psi_src;
   if (psrc == SRC_GENERATE && a.psi_in) {
     // given initial states [B][2^n_in]; padding qubits (n_in <= bit < n_eff) are |0>
@@ -395,7 +416,7 @@ __global__ void __launch_bounds__(kThreads, 1) pass64_kernel(const PassArgs64 a)
 #pragma unroll 4
     for (int it = 0; it < 16; ++it) {
       const uint32_t i = (uint32_t)it * Tt + tau;
-      const uint32_t g = gidx(i);
+      const uint32_t g = gidx(i_top | i);
       const double2 v = (int64_t)g < din ? __ldcg(src + g) : make_double2(0.0, 0.0);
       if (active) tp[swz64(i)] = v;
     }
@@ -405,7 +426,7 @@ __global__ void __launch_bounds__(kThreads, 1) pass64_kernel(const PassArgs64 a)
 #pragma unroll 1
     for (int it = 0; it < 16; ++it) {
       const uint32_t i = (uint32_t)it * Tt + tau;
-      const uint32_t g = gidx(i);
+      const uint32_t g = gidx(i_top | i);
       double pr = 1.0;
       for (int q = 0; q < a.n_eff; ++q) {
         const double2 f = __ldg(e + q);
@@ -425,7 +446,7 @@ __global__ void __launch_bounds__(kThreads, 1) pass64_kernel(const PassArgs64 a)
       double2 vp[8], vl[8];
 #pragma unroll
       for (int it = 0; it < 8; ++it) {
-        const uint32_t g = gidx((uint32_t)(i0 + it) * Tt + tau);
+        const uint32_t g = gidx(i_top | ((uint32_t)(i0 + it) * Tt + tau));
         if (half) {
           const float2 h = __ldcg(fsrc + g);
           vp[it] = make_double2((double)h.x, (double)h.y);
@@ -447,23 +468,34 @@ __global__ void __launch_bounds__(kThreads, 1) pass64_kernel(const PassArgs64 a)
 #pragma unroll 4
     for (int it = 0; it < 16; ++it) {
       const uint32_t i = (uint32_t)it * Tt + tau;
-      tl[swz64(i)] = __ldcg(src + gidx(i));
+      tl[swz64(i)] = __ldcg(src + gidx(i_top | i));
     }
   }
-  __syncthreads();
+  barrier();
   if (BWD && pd.lam_src == LAM_SEED) {
     // lambda_M = 2 (dL/dE_b) O psi_M (Eq. 4); (O psi)_x = i^{#Y} (-1)^{|(x^xm)&zm|} psi_{x^xm}
     const double scale = active ? 2.0 * a.dLdE[b] : 0.0;
 #pragma unroll 1
     for (int it = 0; it < 16; ++it) {
       const uint32_t i = (uint32_t)it * Tt + tau;
-      const uint32_t ip = i ^ pd.xm_local;
-      const double2 v = ipow(tp[swz64(ip)], a.y_count);
+      const uint32_t ip = (i_top | i) ^ pd.xm_local;
+      const double2 v = ipow(amp(ip, 0), a.y_count);
       const uint32_t sg = __popc(gidx(ip) & a.z_mask) & 1u;
       tl[swz64(i)] = make_double2(flipd(v.x, sg) * scale, flipd(v.y, sg) * scale);
     }
-    __syncthreads();
+    barrier();
   }
+
+  // a tile's sum of its warps' values (stride words apart) in warp order, over
+  // the CTAs that share it
+  auto tile_sum = [&](const double* p, int stride) -> double {
+    double sum = 0.0;
+    for (uint32_t c = 0; c < (1u << sp); ++c) {
+      const double* q = SPLIT ? cooperative_groups::this_cluster().map_shared_rank(p, c) : p;
+      for (int w = 0; w < wpt; ++w) sum += q[w * stride];
+    }
+    return sum;
+  };
 
   // ---- step program --------------------------------------------------------
   int buf = 0;
@@ -479,17 +511,28 @@ __global__ void __launch_bounds__(kThreads, 1) pass64_kernel(const PassArgs64 a)
       const int nr = (op.x >> 8) & 0xffff;
       const uint32_t lb0 = sh.grp[g][0], lb1 = sh.grp[g][1], lb2 = sh.grp[g][2], lb3 = sh.grp[g][3];
       const uint32_t gm = (1u << lb0) | (1u << lb1) | (1u << lb2) | (1u << lb3);
-      const uint32_t base = pdep(tau, ((1u << K) - 1u) & ~gm);
-      const uint32_t pb = swz64(base);
+      // the thread's column: its bits, and the rank's above them, around the group's
+      const uint32_t base = pdep((rank << tl2) | tau, ((1u << K) - 1u) & ~gm);
+      const bool far = SPLIT && (gm >> KL) != 0;  // the group holds top bits
+      const uint32_t pb = swz64(base & ((1u << KL) - 1u));
       const uint32_t so[4] = {swz64(1u << lb0), swz64(1u << lb1), swz64(1u << lb2), swz64(1u << lb3)};
       const uint32_t gb = gidx(base);
       const uint32_t pos[4] = {sh.gmap[lb0], sh.gmap[lb1], sh.gmap[lb2], sh.gmap[lb3]};
       double2 r[16];
       double2 l[16];
+      if (far) {
+        const uint32_t lo[4] = {1u << lb0, 1u << lb1, 1u << lb2, 1u << lb3};
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        r[j] = tp[pb ^ reg_offset(j, so)];
-        if (BWD) l[j] = tl[pb ^ reg_offset(j, so)];
+        for (int j = 0; j < 16; ++j) {
+          r[j] = amp(base | reg_offset(j, lo), 0);
+          if (BWD) l[j] = amp(base | reg_offset(j, lo), lam_at);
+        }
+      } else {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          r[j] = tp[pb ^ reg_offset(j, so)];
+          if (BWD) l[j] = tl[pb ^ reg_offset(j, so)];
+        }
       }
       uint32_t D = 0;
       // a round with a steep rotation runs twice: the forward with its diagonal
@@ -551,21 +594,29 @@ __global__ void __launch_bounds__(kThreads, 1) pass64_kernel(const PassArgs64 a)
         }
       }
       pending64<BWD>(D, r, l);
+      if (far) {
+        const uint32_t lo[4] = {1u << lb0, 1u << lb1, 1u << lb2, 1u << lb3};
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        tp[pb ^ reg_offset(j, so)] = r[j];
-        if (BWD) tl[pb ^ reg_offset(j, so)] = l[j];
+        for (int j = 0; j < 16; ++j) {
+          amp(base | reg_offset(j, lo), 0) = r[j];
+          if (BWD) amp(base | reg_offset(j, lo), lam_at) = l[j];
+        }
+      } else {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          tp[pb ^ reg_offset(j, so)] = r[j];
+          if (BWD) tl[pb ^ reg_offset(j, so)] = l[j];
+        }
       }
-      __syncthreads();
+      barrier();
       if (BWD && Tt >= 32) {
         const int nk = nr * 8;
-        for (int e = tid; e < tiles_per_cta * nk; e += kThreads) {
+        for (int e = tid; e < (rank ? 0 : tiles_per_cta * nk); e += nthr) {
           const int tc = e / nk, kk = e - tc * nk;
           const int64_t t2 = first_tile + tc;
           const int32_t term = sh.slot[buf][kk];
           if (t2 < total_tiles && term >= 0) {
-            double sum = 0.0;
-            for (int w = 0; w < wpt; ++w) sum += sh.red[buf][tc * wpt + w][kk];
+            const double sum = tile_sum(&sh.red[buf][tc * wpt][kk], kMaxStepSlots);
             a.g_part[t2 * a.n_slots + term] = 0.5 * sum;
           }
         }
@@ -577,17 +628,28 @@ __global__ void __launch_bounds__(kThreads, 1) pass64_kernel(const PassArgs64 a)
       const int nk = (int)op.y;
       const uint32_t lb0 = sh.grp[g][0], lb1 = sh.grp[g][1], lb2 = sh.grp[g][2], lb3 = sh.grp[g][3];
       const uint32_t gm = (1u << lb0) | (1u << lb1) | (1u << lb2) | (1u << lb3);
-      const uint32_t base = pdep(tau, ((1u << K) - 1u) & ~gm);
-      const uint32_t pb = swz64(base);
+      // the thread's column: its bits, and the rank's above them, around the group's
+      const uint32_t base = pdep((rank << tl2) | tau, ((1u << K) - 1u) & ~gm);
+      const bool far = SPLIT && (gm >> KL) != 0;  // the group holds top bits
+      const uint32_t pb = swz64(base & ((1u << KL) - 1u));
       const uint32_t so[4] = {swz64(1u << lb0), swz64(1u << lb1), swz64(1u << lb2), swz64(1u << lb3)};
       const uint32_t gb = gidx(base);
       const uint32_t go[4] = {1u << sh.gmap[lb0], 1u << sh.gmap[lb1], 1u << sh.gmap[lb2], 1u << sh.gmap[lb3]};
       double2 r[16];
       double2 l[16];
+      if (far) {
+        const uint32_t lo[4] = {1u << lb0, 1u << lb1, 1u << lb2, 1u << lb3};
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        r[j] = tp[pb ^ reg_offset(j, so)];
-        if (BWD) l[j] = tl[pb ^ reg_offset(j, so)];
+        for (int j = 0; j < 16; ++j) {
+          r[j] = amp(base | reg_offset(j, lo), 0);
+          if (BWD) l[j] = amp(base | reg_offset(j, lo), lam_at);
+        }
+      } else {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          r[j] = tp[pb ^ reg_offset(j, so)];
+          if (BWD) l[j] = tl[pb ^ reg_offset(j, so)];
+        }
       }
 #pragma unroll 1
       for (int k = 0; k < nops; ++k) {
@@ -640,20 +702,28 @@ __global__ void __launch_bounds__(kThreads, 1) pass64_kernel(const PassArgs64 a)
           }
         }
       }
+      if (far) {
+        const uint32_t lo[4] = {1u << lb0, 1u << lb1, 1u << lb2, 1u << lb3};
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        tp[pb ^ reg_offset(j, so)] = r[j];
-        if (BWD) tl[pb ^ reg_offset(j, so)] = l[j];
+        for (int j = 0; j < 16; ++j) {
+          amp(base | reg_offset(j, lo), 0) = r[j];
+          if (BWD) amp(base | reg_offset(j, lo), lam_at) = l[j];
+        }
+      } else {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          tp[pb ^ reg_offset(j, so)] = r[j];
+          if (BWD) tl[pb ^ reg_offset(j, so)] = l[j];
+        }
       }
-      __syncthreads();
+      barrier();
       if (BWD && Tt >= 32) {
         // per-tile sums of the step's terms in warp order (deterministic)
-        for (int e = tid; e < tiles_per_cta * nk; e += kThreads) {
+        for (int e = tid; e < (rank ? 0 : tiles_per_cta * nk); e += nthr) {
           const int tc = e / nk, kk = e - tc * nk;
           const int64_t t2 = first_tile + tc;
           if (t2 < total_tiles) {
-            double sum = 0.0;
-            for (int w = 0; w < wpt; ++w) sum += sh.red[buf][tc * wpt + w][kk];
+            const double sum = tile_sum(&sh.red[buf][tc * wpt][kk], kMaxStepSlots);
             a.g_part[t2 * a.n_slots + sh.slot[buf][kk]] = 0.5 * sum;
           }
         }
@@ -665,10 +735,10 @@ __global__ void __launch_bounds__(kThreads, 1) pass64_kernel(const PassArgs64 a)
       for (int it = 0; it < 16; ++it) {
         const uint32_t i = (uint32_t)it * Tt + tau;
         if (!active) continue;
-        if (code == OP_CKPT) sp[gidx(i)] = tp[swz64(i)];
-        else tp[swz64(i)] = sp[gidx(i)];
+        if (code == OP_CKPT) sp[gidx(i_top | i)] = tp[swz64(i)];
+        else tp[swz64(i)] = sp[gidx(i_top | i)];
       }
-      __syncthreads();
+      barrier();
     }
   }
 
@@ -680,14 +750,14 @@ __global__ void __launch_bounds__(kThreads, 1) pass64_kernel(const PassArgs64 a)
     for (int it = 0; it < 16; ++it) {
       const uint32_t i = (uint32_t)it * Tt + tau;
       const double2 v = tp[swz64(i)];
-      if (active) dst[gidx(i)] = make_float2((float)v.x, (float)v.y);
+      if (active) dst[gidx(i_top | i)] = make_float2((float)v.x, (float)v.y);
     }
   } else if (pd.psi_dst != BUF_NONE) {
     double2* dst = state_ptr(pd.psi_dst);
 #pragma unroll 4
     for (int it = 0; it < 16; ++it) {
       const uint32_t i = (uint32_t)it * Tt + tau;
-      if (active) dst[gidx(i)] = tp[swz64(i)];
+      if (active) dst[gidx(i_top | i)] = tp[swz64(i)];
     }
   }
   if (BWD && pd.lam_dst == LAM_BUF) {
@@ -695,7 +765,7 @@ __global__ void __launch_bounds__(kThreads, 1) pass64_kernel(const PassArgs64 a)
 #pragma unroll 4
     for (int it = 0; it < 16; ++it) {
       const uint32_t i = (uint32_t)it * Tt + tau;
-      if (active) dst[gidx(i)] = tl[swz64(i)];
+      if (active) dst[gidx(i_top | i)] = tl[swz64(i)];
     }
   }
   if (!BWD && (pd.flags & PF_EXPECT)) {
@@ -704,28 +774,25 @@ __global__ void __launch_bounds__(kThreads, 1) pass64_kernel(const PassArgs64 a)
 #pragma unroll 1
     for (int it = 0; it < 16; ++it) {
       const uint32_t i = (uint32_t)it * Tt + tau;
-      const uint32_t ip = i ^ pd.xm_local;
+      const uint32_t ip = (i_top | i) ^ pd.xm_local;
       const double2 v = tp[swz64(i)];
-      const double2 w = ipow(tp[swz64(ip)], a.y_count);
+      const double2 w = ipow(amp(ip, 0), a.y_count);
       const uint32_t sg = __popc(gidx(ip) & a.z_mask) & 1u;
       acc += flipd(v.x * w.x + v.y * w.y, sg);  // Re(conj(v) w) with the Z signs
     }
     for (int off = 1; off < lanes; off <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
     if (Tt >= 32) {
       if (lane == 0) sh.dred[warp] = acc;
-      __syncthreads();
-      if (tid < tiles_per_cta) {
+      barrier();
+      if (tid < tiles_per_cta && rank == 0) {
         const int64_t t2 = first_tile + tid;
-        if (t2 < total_tiles) {
-          double sum = 0.0;
-          for (int w = 0; w < wpt; ++w) sum += sh.dred[tid * wpt + w];
-          a.e_part[t2] = sum;
-        }
+        if (t2 < total_tiles) a.e_part[t2] = tile_sum(&sh.dred[tid * wpt], 1);
       }
     } else if (active && (lane & (Tt - 1)) == 0) {
       a.e_part[tile] = acc;
     }
   }
+  if (SPLIT) barrier();  // no CTA leaves while another may read its shared memory
 }
 
 // ---- observables whose X/Y qubits lie outside the tile (App. B.2) -------------
@@ -774,29 +841,63 @@ __global__ void seed_full64_kernel(const double2* psi, double2* lam, int n_eff, 
 // ---- launchers -------------------------------------------------------------------
 cudaError_t launch_pass64(bool bwd, const PassArgs64& a, cudaStream_t st) {
   if (a.pd.K < kRegBits || a.pd.K > kMaxTileBits) return cudaErrorInvalidValue;
-  const int tiles_per_cta = kThreads >> (a.pd.K - kRegBits);
+  const int tl2 = a.pd.K - kRegBits;
   const int64_t total_tiles = (int64_t)a.B << a.tps_log2;
-  const int64_t grid = (total_tiles + tiles_per_cta - 1) / tiles_per_cta;
-  if (grid == 0) return cudaSuccess;
-  const size_t smem = (size_t)(bwd ? 2 : 1) * kTileAmps * sizeof(double2);
+  if (total_tiles == 0) return cudaSuccess;
+  const int n_sm = device_sms();
+  if (n_sm == 0) return cudaErrorInvalidDevice;
   const bool rounds = a.rounds != nullptr, rx = rounds && a.rx_items;
   if (rounds && (a.rpar == nullptr || a.pd.K < 7)) return cudaErrorInvalidValue;  // 8 lanes per tile at least
-  static OptIn once[6];
-  const void* fn = bwd ? (rx       ? reinterpret_cast<const void*>(pass64_kernel<true, true, true>)
-                          : rounds ? reinterpret_cast<const void*>(pass64_kernel<true, true>)
-                                   : reinterpret_cast<const void*>(pass64_kernel<true, false>))
-                       : (rx       ? reinterpret_cast<const void*>(pass64_kernel<false, true, true>)
-                          : rounds ? reinterpret_cast<const void*>(pass64_kernel<false, true>)
-                                   : reinterpret_cast<const void*>(pass64_kernel<false, false>));
-  cudaError_t e = opt_in(fn, smem, once[(bwd ? 3 : 0) + (rx ? 2 : rounds ? 1 : 0)]);
-  if (e != cudaSuccess) return e;
-  if (bwd && rx) pass64_kernel<true, true, true><<<(unsigned)grid, kThreads, smem, st>>>(a);
-  else if (bwd && rounds) pass64_kernel<true, true><<<(unsigned)grid, kThreads, smem, st>>>(a);
-  else if (bwd) pass64_kernel<true, false><<<(unsigned)grid, kThreads, smem, st>>>(a);
-  else if (rx) pass64_kernel<false, true, true><<<(unsigned)grid, kThreads, smem, st>>>(a);
-  else if (rounds) pass64_kernel<false, true><<<(unsigned)grid, kThreads, smem, st>>>(a);
-  else pass64_kernel<false, false><<<(unsigned)grid, kThreads, smem, st>>>(a);
-  return cudaGetLastError();
+  // Each of an SM's four schedulers has its own FP64 lanes and a warp keeps them
+  // busy alone, so the work should sit on all schedulers: CTAs shrink to one tile
+  // (one warp at least) while that leaves SMs without one, and two CTAs share a
+  // 12-qubit tile where the busiest SM's part of a tile, ceil(CTAs / SMs) /
+  // 2^split, falls by it. n = 12, d = 10: step of 64 samples (split) 980 us, of
+  // 128 (one CTA per tile and SM) 1,690 us. (Four or eight CTAs per tile gave
+  // nothing more: that leaves schedulers idle.)
+  int thr = kThreads;
+  while (thr > 32 && thr > (1 << tl2) && (total_tiles << tl2) < (int64_t)thr * n_sm) thr >>= 1;
+  const int64_t whole = (total_tiles + n_sm - 1) / n_sm, halves = (2 * total_tiles + n_sm - 1) / n_sm;
+  const int split = thr == kThreads && thr == 1 << tl2 && halves < 2 * whole ? 1 : 0;
+  PassArgs64 arg = a;
+  arg.split = split;
+  thr >>= split;
+  const int64_t grid = split ? total_tiles << split : (total_tiles + (thr >> tl2) - 1) / (thr >> tl2);
+  const size_t smem = (size_t)(bwd ? 2 : 1) * thr * 16 * sizeof(double2);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)thr);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 1u << split;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = split ? 1 : 0;
+#define QF_RUN(...)                                                                                            \
+  do {                                                                                                         \
+    static OptIn once;                                                                                         \
+    const cudaError_t e_ =                                                                                     \
+        opt_in(reinterpret_cast<const void*>(__VA_ARGS__), 2 * (size_t)kTileAmps * sizeof(double2), once);     \
+    if (e_ != cudaSuccess) return e_;                                                                          \
+    return cudaLaunchKernelEx(&cfg, __VA_ARGS__, arg);                                                         \
+  } while (0)
+  if (split) {
+    if (bwd && rx) QF_RUN(pass64_kernel<true, true, true, true>);
+    if (bwd && rounds) QF_RUN(pass64_kernel<true, true, false, true>);
+    if (bwd) QF_RUN(pass64_kernel<true, false, false, true>);
+    if (rx) QF_RUN(pass64_kernel<false, true, true, true>);
+    if (rounds) QF_RUN(pass64_kernel<false, true, false, true>);
+    QF_RUN(pass64_kernel<false, false, false, true>);
+  }
+  if (bwd && rx) QF_RUN(pass64_kernel<true, true, true>);
+  if (bwd && rounds) QF_RUN(pass64_kernel<true, true>);
+  if (bwd) QF_RUN(pass64_kernel<true, false>);
+  if (rx) QF_RUN(pass64_kernel<false, true, true>);
+  if (rounds) QF_RUN(pass64_kernel<false, true>);
+  QF_RUN(pass64_kernel<false, false>);
+#undef QF_RUN
 }
 
 cudaError_t launch_expect_full64(const double2* psi, int n_eff, int64_t B, int64_t rows, uint32_t xm, uint32_t zm,

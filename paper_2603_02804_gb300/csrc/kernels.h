@@ -206,6 +206,7 @@ struct PassArgs64 {
   double* e_part;         // [B * tiles per sample]
   double* g_part;         // [B * tiles per sample][n_slots]
   int32_t n_slots;
+  int32_t split;          // 2^split CTAs share a tile (set by launch_pass64)
 };
 cudaError_t launch_pass64(bool bwd, const PassArgs64& a, cudaStream_t st);
 cudaError_t launch_expect_full64(const double2* psi, int n_eff, int64_t B, int64_t rows, uint32_t xm, uint32_t zm,

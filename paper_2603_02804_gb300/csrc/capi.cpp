@@ -1753,7 +1753,7 @@ struct qf_batch {
   void* d_tables = nullptr;
   qf::BatchArgs args{};
   int64_t prep_total = 0, n_grad_out = 0;
-  int grid = 0;
+  int clusters = 0, cluster_size = 0;  // of the persistent kernel
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   // the last step's end: every step of a batch writes the same workspace, so
@@ -1874,23 +1874,47 @@ qf_status qf_batch_create(int32_t n_circuits, qf_circuit* const* circuits, const
       bwd_off[i] = o;
       o = al(o + b->circ[i]->fp.bwd.size() * sizeof(qf::PassDesc));
     }
-    // work items: samples of one circuit; largest first
+    // the persistent kernel's clusters: 8 CTAs, or fewer where the device does not hold one
+    for (b->cluster_size = 8; b->cluster_size >= 1; b->cluster_size /= 2)
+      if ((b->clusters = qf::batch_clusters(b->cluster_size)) > 0) break;
+    if (b->clusters <= 0 || cudaEventCreateWithFlags(&b->done, cudaEventDisableTiming) != cudaSuccess) {
+      cudaGetLastError();
+      batch_free(b);
+      delete b;
+      return fail(QF_ERR_CUDA, "the device does not hold the persistent kernel");
+    }
+    // work items: samples of one circuit. Circuits of several tiles per sample
+    // come first, as items for a cluster (enough samples to give each CTA
+    // tiles), then those of one tile, as items for a CTA; longest first.
     std::vector<qf::BatchItem> items;
     std::vector<double> cost;
-    for (int i = 0; i < n_circuits; ++i) {
-      const qf::FusedPlan& P = b->circ[i]->fp;
-      const int tps_log2 = P.n_eff - P.K;
-      const int tpc = qf::kThreads >> (P.K - qf::kRegBits);
-      const int step = tps_log2 == 0 ? tpc : 1;
-      for (int64_t b0 = 0; b0 < b->B[i]; b0 += step) {
-        items.push_back({i, (int32_t)b0});
-        const double ns = (double)std::min<int64_t>(step, b->B[i] - b0);
-        cost.push_back(ns * std::ldexp(1.0, P.n_eff) * (double)std::max(P.n_rounds, 1));
+    std::vector<int> per_item(n_circuits), g_ranks(n_circuits);
+    int n_wide = 0;
+    for (int wide = 1; wide >= 0; --wide) {
+      const size_t at = items.size();
+      for (int i = 0; i < n_circuits; ++i) {
+        const qf::FusedPlan& P = b->circ[i]->fp;
+        if ((P.n_eff > P.K) != (wide != 0)) continue;
+        const int64_t tps = 1ll << (P.n_eff - P.K);
+        const int64_t tpc = qf::kThreads >> (P.K - qf::kRegBits);
+        const int64_t cs = wide ? b->cluster_size : 1;
+        per_item[i] = (int)std::max<int64_t>(1, tpc * cs / tps);
+        g_ranks[i] = tps >= tpc ? (int)std::min(tps / tpc, cs) : 0;
+        for (int64_t b0 = 0; b0 < b->B[i]; b0 += per_item[i]) {
+          items.push_back({i, (int32_t)b0});
+          const int64_t ns = std::min<int64_t>(per_item[i], b->B[i] - b0);
+          const int64_t calls = ((ns * tps + tpc - 1) / tpc + cs - 1) / cs;  // per CTA and pass
+          cost.push_back((double)calls * (double)std::max(P.n_rounds, 1));
+        }
       }
+      std::vector<size_t> ord(items.size() - at);
+      for (size_t k = 0; k < ord.size(); ++k) ord[k] = at + k;
+      std::stable_sort(ord.begin(), ord.end(), [&](size_t x, size_t y) { return cost[x] > cost[y]; });
+      std::vector<qf::BatchItem> sorted;
+      for (size_t k : ord) sorted.push_back(items[k]);
+      std::copy(sorted.begin(), sorted.end(), items.begin() + at);
+      if (wide) n_wide = (int)items.size();
     }
-    std::vector<size_t> ord(items.size());
-    for (size_t k = 0; k < ord.size(); ++k) ord[k] = k;
-    std::stable_sort(ord.begin(), ord.end(), [&](size_t x, size_t y) { return cost[x] > cost[y]; });
     const size_t circ_off = o;
     o = al(o + n_circuits * sizeof(qf::BatchCircuit));
     const size_t items_off = o;
@@ -1956,12 +1980,14 @@ qf_status qf_batch_create(int32_t n_circuits, qf_circuit* const* circuits, const
       r.ba.ops = T.bwd_ops;
       r.ba.rounds = T.bwd_rounds;
       r.ba.rpar = rel<const float4>(w0 + L.rpb);
-      r.ba.g_accum = a.tps_log2 > 0 ? 1 : 0;
+      // (tiles of fewer than 9 qubits write their partials straight to a row per tile)
+      r.ba.g_accum = a.tps_log2 > 0 && g_ranks[i] > 0 && P.K >= 9 ? 1 : 0;
+      r.g_ranks = std::max(g_ranks[i], 1);
       r.fwd = reinterpret_cast<const qf::PassDesc*>(base + fwd_off[i]);
       r.bwd = reinterpret_cast<const qf::PassDesc*>(base + bwd_off[i]);
       r.n_fwd = (int32_t)fp.size();
       r.n_bwd = (int32_t)bp.size();
-      r.samples_per_item = a.tps_log2 == 0 ? (qf::kThreads >> (P.K - qf::kRegBits)) : 1;
+      r.samples_per_item = per_item[i];
       r.loss_kind = loss_kind;
       r.inv_B = 1.0 / (double)b->B[i];
       r.theta_off = b->theta_off[i];
@@ -1998,8 +2024,7 @@ qf_status qf_batch_create(int32_t n_circuits, qf_circuit* const* circuits, const
       gout_pref[i + 1] = gout_pref[i] + c->circ.n_params;
     }
     memcpy(img.data() + circ_off, recs.data(), recs.size() * sizeof(qf::BatchCircuit));
-    for (size_t k = 0; k < ord.size(); ++k)
-      memcpy(img.data() + items_off + k * sizeof(qf::BatchItem), &items[ord[k]], sizeof(qf::BatchItem));
+    memcpy(img.data() + items_off, items.data(), items.size() * sizeof(qf::BatchItem));
     memcpy(img.data() + prep_off, prep_pref.data(), prep_pref.size() * sizeof(int64_t));
     memcpy(img.data() + gout_off, gout_pref.data(), gout_pref.size() * sizeof(int64_t));
     e = cudaMemcpy(d, img.data(), total, cudaMemcpyHostToDevice);
@@ -2013,18 +2038,12 @@ qf_status qf_batch_create(int32_t n_circuits, qf_circuit* const* circuits, const
     b->args.n_circ = n_circuits;
     b->args.items = reinterpret_cast<const qf::BatchItem*>(base + items_off);
     b->args.n_items = (int32_t)items.size();
+    b->args.n_wide = n_wide;
     b->args.prep_off = reinterpret_cast<const int64_t*>(base + prep_off);
     b->args.grad_out_off = reinterpret_cast<const int64_t*>(base + gout_off);
     b->args.n_samples = b->sample_off[n_circuits];
     b->prep_total = prep_pref[n_circuits];
     b->n_grad_out = gout_pref[n_circuits];
-    b->grid = qf::batch_grid();
-    if (b->grid <= 0 || cudaEventCreateWithFlags(&b->done, cudaEventDisableTiming) != cudaSuccess) {
-      cudaGetLastError();
-      batch_free(b);
-      delete b;
-      return fail(QF_ERR_CUDA, "cannot query the device's SM count or make an event");
-    }
   } catch (const std::bad_alloc&) {
     if (b) {
       batch_free(b);
@@ -2074,7 +2093,7 @@ qf_status qf_batch_train_step(qf_batch* b, const float* theta_d, const float* x_
   a.queue = reinterpret_cast<int32_t*>(a.ws + b->queue_off);
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
   QF_CU(batch_begin(b, st));
-  QF_CU(qf::launch_batch(a, b->grid, b->prep_total, b->n_grad_out, st));
+  QF_CU(qf::launch_batch(a, b->clusters, b->cluster_size, b->prep_total, b->n_grad_out, st));
   QF_CU(batch_end(b, st));
   return QF_OK;
 }

@@ -13,6 +13,7 @@
 // (b, j): loads and stores of a step carry it as their immediate offset, one
 // code copy per b. An XOR swizzle (i ^ ((i >> 4) & 15)) needed an instruction
 // or two per address, about 70 a step and thread.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -692,15 +693,14 @@ struct PassShared {
 
 // One CTA's share of a pass: tiles first_tile .. first_tile + tiles_per_cta-1
 // (tile = sample * tiles_per_sample + tile within the sample). Ends with a
-// barrier, so a CTA may call it again for another pass or tile range. LOADS:
-// tile loads in flight per thread and state (8 = the whole tile at once).
+// barrier, so a CTA may call it again for another pass or tile range.
 // KC: the tile's qubits where they are known when compiled (12: one tile per
 // CTA of 256 threads, every tile active), else 0. The constant lets the tile
 // loads, the group bases and the reductions drop their index arithmetic: with
 // the padded layout, 366 -> 291 instructions per warp and round forward and 786
 // -> 659 adjoint; step of n = 20, d = 24, 64 samples 25.10 -> 23.00 ms, of n =
 // 12, d = 20, 256 samples 237 -> 222 us.
-template <bool BWD, bool ROUNDS, int LOADS = 8, bool TC = false, bool RX = false, int KC = 0>
+template <bool BWD, bool ROUNDS, bool TC = false, bool RX = false, int KC = 0>
 __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_tile, float2* smem, PassShared& sh,
                                          const TcCtx* tc = nullptr) {
   uint32_t (&s_lg)[256] = sh.lg;
@@ -850,21 +850,18 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
         half ? reinterpret_cast<const __nv_bfloat162*>(a.hslots) + (int64_t)psrc * a.slot_stride + sbase : nullptr;
     const bool two = BWD && pd.lam_src == LAM_BUF;
     const float2* lsrc = a.lam + sbase;
+    float4 vp[8], vl[8];
 #pragma unroll
-    for (int i0 = 0; i0 < 8; i0 += LOADS) {
-      float4 vp[LOADS], vl[LOADS];
+    for (int it = 0; it < 8; ++it) {
+      const uint32_t g = g_it(it);
+      if (half) vp[it] = bf16x4_to_f4(__ldcg(reinterpret_cast<const uint2*>(hsrc + g)));
+      else vp[it] = __ldcg(reinterpret_cast<const float4*>(src + g));
+      if (two) vl[it] = __ldcg(reinterpret_cast<const float4*>(lsrc + g));
+    }
 #pragma unroll
-      for (int it = 0; it < LOADS; ++it) {
-        const uint32_t g = g_it(i0 + it);
-        if (half) vp[it] = bf16x4_to_f4(__ldcg(reinterpret_cast<const uint2*>(hsrc + g)));
-        else vp[it] = __ldcg(reinterpret_cast<const float4*>(src + g));
-        if (two) vl[it] = __ldcg(reinterpret_cast<const float4*>(lsrc + g));
-      }
-#pragma unroll
-      for (int it = 0; it < LOADS; ++it) {
-        st_pair(tp, p_it(i0 + it), vp[it]);
-        if (two) st_pair(tl, p_it(i0 + it), vl[it]);
-      }
+    for (int it = 0; it < 8; ++it) {
+      st_pair(tp, p_it(it), vp[it]);
+      if (two) st_pair(tl, p_it(it), vl[it]);
     }
   }
   if (BWD && pd.lam_src == LAM_BUF && psrc == SRC_GENERATE && active) {
@@ -1023,12 +1020,11 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
       sb ^= 1;
       if (BWD && Tt >= 32 && a.g_accum) {
         // every tile of this call belongs to one sample: one thread per term sums
-        // the tiles in order and adds to the sample's row (stored by its tile 0);
-        // within a tile the warp sums add in float32, as the warp shuffles do,
-        // then float64 across tiles
+        // the tiles in order and adds to row g_row (stored by the row's first
+        // call); within a tile the warp sums add in float32, as the warp shuffles
+        // do, then float64 across tiles
         const int nk = nr * 8;
-        const int64_t b2 = first_tile >> a.tps_log2;
-        const bool first = (first_tile & ((1ll << a.tps_log2) - 1)) == 0;
+        const bool first = a.g_first != 0;
         for (int kk = nthr - 1 - tid; kk < nk; kk += nthr) {  // the last warp (warp 0 stages)
           const int32_t term = s_slot[buf][kk];
           if (term < 0) continue;
@@ -1039,7 +1035,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
               for (int w = 0; w < wpt; ++w) sf += s_red[buf][tc * wpt + w][kk];
               sum += (double)sf;
             }
-          double* dst = a.g_part + b2 * a.n_slots + term;
+          double* dst = a.g_part + a.g_row * a.n_slots + term;
           *dst = first ? 0.5 * sum : *dst + 0.5 * sum;
         }
         buf ^= 1;
@@ -1152,7 +1148,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
       for (int it = 0; it < 8; ++it) {
         if (!active) continue;
         if (code == OP_CKPT) *reinterpret_cast<float4*>(sp + g_it(it)) = ld_pair(tp, p_it(it));
-        else st_pair(tp, p_it(it), *reinterpret_cast<const float4*>(sp + g_it(it)));
+        else st_pair(tp, p_it(it), __ldcg(reinterpret_cast<const float4*>(sp + g_it(it))));
       }
       __syncthreads();
     }
@@ -1235,7 +1231,7 @@ __global__ void __launch_bounds__(kThreads, MINB) pass_kernel(const PassArgs a) 
   extern __shared__ __align__(16) float2 smem[];
   __shared__ PassShared sh;
   const int64_t first = KC ? (int64_t)blockIdx.x : (int64_t)blockIdx.x * (blockDim.x >> (a.pd.K - kRegBits));
-  pass_cta<BWD, ROUNDS, 8, false, RX, KC>(a, first, smem, sh);
+  pass_cta<BWD, ROUNDS, false, RX, KC>(a, first, smem, sh);
 }
 
 // Forward pass with the rounds on the tensor cores: one 12-qubit tile per
@@ -1262,7 +1258,7 @@ __global__ void __launch_bounds__(kThreads, 2) tc_pass_kernel(const PassArgs a) 
   __syncthreads();
   tc_fence_after();
   TcCtx ctx{tmem_slot, mbar, reinterpret_cast<float*>(smem + kTilePad)};
-  pass_cta<false, true, 8, true, false, 12>(a, (int64_t)blockIdx.x, smem, sh, &ctx);
+  pass_cta<false, true, true, false, 12>(a, (int64_t)blockIdx.x, smem, sh, &ctx);
   // pass_cta ends with a barrier; every tensor-memory access is complete
   tc_fence_after();
   if (warp == 0)
@@ -1688,16 +1684,53 @@ __device__ void load_args(PassArgs& dst, const PassArgs& src, const PassDesc& pd
   __syncthreads();
 }
 
-__device__ void run_item_pass(bool bwd, const PassArgs& a, int32_t b0) {
+// Shared memory of the persistent kernel: psi and lambda tiles, the arguments
+// of the running pass and pass_cta's own (one dynamic block, so that the pass
+// functions, which are called and not inlined, share it).
+struct BatchShared {
+  PassArgs args;
+  PassShared pass;
+};
+__device__ __forceinline__ BatchShared& batch_shared() {
   extern __shared__ __align__(16) float2 smem[];
-  __shared__ PassShared sh;
-  const int tpc = kThreads >> (a.pd.K - kRegBits);
-  // tpc tiles per call: with one tile per sample (tps = 1) the item's samples
-  // b0 .. b0 + tpc - 1 in one call, else the tiles of sample b0 in turn
-  const int64_t tps = 1ll << a.tps_log2;
-  for (int64_t t = 0; t < tps; t += tpc) {
-    if (bwd) pass_cta<true, true, 2>(a, (int64_t)b0 * tps + t, smem, sh);
-    else pass_cta<false, true, 2>(a, (int64_t)b0 * tps + t, smem, sh);
+  return *reinterpret_cast<BatchShared*>(smem + 2 * kTilePad);
+}
+// Called, so that each instance has the registers to itself: inlined side by
+// side in the persistent loop they spilled 156 bytes.
+template <bool BWD, int KC>
+__device__ __noinline__ void batch_pass(int64_t first_tile) {
+  extern __shared__ __align__(16) float2 smem[];
+  BatchShared& bs = batch_shared();
+  pass_cta<BWD, true, false, false, KC>(bs.args, first_tile, smem, bs.pass);
+}
+
+// The tile groups (as many tiles as a CTA holds) rank, rank + n_ranks, ... of
+// one pass over samples b0 .. b0 + ns - 1.
+__device__ void run_item_pass(bool bwd, const BatchCircuit& C, const PassDesc& pd, char* ws, int64_t b0, int ns,
+                              uint32_t rank, uint32_t n_ranks) {
+  BatchShared& bs = batch_shared();
+  load_args(bs.args, bwd ? C.ba : C.fa, pd, ws);
+  const int tpc = kThreads >> (pd.K - kRegBits);
+  const int64_t tps = 1ll << C.fa.tps_log2;
+  const int64_t groups = (ns * tps + tpc - 1) / tpc;
+  for (int64_t g = rank; g < groups; g += n_ranks) {
+    if (bwd && C.ba.g_accum) {
+      // rows per sample: one for each CTA that takes tiles of it
+      const int64_t per = tps / tpc, gs = g & (per - 1);
+      if (threadIdx.x == 0) {
+        bs.args.g_row = (b0 + g / per) * C.g_ranks + (gs & (C.g_ranks - 1));
+        bs.args.g_first = gs < C.g_ranks;
+      }
+      __syncthreads();
+    }
+    const int64_t first = b0 * tps + g * tpc;
+    if (pd.K == kMaxTileBits) {
+      if (bwd) batch_pass<true, 12>(first);
+      else batch_pass<false, 12>(first);
+    } else {
+      if (bwd) batch_pass<true, 0>(first);
+      else batch_pass<false, 0>(first);
+    }
   }
 }
 
@@ -1717,52 +1750,73 @@ __global__ void batch_prep_kernel(const BatchArgs a, int64_t total) {
   prep_one(p, i - a.prep_off[c]);
 }
 
-// Persistent kernel: CTAs take work items (one sample, or a group of small
-// samples, of one circuit; largest first) from an atomic queue and run the
-// item's forward passes, its loss derivative and its adjoint passes
-// themselves, so items never wait on each other.
+// Persistent kernel over two queues of work items (some samples of one circuit,
+// longest first). Items whose samples span several tiles are run by a cluster
+// of CTAs: each pass's tiles are dealt to the CTAs, with a cluster barrier
+// between passes (it also orders their writes to the states). One CTA per
+// sample made the longest item the length of the launch: 32 circuits of 8 to
+// 16 qubits 14.57 -> 7.65 ms. Items of single-tile circuits are then taken by the
+// CTAs one by one. Items never wait on each other.
+__device__ void run_item(const BatchArgs& a, const BatchItem item, bool wide) {
+  namespace cg = cooperative_groups;
+  const BatchCircuit& C = a.circ[item.c];
+  const uint32_t rank = wide ? cg::this_cluster().block_rank() : 0u;
+  const uint32_t n_ranks = wide ? cg::this_cluster().num_blocks() : 1u;
+  const int64_t b0 = item.b0;
+  const int ns = (int)min((int64_t)C.samples_per_item, C.fa.B - b0);
+  auto barrier = [&]() {
+    if (wide) cg::this_cluster().sync();
+    else __syncthreads();
+  };
+  for (int p = 0; p < C.n_fwd; ++p) {
+    run_item_pass(false, C, C.fwd[p], a.ws, b0, ns, rank, n_ranks);
+    barrier();
+  }
+  // E and dL/dE of the item's samples
+  if (rank == 0) {
+    const int64_t tps = 1ll << C.fa.tps_log2;
+    for (int i = (int)threadIdx.x; i < ns; i += kThreads) {
+      const int64_t b = b0 + i;
+      const double* ep = rebase(C.fa.e_part, a.ws) + b * tps;
+      double e = 0.0;
+      for (int64_t t = 0; t < tps; ++t) e += __ldcg(ep + t);
+      const int64_t s = C.sample_off + b;
+      a.E[s] = e;
+      double g = 1.0, lt = e;
+      if (C.loss_kind == 1) {
+        const double dd = e - (double)a.y[s];
+        g = 2.0 * dd * C.inv_B;
+        lt = dd * dd * C.inv_B;
+      }
+      const_cast<double*>(rebase(C.ba.dLdE, a.ws))[b] = g;  // the item's own workspace row
+      a.lterm[s] = lt;
+    }
+  }
+  barrier();
+  for (int p = 0; p < C.n_bwd; ++p) {
+    run_item_pass(true, C, C.bwd[p], a.ws, b0, ns, rank, n_ranks);
+    barrier();
+  }
+}
+
 __global__ void __launch_bounds__(kThreads, 2) batch_kernel(const BatchArgs a) {
-  __shared__ PassArgs s_a;
+  namespace cg = cooperative_groups;
   __shared__ int s_item;
   for (;;) {
-    if (threadIdx.x == 0) s_item = atomicAdd(a.queue, 1);
+    if (cg::this_cluster().block_rank() == 0 && threadIdx.x == 0) s_item = atomicAdd(a.queue, 1);
+    cg::this_cluster().sync();
+    const int it = *cg::this_cluster().map_shared_rank(&s_item, 0);
+    cg::this_cluster().sync();
+    if (it >= a.n_wide) break;
+    run_item(a, a.items[it], true);
+  }
+  for (;;) {
+    if (threadIdx.x == 0) s_item = a.n_wide + atomicAdd(a.queue + 1, 1);
     __syncthreads();
     const int it = s_item;
     __syncthreads();
     if (it >= a.n_items) return;
-    const BatchItem item = a.items[it];
-    const BatchCircuit& C = a.circ[item.c];
-    for (int p = 0; p < C.n_fwd; ++p) {
-      load_args(s_a, C.fa, C.fwd[p], a.ws);
-      run_item_pass(false, s_a, item.b0);
-    }
-    // E and dL/dE of the item's samples (their tiles were written by this CTA)
-    {
-      const int64_t B = C.fa.B;
-      const int64_t tps = 1ll << C.fa.tps_log2;
-      const int ns = (int)min((int64_t)C.samples_per_item, B - item.b0);
-      if ((int)threadIdx.x < ns) {
-        const int64_t b = item.b0 + threadIdx.x;
-        const double* ep = rebase(C.fa.e_part, a.ws) + b * tps;
-        double e = 0.0;
-        for (int64_t t = 0; t < tps; ++t) e += ep[t];
-        const int64_t s = C.sample_off + b;
-        a.E[s] = e;
-        double g = 1.0, lt = e;
-        if (C.loss_kind == 1) {
-          const double dd = e - (double)a.y[s];
-          g = 2.0 * dd * C.inv_B;
-          lt = dd * dd * C.inv_B;
-        }
-        const_cast<double*>(rebase(C.ba.dLdE, a.ws))[b] = g;  // the item's own workspace row
-        a.lterm[s] = lt;
-      }
-      __syncthreads();
-    }
-    for (int p = 0; p < C.n_bwd; ++p) {
-      load_args(s_a, C.ba, C.bwd[p], a.ws);
-      run_item_pass(true, s_a, item.b0);
-    }
+    run_item(a, a.items[it], false);
   }
 }
 
@@ -1775,7 +1829,7 @@ __global__ void batch_g_reduce_kernel(const BatchArgs a, int64_t n_out) {
   const BatchCircuit& C = a.circ[c];
   const int p = (int)(o - a.grad_out_off[c]);
   const double* gp = rebase(C.ba.g_part, a.ws);
-  const int64_t rows = C.ba.g_accum ? C.ba.B : (C.ba.B << C.ba.tps_log2);
+  const int64_t rows = C.ba.g_accum ? C.ba.B * C.g_ranks : (C.ba.B << C.ba.tps_log2);
   double s = 0.0;
   for (int k = C.param_off[p]; k < C.param_off[p + 1]; ++k) {
     const int term = C.param_terms[k];
@@ -1829,20 +1883,56 @@ int64_t stream_grid(int64_t want) {
   return cap > 0 && want > cap ? cap : want;
 }
 
-int batch_grid() { return 2 * device_sms(); }
+namespace {
+constexpr size_t kBatchSmem = 2 * (size_t)kTilePad * sizeof(float2) + sizeof(BatchShared);
 
-cudaError_t launch_batch(const BatchArgs& a, int grid, int64_t prep_total, int64_t n_grad_out, cudaStream_t st) {
+cudaLaunchConfig_t batch_config(int clusters, int size, cudaStream_t st, cudaLaunchAttribute* attr) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(clusters * size));
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = kBatchSmem;
+  cfg.stream = st;
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = (unsigned)size;
+  attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+cudaError_t batch_opt_in() {
   static OptIn once;
-  const size_t smem = 2 * (size_t)kTilePad * sizeof(float2);
-  cudaError_t e = opt_in(reinterpret_cast<const void*>(batch_kernel), smem, once);
+  return opt_in(reinterpret_cast<const void*>(batch_kernel), kBatchSmem, once);
+}
+}  // namespace
+
+// Clusters of `size` CTAs of the persistent kernel that the device runs at once
+// (0 when it cannot).
+int batch_clusters(int size) {
+  cudaLaunchAttribute attr;
+  const cudaLaunchConfig_t cfg = batch_config(1, size, nullptr, &attr);
+  int n = 0;
+  if (batch_opt_in() != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, reinterpret_cast<const void*>(batch_kernel), &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
+}
+
+cudaError_t launch_batch(const BatchArgs& a, int clusters, int cluster_size, int64_t prep_total, int64_t n_grad_out,
+                         cudaStream_t st) {
+  cudaError_t e = batch_opt_in();
   if (e != cudaSuccess) return e;
   if (prep_total > 0) batch_prep_kernel<<<(unsigned)((prep_total + 63) / 64), 64, 0, st>>>(a, prep_total);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if ((e = cudaMemsetAsync(a.queue, 0, sizeof(int32_t), st)) != cudaSuccess) return e;
+  if ((e = cudaMemsetAsync(a.queue, 0, 2 * sizeof(int32_t), st)) != cudaSuccess) return e;
   if (a.n_items > 0) {
-    const int g = grid < a.n_items ? grid : a.n_items;
-    batch_kernel<<<(unsigned)g, kThreads, smem, st>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    const int narrow = (a.n_items - a.n_wide + cluster_size - 1) / cluster_size;
+    const int want = a.n_wide > narrow ? a.n_wide : narrow;
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = batch_config(clusters < want ? clusters : want, cluster_size, st, &attr);
+    if ((e = cudaLaunchKernelEx(&cfg, batch_kernel, a)) != cudaSuccess) return e;
   }
   if (n_grad_out > 0) batch_g_reduce_kernel<<<(unsigned)((n_grad_out * 32 + 255) / 256), 256, 0, st>>>(a, n_grad_out);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;

@@ -34,7 +34,9 @@ struct PassArgs {
   double* e_part;         // [B * tiles per sample]
   double* g_part;         // [B * tiles per sample][n_slots], or [B][n_slots] when g_accum
   int32_t n_slots;
-  int32_t g_accum;        // round programs: add the partials of a sample's tiles into one row
+  int32_t g_accum;        // round programs: a call's tiles are of one sample, its partials add into row g_row
+  int32_t g_first;        // the row's first call stores instead
+  int64_t g_row;
   int32_t rx_items;       // round programs with RX items (the RX-capable kernels run them)
   // The pass that computes the expectation may also finish the loss: with
   // done != null, the last CTA to finish sums E from e_part and writes E, the
@@ -223,7 +225,8 @@ struct BatchCircuit {
   const PassDesc* fwd;        // forward passes (observable folded in)
   const PassDesc* bwd;
   int32_t n_fwd, n_bwd;
-  int32_t samples_per_item;   // samples of one work item (tiles per CTA when a tile is a sample)
+  int32_t samples_per_item;   // samples of one work item
+  int32_t g_ranks;            // g_accum: rows per sample, one per CTA that takes tiles of it
   int32_t loss_kind;          // QF_LOSS_SUM or QF_LOSS_MSE
   double inv_B;
   int64_t theta_off, x_off, sample_off, grad_off;
@@ -241,9 +244,10 @@ struct BatchItem {
 struct BatchArgs {
   const BatchCircuit* circ;
   int32_t n_circ;
-  const BatchItem* items;
+  const BatchItem* items;      // n_wide items for clusters, then those for single CTAs
   int32_t n_items;
-  int32_t* queue;              // work-queue head (zeroed before each launch)
+  int32_t n_wide;
+  int32_t* queue;              // the two work-queue heads (zeroed before each launch)
   char* ws;
   const float* theta;
   const float* x;
@@ -259,9 +263,10 @@ struct BatchArgs {
 
 // prep, work-queue reset, persistent forward+adjoint, gradient and loss
 // reductions: 4 kernels and one memset on `st`.
-cudaError_t launch_batch(const BatchArgs& a, int grid, int64_t prep_total, int64_t n_grad_out, cudaStream_t st);
-// Persistent batch kernel grid: two CTAs per SM of the current device.
-int batch_grid();
+cudaError_t launch_batch(const BatchArgs& a, int clusters, int cluster_size, int64_t prep_total, int64_t n_grad_out,
+                         cudaStream_t st);
+// Clusters of `size` CTAs of the persistent kernel that the current device holds.
+int batch_clusters(int size);
 // SMs of the current device (queried once per device; 0 if the query fails).
 int device_sms();
 // Grid of a grid-strided kernel that wants `want` CTAs: at most 16 per SM.

@@ -1,0 +1,81 @@
+"""Launch shapes that depend on the number of tiles: CTAs of 32 to 256 threads
+for small tiles, and two CTAs per 12-qubit complex128 tile."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import oracle as orc
+from paper_2603_02804_gb300 import build as qbuild
+from paper_2603_02804_gb300.torch_api import Batch, Simulator
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    qbuild.build()
+    orc.build()
+
+
+def check(sim, circ, n, P, B, obs, real, tol, seed):
+    rng = np.random.default_rng(seed)
+    theta = rng.uniform(0, 2 * np.pi, P).astype(real)
+    x = rng.uniform(0, np.pi, (B, n)).astype(real)
+    y = (2 * rng.integers(0, 2, B) - 1).astype(real)
+    loss, E, g = sim.train_step(*(torch.from_numpy(v).cuda() for v in (theta, x, y)), loss="mse")
+    t64, x64 = theta.astype(np.float64), x.astype(np.float64)
+    Er = orc.expectation(circ, t64, x64, obs)
+    gr, _ = orc.gradient(circ, t64, x64, obs, dLdE=orc.mse_dLdE(Er, y))
+    assert np.max(np.abs(E.cpu().numpy() - Er)) < tol
+    assert np.max(np.abs(g.cpu().numpy() - gr)) < tol
+    assert abs(loss.item() - orc.mse_loss(Er, y)) < tol * 4
+
+
+# batches around the sizes where the CTA shrinks to 128, 64 and 32 threads on a GPU of about 150 SMs, ragged
+# tails of a CTA's tiles among them; the parity tests' tolerances (1e-5 complex64, 1e-11 complex128)
+@pytest.mark.parametrize("n,B", [(4, 3), (5, 700), (7, 1), (7, 37), (7, 1400), (8, 600), (8, 1300), (9, 330),
+                                 (10, 75), (10, 310), (11, 151), (11, 153)])
+def test_small_tiles(n, B):
+    check(Simulator(n, 2, B, obs="ZX"), orc.hea(n, 2), n, 6 * n, B, "ZX", np.float32, 1e-5, n * B)
+
+
+def generic_rows(n, d):
+    rows = []
+    for layer in range(d):
+        for q in range(n):
+            rows += [(1, q, -1, (layer * n + q) * 2), (2, q, -1, (layer * n + q) * 2 + 1)]
+        rows += [(4, q, q + 1, -1) for q in range(n - 1)]
+    return rows
+
+
+@pytest.mark.parametrize("program", ["rounds", "cnot"])
+@pytest.mark.parametrize("n,B", [(7, 3), (11, 5), (12, 1), (12, 76), (12, 80), (13, 3)])
+def test_complex128_shapes(n, B, program):
+    """Whole and shared tiles; X and Y on the bits that a shared tile splits."""
+    obs = "Z" + "I" * (n - 2) + "Y" if n <= 12 else "ZX"
+    if program == "rounds":
+        sim, circ, P = Simulator(n, 2, B, obs=obs, precision="complex128"), orc.hea(n, 2), 6 * n
+    else:
+        rows, P = generic_rows(n, 2), 4 * n
+        sim = Simulator(n, 0, B, gates=rows, n_params=P, obs=obs, precision="complex128")
+        circ = orc.Circuit(n=n, gates=np.array(rows, np.int32), n_params=P)
+    check(sim, circ, n, P, B, obs, np.float64, 1e-11, n + B)
+
+
+@pytest.mark.parametrize("K,specs", [(8, [(9, 2, 5), (10, 2, 3), (13, 2, 2)]), (9, [(10, 2, 9), (12, 2, 3), (14, 1, 2)]),
+                                     (12, [(13, 2, 9), (15, 2, 3), (16, 1, 2), (17, 1, 1), (12, 2, 5), (8, 3, 40)])])
+def test_batch_tiles_dealt_to_a_cluster(K, specs):
+    """Persistent batches whose samples span 2 to 32 tiles, of every tile width
+    class (several samples per CTA, one tile per CTA, several per CTA)."""
+    rng = np.random.default_rng(K)
+    th = [rng.uniform(0, 2 * np.pi, 3 * n * d).astype(np.float32) for n, d, _ in specs]
+    xs = [rng.uniform(0, np.pi, (B, n)).astype(np.float32) for n, _, B in specs]
+    cat = lambda v: torch.from_numpy(np.concatenate([a.reshape(-1) for a in v])).cuda()
+    bt = Batch(specs, tile_bits=K)
+    _, E, g = bt.train_step(cat(th), cat(xs))
+    E, g = E.cpu().numpy(), g.cpu().numpy()
+    for i, (n, d, B) in enumerate(specs):
+        c, t64, x64 = orc.hea(n, d), th[i].astype(np.float64), xs[i].astype(np.float64)
+        gr, Er = orc.gradient(c, t64, x64, "Z")
+        assert np.max(np.abs(E[bt.sample_off[i]:bt.sample_off[i + 1]] - Er)) < 1e-5, (n, d, B)
+        assert np.max(np.abs(g[bt.theta_off[i]:bt.theta_off[i + 1]] - gr)) < 1e-5 * B, (n, d, B)

@@ -1981,8 +1981,15 @@ cudaError_t launch_pass(bool bwd, const PassArgs& a, cudaStream_t st, int fwd_ct
     __VA_ARGS__<<<(unsigned)grid, thr, smem, st>>>(a);                                       \
     return cudaGetLastError();                                                               \
   } while (0)
+  // one CTA per SM at most: the adjoint's registers need not leave room for two
+  // (the two-CTA instance of runtime tile sizes spills: n = 8, d = 20, 64 samples
+  // 102 us a step against 96)
+  const bool alone = grid <= n_sm;
   if (bwd) {
+    if (!rounds && alone) QF_RUN(pass_kernel<true, false, false, 1>);
     if (!rounds) QF_RUN(pass_kernel<true, false>);
+    if (rx && alone && !k12) QF_RUN(pass_kernel<true, true, true, 1>);
+    if (alone && !k12 && !rx) QF_RUN(pass_kernel<true, true, false, 1>);
     if (rx && k12) QF_RUN(pass_kernel<true, true, true, 2, 12>);
     if (rx) QF_RUN(pass_kernel<true, true, true>);
     if (k12) QF_RUN(pass_kernel<true, true, false, 2, 12>);

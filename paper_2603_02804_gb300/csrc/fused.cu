@@ -906,9 +906,14 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
   uint32_t pend = 0;  // links whose CZ signs the tile's amplitudes still lack (round programs)
   int32_t pc = pd.op_begin;
   const uint2* ops = a.ops;
+  // (round programs: one op per step, read a step ahead)
+  uint2 next = make_uint2(0u, 0u);
+  if (ROUNDS && pc < pd.op_end) next = __ldg(ops + pc);
 #pragma unroll 1
   while (pc < pd.op_end) {
-    const uint2 op = __ldg(ops + pc++);
+    const uint2 op = ROUNDS ? next : __ldg(ops + pc);
+    ++pc;
+    if (ROUNDS && pc < pd.op_end) next = __ldg(ops + pc);
     const uint32_t code = op.x & 15u;
     if (ROUNDS && code == OP_STEP) {
       // ---- round step: straight-line rounds over the 4 register bits

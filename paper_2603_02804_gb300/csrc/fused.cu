@@ -702,7 +702,7 @@ struct PassShared {
 // 12, d = 20, 256 samples 237 -> 222 us.
 template <bool BWD, bool ROUNDS, bool TC = false, bool RX = false, int KC = 0>
 __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_tile, float2* smem, PassShared& sh,
-                                         const TcCtx* tc = nullptr) {
+                                         const TcCtx* tc = nullptr, float (*acc_rows)[8][32] = nullptr) {
   uint32_t (&s_lg)[256] = sh.lg;
   float (&s_red)[2][kThreads / 32][kMaxStepSlots] = sh.red;
   int32_t (&s_slot)[2][kMaxStepSlots] = sh.slot;
@@ -1077,32 +1077,70 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
         r[j] = at[reg_off(j, so)];
         if (BWD) l[j] = at[lam_at + reg_off(j, so)];
       }
+      // ops are read two ahead and their coefficients one ahead: a step's ops
+      // run one after another, and each was two dependent loads
+      auto coef = [&](uint2 o, float4& m0, float4& m1) {
+        if (!BWD && (o.x & 15u) == OP_U) {
+          m0 = __ldg(a.mats + 2 * (o.x >> 8));
+          m1 = __ldg(a.mats + 2 * (o.x >> 8) + 1);
+        } else if (BWD && (o.x & 15u) == OP_G) {
+          const float2 v = __ldg(a.cs + o.y);
+          m0 = make_float4(v.x, v.y, 0.f, 0.f);
+        }
+      };
+      uint2 o1 = make_uint2(0u, 0u), o2 = o1;
+      float4 m0 = make_float4(0.f, 0.f, 0.f, 0.f), m1 = m0;
+      if (nops > 0) o1 = __ldg(ops + pc);
+      if (nops > 1) o2 = __ldg(ops + pc + 1);
+      if (nops > 0) coef(o1, m0, m1);
+      pc += nops;
 #pragma unroll 1
       for (int k = 0; k < nops; ++k) {
-        const uint2 o = __ldg(ops + pc++);
+        const uint2 o = o1;
+        const float4 c0 = m0, c1 = m1;
+        o1 = o2;
+        if (k + 1 < nops) coef(o1, m0, m1);
+        if (k + 2 < nops) o2 = __ldg(ops + pc - nops + k + 2);
         const uint32_t oc = o.x & 15u;
         if (!BWD && oc == OP_U) {
-          const uint32_t m = o.x >> 8;
-          const float4 m0 = __ldg(a.mats + 2 * m), m1 = __ldg(a.mats + 2 * m + 1);
           switch ((o.x >> 4) & 3u) {
-            case 0: apply_u<0>(r, m0, m1); break;
-            case 1: apply_u<1>(r, m0, m1); break;
-            case 2: apply_u<2>(r, m0, m1); break;
-            default: apply_u<3>(r, m0, m1); break;
+            case 0: apply_u<0>(r, c0, c1); break;
+            case 1: apply_u<1>(r, c0, c1); break;
+            case 2: apply_u<2>(r, c0, c1); break;
+            default: apply_u<3>(r, c0, c1); break;
           }
         } else if (BWD && oc == OP_G) {
           const uint32_t rr = (o.x >> 4) & 3u, kind = (o.x >> 6) & 3u, ks = (o.x >> 8) & 0xffu;
-          const float2 csv = __ldg(a.cs + o.y);
           float acc;
-          if (kind == G_RZ) acc = bwd_dispatch_r<G_RZ>(rr, r, l, csv.x, csv.y);
-          else if (kind == G_RY) acc = bwd_dispatch_r<G_RY>(rr, r, l, csv.x, csv.y);
-          else acc = bwd_dispatch_r<G_RX>(rr, r, l, csv.x, csv.y);
-          for (int off = 1; off < lanes; off <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-          if (Tt >= 32) {
-            if (lane == 0) s_red[buf][warp][ks] = acc;
-            if (tid == 0) s_slot[buf][ks] = (int32_t)o.y;
-          } else if (active && (lane & (Tt - 1)) == 0) {
-            a.g_part[tile * a.n_slots + o.y] = 0.5 * (double)acc;
+          if (kind == G_RZ) acc = bwd_dispatch_r<G_RZ>(rr, r, l, c0.x, c0.y);
+          else if (kind == G_RY) acc = bwd_dispatch_r<G_RY>(rr, r, l, c0.x, c0.y);
+          else acc = bwd_dispatch_r<G_RX>(rr, r, l, c0.x, c0.y);
+          if (lanes >= 8) {
+            // eight terms are reduced over the tile's lanes at once (a warp's own
+            // rows: no barrier; the term ids are the same in every warp): five
+            // shuffles in a chain after each rotation, and the loads of its op,
+            // took as long as the arithmetic (n = 10 with CNOTs, d = 6, 100
+            // samples: step 163 -> 138 us)
+            float (&s_acc)[8][32] = acc_rows[warp];
+            s_acc[ks & 7u][lane] = acc;
+            if (lane == 0) s_slot[buf][ks] = (int32_t)o.y;
+            if ((ks & 7u) == 7u || (int)ks == nk - 1) {
+              __syncwarp();
+              float v[8];
+#pragma unroll
+              for (int i = 0; i < 8; ++i) v[i] = (uint32_t)i <= (ks & 7u) ? s_acc[i][lane] : 0.f;
+              int idx;
+              const float sum = butterfly8(v, lanes, lane, idx);
+              const uint32_t kk = (ks & ~7u) + (uint32_t)idx;
+              if ((lane & ((lanes >> 3) - 1)) == 0 && kk <= ks) {
+                if (Tt >= 32) s_red[buf][warp][kk] = sum;
+                else if (active) a.g_part[tile * a.n_slots + s_slot[buf][kk]] = 0.5 * (double)sum;
+              }
+              __syncwarp();
+            }
+          } else {
+            for (int off = 1; off < lanes; off <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+            if (active && (lane & (Tt - 1)) == 0) a.g_part[tile * a.n_slots + o.y] = 0.5 * (double)acc;
           }
         } else if (oc == OP_CNOT) {
           const bool creg = ((o.y >> 8) & 1u) != 0;
@@ -1236,7 +1274,12 @@ __global__ void __launch_bounds__(kThreads, MINB) pass_kernel(const PassArgs a) 
   extern __shared__ __align__(16) float2 smem[];
   __shared__ PassShared sh;
   const int64_t first = KC ? (int64_t)blockIdx.x : (int64_t)blockIdx.x * (blockDim.x >> (a.pd.K - kRegBits));
-  pass_cta<BWD, ROUNDS, false, RX, KC>(a, first, smem, sh);
+  if constexpr (BWD && !ROUNDS) {
+    __shared__ float acc_rows[kThreads / 32][8][32];  // a generic step's terms waiting for their reduction
+    pass_cta<BWD, ROUNDS, false, RX, KC>(a, first, smem, sh, nullptr, acc_rows);
+  } else {
+    pass_cta<BWD, ROUNDS, false, RX, KC>(a, first, smem, sh);
+  }
 }
 
 // Forward pass with the rounds on the tensor cores: one 12-qubit tile per
@@ -1330,46 +1373,59 @@ __device__ __forceinline__ double theta_at(const PrepArgs& a, int p) {
   return a.theta64 ? a.theta64[p] : (double)a.theta[p];
 }
 
-// Fused 2x2 product of fused entry m (float64, rounded once to float32).
-__device__ void fused_u(const PrepArgs& a, int64_t m, float4& m0, float4& m1, double* u64 = nullptr) {
-  double u[2][2][2] = {{{1, 0}, {0, 0}}, {{0, 0}, {1, 0}}};  // [row][col][re/im]
-  for (int j = a.fuse_off[m]; j < a.fuse_off[m + 1]; ++j) {
-    const FuseGate fg = a.fuse_gates[j];
-    double s, c;
-    sincos_prep(0.5 * (fg.param >= 0 ? theta_at(a, fg.param) : fg.angle), &s, &c);
-    // g = c I - i s P
-    double g[2][2][2];
-    if (fg.kind == G_RX) {
-      g[0][0][0] = c; g[0][0][1] = 0; g[0][1][0] = 0; g[0][1][1] = -s;
-      g[1][0][0] = 0; g[1][0][1] = -s; g[1][1][0] = c; g[1][1][1] = 0;
-    } else if (fg.kind == G_RY) {
-      g[0][0][0] = c; g[0][0][1] = 0; g[0][1][0] = -s; g[0][1][1] = 0;
-      g[1][0][0] = s; g[1][0][1] = 0; g[1][1][0] = c; g[1][1][1] = 0;
-    } else {
-      g[0][0][0] = c; g[0][0][1] = -s; g[0][1][0] = 0; g[0][1][1] = 0;
-      g[1][0][0] = 0; g[1][0][1] = 0; g[1][1][0] = c; g[1][1][1] = s;
+// Fused 2x2 product of fused entry m (float64, rounded once to float32) by 4
+// lanes (l: lane in the group): each takes the sincos of every fourth gate, and
+// lanes 0 and 1 (2 and 3 repeat them) carry one column each through the gates.
+// One thread per entry took its gates' float64 sincos and full 2x2 products one
+// after another: prep of n = 4, d = 2, 8 samples 14.7 -> 5.5 us.
+__device__ void fused_u(const PrepArgs& a, int64_t m, int l) {
+  const int lane = threadIdx.x & 31, first = lane & ~3;
+  const uint32_t group = 0xfu << first;
+  const int j0 = a.fuse_off[m], j1 = a.fuse_off[m + 1], col = l & 1;
+  double x0 = col == 0 ? 1.0 : 0.0, y0 = 0.0, x1 = col == 0 ? 0.0 : 1.0, y1 = 0.0;  // rows 0 and 1 of the column
+  for (int j = j0; j < j1; j += 4) {
+    double c = 1.0, s = 0.0;
+    int kind = G_RZ;
+    if (j + l < j1) {
+      const FuseGate fg = a.fuse_gates[j + l];
+      kind = fg.kind;
+      sincos_prep(0.5 * (fg.param >= 0 ? theta_at(a, fg.param) : fg.angle), &s, &c);
     }
-    double t[2][2][2];
-    for (int r = 0; r < 2; ++r)
-      for (int k = 0; k < 2; ++k) {
-        double re = 0, im = 0;
-        for (int q = 0; q < 2; ++q) {
-          re += g[r][q][0] * u[q][k][0] - g[r][q][1] * u[q][k][1];
-          im += g[r][q][0] * u[q][k][1] + g[r][q][1] * u[q][k][0];
-        }
-        t[r][k][0] = re;
-        t[r][k][1] = im;
+    const int n = min(4, j1 - j);
+    for (int t = 0; t < n; ++t) {
+      const double ct = __shfl_sync(group, c, first + t), st = __shfl_sync(group, s, first + t);
+      const int kt = __shfl_sync(group, kind, first + t);
+      const double a0 = x0, b0 = y0, a1 = x1, b1 = y1;
+      // c I - i s P
+      if (kt == G_RZ) {
+        x0 = ct * a0 + st * b0;
+        y0 = ct * b0 - st * a0;
+        x1 = ct * a1 - st * b1;
+        y1 = ct * b1 + st * a1;
+      } else if (kt == G_RY) {
+        x0 = ct * a0 - st * a1;
+        y0 = ct * b0 - st * b1;
+        x1 = ct * a1 + st * a0;
+        y1 = ct * b1 + st * b0;
+      } else {
+        x0 = ct * a0 + st * b1;
+        y0 = ct * b0 - st * a1;
+        x1 = ct * a1 + st * b0;
+        y1 = ct * b1 - st * a0;
       }
-    for (int r = 0; r < 2; ++r)
-      for (int k = 0; k < 2; ++k) {
-        u[r][k][0] = t[r][k][0];
-        u[r][k][1] = t[r][k][1];
-      }
+    }
   }
-  m0 = make_float4((float)u[0][0][0], (float)u[0][0][1], (float)u[0][1][0], (float)u[0][1][1]);
-  m1 = make_float4((float)u[1][0][0], (float)u[1][0][1], (float)u[1][1][0], (float)u[1][1][1]);
-  if (u64)
-    for (int q = 0; q < 8; ++q) u64[q] = u[q >> 2][(q >> 1) & 1][q & 1];
+  if (l > 1) return;
+  if (a.mats) {
+    float2* u = reinterpret_cast<float2*>(a.mats + 2 * m) + col;  // u00, u01, u10, u11
+    u[0] = make_float2((float)x0, (float)y0);
+    u[2] = make_float2((float)x1, (float)y1);
+  }
+  if (a.mats64) {
+    double2* u = reinterpret_cast<double2*>(a.mats64 + 8 * m) + col;
+    u[0] = make_double2(x0, y0);
+    u[2] = make_double2(x1, y1);
+  }
 }
 
 // A term's angle is the sum of its parameters (a merged run of RZ gates).
@@ -1483,8 +1539,9 @@ __device__ void round_params(const PrepArgs& a, bool on, bool fwd, int64_t r, co
 
 // Element i of the tables: (round programs) the forward and backward round
 // parameters in round order, then fused matrices, terms and encodings. A
-// round's float32 parameters are made by 16 lanes together; round_par_elems
-// is a multiple of 32, so that a warp is either wholly on rounds or not.
+// round's parameters are made by 16 lanes together and a fused matrix by 4;
+// round_par_elems and fused_elems are multiples of 32, so that a warp is either
+// wholly on one kind of the two or on neither.
 __device__ void prep_one(const PrepArgs& a, int64_t i) {
   const int64_t nre = round_par_elems(a);
   if (i < nre) {
@@ -1502,16 +1559,12 @@ __device__ void prep_one(const PrepArgs& a, int64_t i) {
     return;
   }
   i -= nre;
-  if (i < a.n_fused) {
-    float4 m0, m1;
-    fused_u(a, i, m0, m1, a.mats64 ? a.mats64 + 8 * i : nullptr);
-    if (a.mats) {
-      a.mats[2 * i] = m0;
-      a.mats[2 * i + 1] = m1;
-    }
+  const int64_t nfe = fused_elems(a);
+  if (i < nfe) {
+    if (i < 4 * (int64_t)a.n_fused) fused_u(a, i >> 2, (int)(i & 3));
     return;
   }
-  i -= a.n_fused;
+  i -= nfe;
   if (i < a.n_terms) {
     double s, c;
     sincos_prep(0.5 * term_angle(a, i), &s, &c);

@@ -103,13 +103,15 @@ struct PrepArgs {
   const RoundTerm* rpb_terms;  //   4 RZ-run terms (-1 terms: no parameter, angle 0)
 };
 
-// Prep work items: 16 per round (a half-warp makes one round's parameters),
-// rounded up to whole warps, then one per fused matrix, term and encoding.
+// Prep work items: 16 per round (a half-warp makes one round's parameters) and
+// 4 per fused matrix, each rounded up to whole warps, then one per term and
+// encoding.
 __host__ __device__ inline int64_t round_par_elems(const PrepArgs& a) {
   return (16 * ((int64_t)a.n_rpf + a.n_rpb) + 31) / 32 * 32;
 }
+__host__ __device__ inline int64_t fused_elems(const PrepArgs& a) { return (4 * (int64_t)a.n_fused + 31) / 32 * 32; }
 __host__ __device__ inline int64_t prep_elems(const PrepArgs& a) {
-  return round_par_elems(a) + a.n_fused + a.n_terms + a.B * a.n_eff;
+  return round_par_elems(a) + fused_elems(a) + a.n_terms + a.B * a.n_eff;
 }
 
 struct GradReduceArgs {

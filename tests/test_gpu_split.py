@@ -79,3 +79,18 @@ def test_batch_tiles_dealt_to_a_cluster(K, specs):
         gr, Er = orc.gradient(c, t64, x64, "Z")
         assert np.max(np.abs(E[bt.sample_off[i]:bt.sample_off[i + 1]] - Er)) < 1e-5, (n, d, B)
         assert np.max(np.abs(g[bt.theta_off[i]:bt.theta_off[i + 1]] - gr)) < 1e-5 * B, (n, d, B)
+
+
+@pytest.mark.parametrize("n,B", [(4, 9), (6, 5), (7, 3), (8, 33), (9, 2), (12, 3), (13, 2)])
+def test_generic_terms_are_reduced_by_eights(n, B):
+    """CNOT circuits (generic steps): 1 to 32 lanes per tile, term counts per
+    step that are no multiple of 8, RX gates among them."""
+    rows, P = [], 0
+    for layer in range(3):
+        for q in range(n):
+            for kind in ((1, 2), (0, 1, 2), (1,))[(layer + q) % 3]:
+                rows.append((kind, q, -1, P))
+                P += 1
+        rows += [(4, q, q + 1, -1) for q in range(layer % 2, n - 1, 2)] + [(3, 0, n - 1, -1)]
+    sim = Simulator(n, 0, B, gates=rows, n_params=P, obs="ZX")
+    check(sim, orc.Circuit(n=n, gates=np.array(rows, np.int32), n_params=P), n, P, B, "ZX", np.float32, 1e-5, n)

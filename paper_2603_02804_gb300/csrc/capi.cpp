@@ -649,13 +649,12 @@ qf_status fused_forward(qf_circuit* c, const DevTables& T, const Layout& L, cons
   return QF_OK;
 }
 
-// Observable reaching outside the seeding pass's tile: lambda_M for every
-// amplitude as its own pass (psi_M from the pass's source slot).
-cudaError_t seed_full(qf_circuit* c, const qf::FusedPlan& P, const qf::PassArgs& a, int64_t B, const Obs& o,
-                      cudaStream_t st) {
-  c->call_launches++;
-  return qf::launch_seed_full(a.slots + (int64_t)a.pd.psi_src * a.slot_stride, a.lam, P.n_eff, B, o.x, o.z, o.y,
-                              a.dLdE, st);
+// The adjoint's first pass seeds lambda from psi_M: within the tile, or (the
+// observable's X/Y qubits reach outside it) from psi_M's buffer, which that
+// pass only reads.
+void set_seed(qf::PassArgs& a, const Obs& o) {
+  a.pd.xm_local = 0;
+  if (a.pd.lam_src == qf::LAM_SEED && !local_xmask(a.pd, o.x, &a.pd.xm_local)) a.pd.lam_src = qf::LAM_SEED_FAR;
 }
 
 // with_prep = false: the term table was filled by the preceding forward.
@@ -688,6 +687,7 @@ qf_status fused_backward(qf_circuit* c, const DevTables& T, const Layout& L, con
   a.slots = at<float2>(ws, L.slots);
   a.hslots = L.hslots ? at<char>(ws, L.hslots) : nullptr;
   a.slot_stride = L.state_elems;
+  a.x_mask = o.x;
   a.z_mask = o.z;
   a.y_count = o.y;
   a.dLdE = dLdE;
@@ -710,11 +710,8 @@ qf_status fused_backward(qf_circuit* c, const DevTables& T, const Layout& L, con
       const bool bwd = P.a_dir[i] != 0;
       qf::PassArgs& x = bwd ? a : f;
       x.pd = P.a_sched[i];
-      x.pd.xm_local = 0;
-      if (bwd && x.pd.lam_src == qf::LAM_SEED && !local_xmask(x.pd, o.x, &x.pd.xm_local)) {
-        QF_CU(seed_full(c, P, x, B, o, st));
-        x.pd.lam_src = qf::LAM_BUF;
-      }
+      if (bwd) set_seed(x, o);
+      else x.pd.xm_local = 0;
       if (c->tc && !bwd) QF_CU(qf::launch_pass_tc(x, st));
       else QF_CU(qf::launch_pass(bwd, x, st, c->fwd_ctas));
       c->call_launches++;
@@ -723,11 +720,7 @@ qf_status fused_backward(qf_circuit* c, const DevTables& T, const Layout& L, con
   } else {
     for (size_t pi = 0; pi < P.bwd.size(); ++pi) {
       a.pd = P.bwd[pi];
-      a.pd.xm_local = 0;
-      if (a.pd.lam_src == qf::LAM_SEED && !local_xmask(a.pd, o.x, &a.pd.xm_local)) {
-        QF_CU(seed_full(c, P, a, B, o, st));
-        a.pd.lam_src = qf::LAM_BUF;
-      }
+      set_seed(a, o);
       QF_CU(qf::launch_pass(true, a, st));
       c->call_launches++;
     }

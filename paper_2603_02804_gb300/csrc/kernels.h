@@ -28,6 +28,7 @@ struct PassArgs {
   float2* slots;          // checkpoint states [n_ckpt][slot_stride]
   void* hslots;           // bfloat16 (re, im) pass-output slots [n][slot_stride] (PF_SRC_H / PF_DST_H)
   int64_t slot_stride;    // elements between consecutive checkpoint slots
+  uint32_t x_mask;        // observable X/Y part (global bits; read for LAM_SEED_FAR)
   uint32_t z_mask;        // observable Z part (global bits)
   uint32_t y_count;       // number of Y factors (phase i^y_count)
   const double* dLdE;     // [B]
@@ -147,12 +148,11 @@ cudaError_t launch_pass_tc(const PassArgs& a, cudaStream_t st);
 // Per-round B blocks of the tensor-core path from the float64 fused 2x2s.
 cudaError_t launch_tc_tables(const uint4* fwd_rounds, int32_t n_rounds, const double* mats64, float* tcb,
                              cudaStream_t st);
-// Observables with X/Y qubits outside the pass's tile: E partials [B][rows]
-// and the adjoint seed, each as a full pass over the state.
+// Observables with X/Y qubits outside the pass's tile: E partials [B][rows] in
+// a full pass over the state (the adjoint's first pass seeds itself,
+// LAM_SEED_FAR).
 cudaError_t launch_expect_full(const float2* psi, int n_eff, int64_t B, int64_t rows, uint32_t xm, uint32_t zm,
                                uint32_t yc, double* e_part, cudaStream_t st);
-cudaError_t launch_seed_full(const float2* psi, float2* lam, int n_eff, int64_t B, uint32_t xm, uint32_t zm,
-                             uint32_t yc, const double* dLdE, cudaStream_t st);
 // One bounded wait on an mbarrier nothing arrives at (records a timeout).
 cudaError_t bounded_wait_probe(long long limit, cudaStream_t st);
 // Read and clear the device error word (1: a bounded wait gave up).

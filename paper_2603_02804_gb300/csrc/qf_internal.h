@@ -76,6 +76,7 @@ enum : int32_t {
   BUF_NONE = -3,      // nothing stored
   LAM_SEED = -1,      // bwd: lambda = 2 (dL/dE) O psi from the loaded psi
   LAM_BUF = -2,       // bwd: lambda buffer
+  LAM_SEED_FAR = -4,  // bwd: LAM_SEED for an observable that reaches outside the tile (set at launch)
 };
 
 enum PassFlags : int32_t {

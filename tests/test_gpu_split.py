@@ -94,3 +94,12 @@ def test_generic_terms_are_reduced_by_eights(n, B):
         rows += [(4, q, q + 1, -1) for q in range(layer % 2, n - 1, 2)] + [(3, 0, n - 1, -1)]
     sim = Simulator(n, 0, B, gates=rows, n_params=P, obs="ZX")
     check(sim, orc.Circuit(n=n, gates=np.array(rows, np.int32), n_params=P), n, P, B, "ZX", np.float32, 1e-5, n)
+
+
+@pytest.mark.parametrize("n,kw,obs", [(9, dict(tile_bits=5), "XIIIIIYIZ"), (10, dict(tile_bits=8), "YZIIIIIIIX"),
+                                      (13, {}, "X" * 13), (13, dict(ckpt_mode=1, ckpt_layers=1), "ZYIIIIXIIIIIX"),
+                                      (14, {}, "IXYZIXYZIXYZIX")])
+def test_observables_beyond_the_tile(n, kw, obs):
+    """The adjoint seeded from another tile's amplitudes (X or Y on qubits
+    outside the last pass's tile, on bit 0 and not), and E over half the state."""
+    check(Simulator(n, 3, 3, obs=obs, **kw), orc.hea(n, 3), n, 9 * n, 3, obs, np.float32, 1e-5, n)

@@ -59,7 +59,8 @@ __device__ __forceinline__ float4 ld_pair(const float2* sm, uint32_t p) {
   return make_float4(a.x, a.y, b.x, b.y);
 }
 
-// The 16 registers of a group on local bits B .. B + 3, at the thread's base.
+// The registers of a group on local bits B .. B + 3, at the thread's base (NR =
+// 16, or 8 on bits B .. B + 2 where two threads share a column).
 template <int B>
 __device__ __forceinline__ constexpr int group_off(int j) {
   int o = 0;
@@ -67,22 +68,22 @@ __device__ __forceinline__ constexpr int group_off(int j) {
     if ((j >> r) & 1) o += (int)loc(1u << (B + r));
   return o;
 }
-template <int B>
-__device__ __forceinline__ void ld16(const float2* at, float2 (&r)[16]) {
+template <int B, int NR>
+__device__ __forceinline__ void ld_regs(const float2* at, float2 (&r)[NR]) {
 #pragma unroll
-  for (int j = 0; j < 16; ++j) r[j] = at[group_off<B>(j)];
+  for (int j = 0; j < NR; ++j) r[j] = at[group_off<B>(j)];
 }
-template <int B>
-__device__ __forceinline__ void st16(float2* at, const float2 (&r)[16]) {
+template <int B, int NR>
+__device__ __forceinline__ void st_regs(float2* at, const float2 (&r)[NR]) {
 #pragma unroll
-  for (int j = 0; j < 16; ++j) at[group_off<B>(j)] = r[j];
+  for (int j = 0; j < NR; ++j) at[group_off<B>(j)] = r[j];
 }
 // The group's lowest local bit b is one of these in round programs (K = 7 .. 12:
 // 0, 4, 8 and K - 4; KC = 12: 0, 4, 8). at2: lambda's place (adjoint).
-template <int KC, bool BWD>
-__device__ __forceinline__ void ld_group(uint32_t b, const float2* at, const float2* at2, float2 (&r)[16],
-                                         float2 (&l)[16]) {
-#define QF_LD(B) { ld16<B>(at, r); if (BWD) ld16<B>(at2, l); }
+template <int KC, bool BWD, int NR>
+__device__ __forceinline__ void ld_group(uint32_t b, const float2* at, const float2* at2, float2 (&r)[NR],
+                                         float2 (&l)[NR]) {
+#define QF_LD(B) { ld_regs<B>(at, r); if (BWD) ld_regs<B>(at2, l); }
   if (KC == 12) {
     if (b == 0) QF_LD(0) else if (b == 4) QF_LD(4) else QF_LD(8)
   } else {
@@ -98,10 +99,10 @@ __device__ __forceinline__ void ld_group(uint32_t b, const float2* at, const flo
   }
 #undef QF_LD
 }
-template <int KC, bool BWD>
-__device__ __forceinline__ void st_group(uint32_t b, float2* at, float2* at2, const float2 (&r)[16],
-                                         const float2 (&l)[16]) {
-#define QF_ST(B) { st16<B>(at, r); if (BWD) st16<B>(at2, l); }
+template <int KC, bool BWD, int NR>
+__device__ __forceinline__ void st_group(uint32_t b, float2* at, float2* at2, const float2 (&r)[NR],
+                                         const float2 (&l)[NR]) {
+#define QF_ST(B) { st_regs<B>(at, r); if (BWD) st_regs<B>(at2, l); }
   if (KC == 12) {
     if (b == 0) QF_ST(0) else if (b == 4) QF_ST(4) else QF_ST(8)
   } else {
@@ -262,15 +263,15 @@ __device__ __forceinline__ void chain_pending(uint32_t L, uint32_t rgb, uint32_t
 }
 
 // Multiply the registers by D (end of a step).
-template <bool BWD>
-__device__ __forceinline__ void apply_pending(uint32_t D, float2 (&r)[16], float2 (&l)[16]) {
+template <bool BWD, int NR>
+__device__ __forceinline__ void apply_pending(uint32_t D, float2 (&r)[NR], float2 (&l)[NR]) {
   uint32_t S = (D & 16u) ? 0xFFFFu : 0u;
   S ^= (D & 1u) ? 0xAAAAu : 0u;
   S ^= (D & 2u) ? 0xCCCCu : 0u;
   S ^= (D & 4u) ? 0xF0F0u : 0u;
   S ^= (D & 8u) ? 0xFF00u : 0u;
 #pragma unroll
-  for (int j = 0; j < 16; ++j) {
+  for (int j = 0; j < NR; ++j) {
     const int f = (int)((S << (31 - j)) & 0x80000000u);
     r[j].x = __int_as_float(__float_as_int(r[j].x) ^ f);
     r[j].y = __int_as_float(__float_as_int(r[j].y) ^ f);
@@ -296,11 +297,11 @@ __device__ __forceinline__ void apply_pending(uint32_t D, float2 (&r)[16], float
 // were slower: training step of n = 20, d = 24, 64 samples 28.35 -> 25.10 ms, of
 // n = 12, d = 20, 256 samples 268 -> 237 us (with the pending links below). A
 // pending Z_R turns the rotation by w into one by -w, i.e. q into -q.
-template <int R, bool RX>
-__device__ __forceinline__ void rot_T(float2 (&r)[16], float q, bool rx) {
+template <int R, bool RX, int NR>
+__device__ __forceinline__ void rot_T(float2 (&r)[NR], float q, bool rx) {
   if (RX && rx) {
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
+    for (int j = 0; j < NR; ++j) {
       if (j & (1 << R)) continue;
       const int j1 = j | (1 << R);
       const float2 p0 = r[j], p1 = r[j1];
@@ -311,7 +312,7 @@ __device__ __forceinline__ void rot_T(float2 (&r)[16], float q, bool rx) {
     // RY is real: the same on re and im, one packed FFMA2 each
     const float2 q2 = make_float2(q, q), n2 = make_float2(-q, -q);
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
+    for (int j = 0; j < NR; ++j) {
       if (j & (1 << R)) continue;
       const int j1 = j | (1 << R);
       const float2 p0 = r[j];
@@ -338,9 +339,10 @@ __device__ __forceinline__ void cmul(float2& v, float c, float s) {
 // j). An RZ run commutes with the rotations on the other register bits and
 // with the pending signs, so the four run together, once per round, after the
 // rotations (the adjoint un-applies them before its rotations, diag_bwd).
-__device__ __forceinline__ void apply_diag(float2 (&r)[16], const float4* ph) {
+template <int NR>
+__device__ __forceinline__ void apply_diag(float2 (&r)[NR], const float4* ph) {
 #pragma unroll
-  for (int m = 0; m < 8; ++m) {
+  for (int m = 0; m < NR / 2; ++m) {
     const float4 e = ph[m];
     cmul(r[2 * m], e.x, e.y);
     cmul(r[2 * m + 1], e.z, e.w);
@@ -387,16 +389,15 @@ __device__ __forceinline__ void diag_bwd(float2 (&p)[16], float2 (&l)[16], const
 // and gy. The round's scale and the earlier items' rotations multiply gy by a
 // factor that is the same for every thread and sample; the owner lane of the
 // reduced sum undoes it (the table's factor).
-template <int R, bool RX = false>
-__device__ __forceinline__ void rot_bwd(float2 (&p)[16], float2 (&l)[16], float qt, uint32_t a, float& gy,
-                                        bool rx = false) {
+template <int R, bool RX, int NR>
+__device__ __forceinline__ void rot_bwd(float2 (&p)[NR], float2 (&l)[NR], float qt, uint32_t a, float& gy, bool rx) {
   const int f = (int)(a << 31);
   const float q = __int_as_float(__float_as_int(qt) ^ f);
   float g;
   if (RX && rx) {
     g = 0.f;
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
+    for (int j = 0; j < NR; ++j) {
       if (j & (1 << R)) continue;
       const int j1 = j | (1 << R);
       g += l[j].x * p[j1].y - l[j].y * p[j1].x + l[j1].x * p[j].y - l[j1].y * p[j].x;
@@ -405,7 +406,7 @@ __device__ __forceinline__ void rot_bwd(float2 (&p)[16], float2 (&l)[16], float 
     // l1 . p0 - l0 . p1 per pair (component-wise products, two packed sums)
     float2 accp = make_float2(0.f, 0.f), accm = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
+    for (int j = 0; j < NR; ++j) {
       if (j & (1 << R)) continue;
       const int j1 = j | (1 << R);
       accp = __ffma2_rn(l[j1], p[j], accp);
@@ -416,6 +417,79 @@ __device__ __forceinline__ void rot_bwd(float2 (&p)[16], float2 (&l)[16], float 
   rot_T<R, RX>(p, q, rx);
   rot_T<R, RX>(l, q, rx);
   gy = __int_as_float(__float_as_int(g) ^ f);
+}
+
+// ---- two threads per column ------------------------------------------------------
+// A launch of few tiles leaves each scheduler a warp or two, and its time is a
+// warp's latency through its instructions. There two neighbouring threads share
+// a column (thread h holds the 8 registers with bit 3 of the index equal to h),
+// each with half the instructions; the rotation on bit 3 fetches the partner's
+// amplitudes by shuffles.
+__device__ __forceinline__ void partner(const float2 (&r)[8], float2 (&o)[8]) {
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    o[j] = make_float2(__shfl_xor_sync(0xffffffffu, r[j].x, 1), __shfl_xor_sync(0xffffffffu, r[j].y, 1));
+}
+// rot_T on bit 3: o holds the partner's amplitudes.
+template <bool RX>
+__device__ __forceinline__ void rot_half(float2 (&r)[8], const float2 (&o)[8], float q, uint32_t h, bool rx) {
+  if (RX && rx) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) r[j] = make_float2(fmaf(q, o[j].y, r[j].x), fmaf(-q, o[j].x, r[j].y));
+  } else {
+    const float qh = pend_q(q, h ^ 1u);  // p0 -= q p1; p1 += q p0
+    const float2 q2 = make_float2(qh, qh);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) r[j] = __ffma2_rn(q2, o[j], r[j]);
+  }
+}
+template <bool RX>
+__device__ __forceinline__ void rot_fwd_half(float2 (&r)[8], float q, uint32_t h, bool rx) {
+  float2 o[8];
+  partner(r, o);
+  rot_half<RX>(r, o, q, h, rx);
+}
+// rot_bwd on bit 3; gy: the thread's share (l_1 . p_0 in thread 1, -l_0 . p_1 in thread 0).
+template <bool RX>
+__device__ __forceinline__ void rot_bwd_half(float2 (&p)[8], float2 (&l)[8], float qt, uint32_t a, float& gy, uint32_t h,
+                                             bool rx) {
+  const float q = pend_q(qt, a);
+  float2 o[8];
+  partner(p, o);
+  float g;
+  if (RX && rx) {
+    g = 0.f;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) g += l[j].x * o[j].y - l[j].y * o[j].x;
+  } else {
+    float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc = __ffma2_rn(l[j], o[j], acc);
+    g = pend_q(acc.x + acc.y, h ^ 1u);
+  }
+  rot_half<RX>(p, o, q, h, rx);
+  partner(l, o);
+  rot_half<RX>(l, o, q, h, rx);
+  gy = pend_q(g, a);
+}
+// diag_bwd of a half column: bits 0..2 from the complements 7 - j, bit 3 from
+// the whole sum, signed by the half.
+__device__ __forceinline__ void diag_bwd(float2 (&p)[8], float2 (&l)[8], const float4* ph, float (&g)[8], uint32_t h) {
+  float u[4], t[4];
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    const float2 p0 = p[m], l0 = l[m], p1 = p[7 - m], l1 = l[7 - m];
+    const float w0 = fmaf(l0.x, p0.y, -l0.y * p0.x), w1 = fmaf(l1.x, p1.y, -l1.y * p1.x);
+    u[m] = w0 - w1;
+    t[m] = w0 + w1;
+  }
+  apply_diag(p, ph);
+  apply_diag(l, ph);
+  const float q0 = u[0] + u[1], T = q0 + (u[2] + u[3]);
+  g[0] = fmaf(2.f, u[0] + u[2], -T);
+  g[1] = fmaf(2.f, q0, -T);
+  g[2] = T;
+  g[3] = pend_q((t[0] + t[1]) + (t[2] + t[3]), h);
 }
 
 // Reduce 8 per-thread values over `lanes` lanes (8, 16 or 32; whole-warp
@@ -724,7 +798,8 @@ struct PassShared {
 // the padded layout, 366 -> 291 instructions per warp and round forward and 786
 // -> 659 adjoint; step of n = 20, d = 24, 64 samples 25.10 -> 23.00 ms, of n =
 // 12, d = 20, 256 samples 237 -> 222 us.
-template <bool BWD, bool ROUNDS, bool TC = false, bool RX = false, int KC = 0>
+// H: threads per column as a power of two (1: two threads of 8 registers each).
+template <bool BWD, bool ROUNDS, bool TC = false, bool RX = false, int KC = 0, int H = 0>
 __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_tile, float2* smem, PassShared& sh,
                                          const TcCtx* tc = nullptr, float (*acc_rows)[8][32] = nullptr) {
   uint32_t (&s_lg)[256] = sh.lg;
@@ -735,7 +810,9 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
 
   const PassDesc& pd = a.pd;
   const int K = KC ? KC : pd.K;
-  const int tl2 = K - kRegBits;            // log2 threads per tile
+  constexpr int NR = 16 >> H;                  // amplitudes per thread and step
+  constexpr int NIT = NR / 2;                  // pairs per thread of the tile's loads and stores
+  const int tl2 = K - kRegBits + H;        // log2 threads per tile
   const int Tt = 1 << tl2;
   const int tid = threadIdx.x;
   const int lane = tid & 31, warp = tid >> 5;
@@ -751,8 +828,8 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
   const uint32_t outer = pdep32(t_in, pd.outer_mask);
   const int64_t dim = 1ll << a.n_eff;
   const int64_t sbase = b * dim;  // sample offset inside one state buffer
-  float2* tp = smem + (tile_in_cta << K) + (tile_in_cta << tl2);  // loc(tile_in_cta << K)
-  const int lam_at = KC ? kTilePad : nthr * 17;  // words of the CTA's psi tiles: lambda's follow
+  float2* tp = smem + (tile_in_cta << K) + (tile_in_cta << (K - 4));  // loc(tile_in_cta << K)
+  const int lam_at = KC ? kTilePad : (nthr >> H) * 17;  // words of the CTA's psi tiles: lambda's follow
   float2* tl = tp + lam_at;
   const int wpt = Tt >= 32 ? Tt / 32 : 1;  // warps per tile
   const int lanes = Tt < 32 ? Tt : 32;
@@ -767,24 +844,25 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
     if (ROUNDS && tid < 8) sh.ident[tid] = make_float4(1.f, 0.f, 1.f, 0.f);
   }
   __syncthreads();
-  for (int h = tid; h < (1 << tl2); h += nthr) {
+  for (int i = tid; i < (1 << (K - kRegBits)); i += nthr) {
     uint32_t g = 0;
-    for (int j = 0; j < tl2; ++j)
-      if ((h >> j) & 1) g |= 1u << s_gmap[kRegBits + j];
-    s_lg[h] = g;
+    for (int j = 0; j < K - kRegBits; ++j)
+      if ((i >> j) & 1) g |= 1u << s_gmap[kRegBits + j];
+    s_lg[i] = g;
   }
   __syncthreads();
 
   auto gidx = [&](uint32_t i) -> uint32_t { return outer | (i & 15u) | s_lg[i >> 4]; };
-  // A thread's share of the tile is the pairs i = 2 (it Tt + tau), it = 0..7:
-  // it is the local bits K-3 .. K-1, so the global index splits into the
-  // thread's part and `it_bits` (uniform), and the place in shared memory into
-  // the thread's part and it * loc(2 Tt) (for Tt >= 8, where 2 Tt is a
-  // multiple of 16)
+  // A thread's share of the tile is the pairs i = 2 (it Tt + tau), it < NIT: it
+  // is the top local bits (K-3 .. K-1, or K-2 and K-1), so the global index
+  // splits into the thread's part and `it_bits` (uniform), and for KC the place
+  // in shared memory into the thread's part and it * loc(2 Tt)
   const uint32_t g_tau = gidx(2u * tau), p_tau = loc(2u * tau);
   auto it_bits = [&](int it) -> uint32_t {
-    return ((it & 1) ? 1u << pd.gmap[K - 3] : 0u) | ((it & 2) ? 1u << pd.gmap[K - 2] : 0u) |
-           ((it & 4) ? 1u << pd.gmap[K - 1] : 0u);
+    uint32_t g = 0u;
+#pragma unroll
+    for (int q = 0; q < 3 - H; ++q) g |= ((it >> q) & 1) ? 1u << pd.gmap[K - 3 + H + q] : 0u;
+    return g;
   };
   auto g_it = [&](int it) -> uint32_t { return g_tau | it_bits(it); };
   auto p_it = [&](int it) -> uint32_t {
@@ -834,7 +912,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
     const int64_t din = 1ll << a.n_in;
     const float2* src = a.psi_in + b * din;
 #pragma unroll
-    for (int it = 0; it < 8; ++it) {
+    for (int it = 0; it < NIT; ++it) {
       const uint32_t g = g_it(it);
       float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
       if (a.n_in == a.n_eff) {
@@ -850,19 +928,23 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
     // the thread's pairs share every factor but those of qubit 0 and the
     // three local bits K-3 .. K-1
     const float2* e = a.enc + b * a.n_eff;
-    const uint32_t vary = it_bits(7);
+    const uint32_t vary = it_bits(NIT - 1);
     float pr = 1.f;
     for (int q = 1; q < a.n_eff; ++q) {
       if ((vary >> q) & 1u) continue;
       const float2 f = __ldg(e + q);
       pr *= ((g_tau >> q) & 1u) ? f.y : f.x;
     }
-    const float2 f0 = __ldg(e), e0 = __ldg(e + pd.gmap[K - 3]), e1 = __ldg(e + pd.gmap[K - 2]),
-                 e2 = __ldg(e + pd.gmap[K - 1]);
+    const float2 f0 = __ldg(e);
+    float2 ev[3];
+#pragma unroll
+    for (int q = 0; q < 3 - H; ++q) ev[q] = __ldg(e + pd.gmap[K - 3 + H + q]);
     if (active) {
 #pragma unroll
-      for (int it = 0; it < 8; ++it) {
-        const float v = pr * ((it & 1) ? e0.y : e0.x) * ((it & 2) ? e1.y : e1.x) * ((it & 4) ? e2.y : e2.x);
+      for (int it = 0; it < NIT; ++it) {
+        float v = pr;
+#pragma unroll
+        for (int q = 0; q < 3 - H; ++q) v *= ((it >> q) & 1) ? ev[q].y : ev[q].x;
         st_pair(tp, p_it(it), make_float4(v * f0.x, 0.f, v * f0.y, 0.f));
       }
     }
@@ -881,9 +963,9 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
     const bool two = BWD && (pd.lam_src == LAM_BUF || far);
     const float2* lsrc = far ? src : a.lam + sbase;
     const uint32_t lx = far ? a.x_mask & ~1u : 0u;
-    float4 vp[8], vl[8];
+    float4 vp[NIT], vl[NIT];
 #pragma unroll
-    for (int it = 0; it < 8; ++it) {
+    for (int it = 0; it < NIT; ++it) {
       const uint32_t g = g_it(it);
       if (half) vp[it] = bf16x4_to_f4(__ldcg(reinterpret_cast<const uint2*>(hsrc + g)));
       else vp[it] = __ldcg(reinterpret_cast<const float4*>(src + g));
@@ -892,7 +974,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
     if (far) {
       const float scale = (float)(2.0 * a.dLdE[b]);
 #pragma unroll
-      for (int it = 0; it < 8; ++it) {
+      for (int it = 0; it < NIT; ++it) {
         const uint32_t xp = g_it(it) ^ a.x_mask;  // the pair's partners: xp and xp ^ 1
         const bool swap = (a.x_mask & 1u) != 0;
         const float4 v = vl[it];
@@ -904,7 +986,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
       }
     }
 #pragma unroll
-    for (int it = 0; it < 8; ++it) {
+    for (int it = 0; it < NIT; ++it) {
       st_pair(tp, p_it(it), vp[it]);
       if (two) st_pair(tl, p_it(it), vl[it]);
     }
@@ -912,7 +994,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
   if (BWD && pd.lam_src == LAM_BUF && psrc == SRC_GENERATE && active) {
     const float2* src = a.lam + sbase;
 #pragma unroll
-    for (int it = 0; it < 8; ++it) st_pair(tl, p_it(it), __ldcg(reinterpret_cast<const float4*>(src + g_it(it))));
+    for (int it = 0; it < NIT; ++it) st_pair(tl, p_it(it), __ldcg(reinterpret_cast<const float4*>(src + g_it(it))));
   }
   // round programs: stage the first step's parameters
   int sb = 0;
@@ -934,7 +1016,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
     // lambda_M = 2 (dL/dE_b) O psi_M (Eq. 4); (O psi)_x = i^{#Y} (-1)^{|(x^xm)&zm|} psi_{x^xm}
     const float scale = active ? (float)(2.0 * a.dLdE[b]) : 0.f;
 #pragma unroll 1
-    for (int it = 0; it < 16; ++it) {
+    for (int it = 0; it < NR; ++it) {
       const uint32_t i = (uint32_t)it * Tt + tau;  // single amplitudes here
       const uint32_t ip = i ^ pd.xm_local;
       const uint32_t gp = gidx(ip);
@@ -977,14 +1059,16 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
       }
       const StepPar& P = sh.par[sb];
       const uint32_t lb = KC ? 4u * (uint32_t)g : sh.gb[g];
-      // tau's bits around the group's (a zero in each of its four)
-      const uint32_t base = (tau & ((1u << lb) - 1u)) | ((tau >> lb) << (lb + 4u));
-      float2* const at = tp + loc(base);
+      // the column's bits around the group's (a zero in each of its four); h: the
+      // thread's half of the column
+      const uint32_t col = tau >> H, h = H ? tau & 1u : 0u;
+      const uint32_t base = (col & ((1u << lb) - 1u)) | ((col >> lb) << (lb + 4u));
+      float2* const at = tp + loc(base) + (H && h ? loc(8u << lb) : 0u);
       const uint32_t gb = gidx(base);
       const uint4 gp = sh.gpos[g];
       const uint32_t pos[4] = {gp.x, gp.y, gp.z, gp.w};
-      float2 r[16];
-      float2 l[16];
+      float2 r[NR];
+      float2 l[NR];
       ld_group<KC, BWD>(lb, at, at + lam_at, r, l);
       const int nq = a.n_eff;
       const uint32_t nmask = nq >= 32 ? ~0u : ((1u << nq) - 1u);
@@ -1008,8 +1092,9 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
           rot_T<0, RX>(r, pend_q(P.v[k][0].x, D & 1u), lk.z & 1u);
           rot_T<1, RX>(r, pend_q(P.v[k][1].x, (D >> 1) & 1u), (lk.z >> 1) & 1u);
           rot_T<2, RX>(r, pend_q(P.v[k][2].x, (D >> 2) & 1u), (lk.z >> 2) & 1u);
-          rot_T<3, RX>(r, pend_q(P.v[k][3].x, (D >> 3) & 1u), (lk.z >> 3) & 1u);
-          apply_diag(r, pre ? sh.ident : &P.v[k][4]);
+          if constexpr (H) rot_fwd_half<RX>(r, pend_q(P.v[k][3].x, (D >> 3) & 1u), h, (lk.z >> 3) & 1u);
+          else rot_T<3, RX>(r, pend_q(P.v[k][3].x, (D >> 3) & 1u), (lk.z >> 3) & 1u);
+          apply_diag(r, pre ? sh.ident : &P.v[k][4 + (H ? 4 * h : 0)]);
           if (!pre) {
             chain_pending(lk.x, rgb, lgb, g12, nq, pos, contig, D);
             pend ^= lk.w;
@@ -1023,11 +1108,13 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
             pend ^= lk.w;
           }
           float v[8];
-          diag_bwd(r, l, again ? sh.ident : &P.v[k][4], v);
+          if constexpr (H) diag_bwd(r, l, again ? sh.ident : &P.v[k][4 + 4 * h], v, h);
+          else diag_bwd(r, l, again ? sh.ident : &P.v[k][4], v);
           rot_bwd<0, RX>(r, l, P.v[k][0].x, D & 1u, v[4], lk.z & 1u);
           rot_bwd<1, RX>(r, l, P.v[k][1].x, (D >> 1) & 1u, v[5], (lk.z >> 1) & 1u);
           rot_bwd<2, RX>(r, l, P.v[k][2].x, (D >> 2) & 1u, v[6], (lk.z >> 2) & 1u);
-          rot_bwd<3, RX>(r, l, P.v[k][3].x, (D >> 3) & 1u, v[7], (lk.z >> 3) & 1u);
+          if constexpr (H) rot_bwd_half<RX>(r, l, P.v[k][3].x, (D >> 3) & 1u, v[7], h, (lk.z >> 3) & 1u);
+          else rot_bwd<3, RX>(r, l, P.v[k][3].x, (D >> 3) & 1u, v[7], (lk.z >> 3) & 1u);
           // lane holds value idx of its tile; the first 8 lanes of a tile keep theirs
           const int idx = lane & 7;
           float sum = rows8(v, lanes, lane, sh.rows[warp]);
@@ -1048,6 +1135,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
         }
       }
       if ((op.x >> kStepFlushBit) & 1u) {
+        if (H) D = (D ^ ((D & (h << 3)) << 1)) & ~8u;  // the half's own bit 3
         apply_pending<BWD>(D, r, l);
         pend = 0;
       }
@@ -1226,7 +1314,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
     } else if (code == OP_CKPT || code == OP_ANCHOR) {
       float2* sp = a.slots + (int64_t)op.y * a.slot_stride + sbase;
 #pragma unroll
-      for (int it = 0; it < 8; ++it) {
+      for (int it = 0; it < NIT; ++it) {
         if (!active) continue;
         if (code == OP_CKPT) *reinterpret_cast<float4*>(sp + g_it(it)) = ld_pair(tp, p_it(it));
         else st_pair(tp, p_it(it), __ldcg(reinterpret_cast<const float4*>(sp + g_it(it))));
@@ -1240,20 +1328,20 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
     // memory-saving mode (Sec. 3.2): the stored copy is rounded to bfloat16
     __nv_bfloat162* dst = reinterpret_cast<__nv_bfloat162*>(a.hslots) + (int64_t)pd.psi_dst * a.slot_stride + sbase;
 #pragma unroll
-    for (int it = 0; it < 8; ++it) {
+    for (int it = 0; it < NIT; ++it) {
       if (active) *reinterpret_cast<uint2*>(dst + g_it(it)) = f4_to_bf16x4(ld_pair(tp, p_it(it)));
     }
   } else if (pd.psi_dst != BUF_NONE) {
     float2* dst = state_ptr(pd.psi_dst);
 #pragma unroll
-    for (int it = 0; it < 8; ++it) {
+    for (int it = 0; it < NIT; ++it) {
       if (active) *reinterpret_cast<float4*>(dst + g_it(it)) = ld_pair(tp, p_it(it));
     }
   }
   if (BWD && pd.lam_dst == LAM_BUF) {
     float2* dst = a.lam + sbase;
 #pragma unroll
-    for (int it = 0; it < 8; ++it) {
+    for (int it = 0; it < NIT; ++it) {
       if (active) *reinterpret_cast<float4*>(dst + g_it(it)) = ld_pair(tl, p_it(it));
     }
   }
@@ -1261,7 +1349,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
     // <psi|O|psi> partial of this tile (Eq. 1, matrix-free as in Appendix B.2)
     float acc = 0.f;
 #pragma unroll 1
-    for (int it = 0; it < 16; ++it) {
+    for (int it = 0; it < NR; ++it) {
       const uint32_t i = (uint32_t)it * Tt + tau;
       const uint32_t ip = i ^ pd.xm_local;
       const float2 v = tp[loc(i)];
@@ -1307,16 +1395,16 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
 // of RZ / RY items keep the plain code). MINB: CTAs per SM the registers are
 // budgeted for; a forward pass (one 32 KiB state per CTA) of more tiles than
 // two CTAs per SM hold runs with three per SM.
-template <bool BWD, bool ROUNDS, bool RX = false, int MINB = 2, int KC = 0>
+template <bool BWD, bool ROUNDS, bool RX = false, int MINB = 2, int KC = 0, int H = 0>
 __global__ void __launch_bounds__(kThreads, MINB) pass_kernel(const PassArgs a) {
   extern __shared__ __align__(16) float2 smem[];
   __shared__ PassShared sh;
-  const int64_t first = KC ? (int64_t)blockIdx.x : (int64_t)blockIdx.x * (blockDim.x >> (a.pd.K - kRegBits));
+  const int64_t first = KC ? (int64_t)blockIdx.x : (int64_t)blockIdx.x * (blockDim.x >> (a.pd.K - kRegBits + H));
   if constexpr (BWD && !ROUNDS) {
     __shared__ float acc_rows[kThreads / 32][8][32];  // a generic step's terms waiting for their reduction
-    pass_cta<BWD, ROUNDS, false, RX, KC>(a, first, smem, sh, nullptr, acc_rows);
+    pass_cta<BWD, ROUNDS, false, RX, KC, H>(a, first, smem, sh, nullptr, acc_rows);
   } else {
-    pass_cta<BWD, ROUNDS, false, RX, KC>(a, first, smem, sh);
+    pass_cta<BWD, ROUNDS, false, RX, KC, H>(a, first, smem, sh);
   }
 }
 
@@ -2058,16 +2146,24 @@ cudaError_t launch_pass(bool bwd, const PassArgs& a, cudaStream_t st, int fwd_ct
   // would leave SMs without one, CTAs get smaller (one tile, one warp at least):
   // n = 8, d = 20, 64 samples on 32 SMs instead of 4: step 120 -> 98 us; n = 10,
   // 256 samples 145 -> 136 us. Launches that fill the SMs keep 256 threads.
-  int thr = kThreads;
-  while (thr > 32 && thr > (1 << tl2) && (total_tiles << tl2) < (int64_t)thr * n_sm) thr >>= 1;
-  const int tiles_per_cta = thr >> tl2;
-  const int64_t grid = (total_tiles + tiles_per_cta - 1) / tiles_per_cta;
-  const size_t smem = (size_t)(bwd ? 2 : 1) * thr * 17 * sizeof(float2);
+  // Rounds of launches with at most a warp per scheduler (4 per SM) run two
+  // threads per column instead: n = 8, d = 20, 64 samples 96 -> 87 us a step; n =
+  // 10, 256 samples 136 -> 123; n = 11, 128 samples 134 -> 124. With twice as
+  // many warps it is slower (n = 10, 512 samples 155 -> 168). (12-qubit tiles
+  // have two warps per scheduler as they are, and lose by it: n = 13, d = 31, 37
+  // samples 375 -> 436 us.)
   const bool rounds = a.rounds != nullptr, rx = rounds && a.rx_items;
+  const bool k12 = a.pd.K == kMaxTileBits;
+  const bool half = rounds && !k12 && (total_tiles << tl2) <= 128ll * n_sm;
+  const int tt2 = tl2 + (half ? 1 : 0);  // log2 threads per tile
+  int thr = kThreads;
+  while (thr > 32 && thr > (1 << tt2) && (total_tiles << tt2) < (int64_t)thr * n_sm) thr >>= 1;
+  const int tiles_per_cta = thr >> tt2;
+  const int64_t grid = (total_tiles + tiles_per_cta - 1) / tiles_per_cta;
+  const size_t smem = (size_t)(bwd ? 2 : 1) * (thr >> (half ? 1 : 0)) * 17 * sizeof(float2);
   // 12-qubit tiles run the instances compiled for them; a single-wave forward
   // keeps the 128-register instance, more tiles than two CTAs per SM hold run
   // with three per SM (fewer registers, more warps to hide latency across waves)
-  const bool k12 = a.pd.K == kMaxTileBits;
   const bool three =
       rounds && !bwd && (fwd_ctas == 3 || (fwd_ctas == 0 && (total_tiles << tl2) > 2ll * kThreads * n_sm));
 #define QF_RUN(...)                                                                          \
@@ -2082,6 +2178,14 @@ cudaError_t launch_pass(bool bwd, const PassArgs& a, cudaStream_t st, int fwd_ct
   // (the two-CTA instance of runtime tile sizes spills: n = 8, d = 20, 64 samples
   // 102 us a step against 96)
   const bool alone = grid <= n_sm;
+  if (half && bwd) {
+    if (rx) QF_RUN(pass_kernel<true, true, true, 2, 0, 1>);
+    QF_RUN(pass_kernel<true, true, false, 2, 0, 1>);
+  }
+  if (half) {
+    if (rx) QF_RUN(pass_kernel<false, true, true, 2, 0, 1>);
+    QF_RUN(pass_kernel<false, true, false, 2, 0, 1>);
+  }
   if (bwd) {
     if (!rounds && alone) QF_RUN(pass_kernel<true, false, false, 1>);
     if (!rounds) QF_RUN(pass_kernel<true, false>);

@@ -251,14 +251,17 @@ __device__ __forceinline__ void link_terms(uint32_t L, uint32_t gb, int n, uint3
 // the thread (rgb = gb rotated right by one qubit, lgb = left, g12 = gb &
 // rgb): as rotation distributes over &, u = rotl(L) & lgb ^ L & rgb (the
 // link_terms u), and the constant part is |L & g12|. When the register bits
-// sit on consecutive qubits (contig), A is one shift of u.
+// sit on consecutive qubits (kContig), A is one shift of u. qubits: those of
+// the register bits, a byte each.
+constexpr uint32_t kContig = 0x80u;
 __device__ __forceinline__ void chain_pending(uint32_t L, uint32_t rgb, uint32_t lgb, uint32_t g12, int n,
-                                                const uint32_t (&p)[4], bool contig, uint32_t& D) {
-  const uint32_t nmask = n >= 32 ? ~0u : ((1u << n) - 1u);
-  const uint32_t u = ((((L << 1) | (L >> (n - 1))) & nmask) & lgb) ^ (L & rgb);
-  const uint32_t A = contig ? (u >> p[0]) & 15u
-                            : ((u >> p[0]) & 1u) | (((u >> p[1]) & 1u) << 1) | (((u >> p[2]) & 1u) << 2) |
-                                  (((u >> p[3]) & 1u) << 3);
+                                                uint32_t qubits, uint32_t& D) {
+  // (lgb has no bits from n on, so the rotation of L needs no mask of its own)
+  const uint32_t u = (((L << 1) | (L >> (n - 1))) & lgb) ^ (L & rgb);
+  const uint32_t A = (qubits & kContig) ? (u >> (qubits & 31u)) & 15u
+                                        : ((u >> (qubits & 31u)) & 1u) | (((u >> ((qubits >> 8) & 31u)) & 1u) << 1) |
+                                              (((u >> ((qubits >> 16) & 31u)) & 1u) << 2) |
+                                              (((u >> ((qubits >> 24) & 31u)) & 1u) << 3);
   D ^= A | ((__popc(L & g12) & 1u) << 4);
 }
 
@@ -775,9 +778,10 @@ template <class Y>
 __device__ void loss_block(int kind, double* E, const Y* y, int64_t B, double scale, double* loss, double* dLdE,
                            const double* e_part, int tps, int tid, int nthr);
 
-struct PassShared {
+template <bool ROWS>
+struct PassSharedT {
   StepPar par[2];
-  float rows[kThreads / 32][32][8];  // round adjoints: a round's values of each lane
+  float rows[ROWS ? kThreads / 32 : 1][32][8];  // round adjoints: a round's values of each lane
   float4 ident[8];             // the diagonal of a round's run that has none
   uint32_t ticket;             // the CTA's finishing order (loss on the last CTA)
   uint32_t lg[256];
@@ -786,8 +790,10 @@ struct PassShared {
   double dred[kThreads / 32];
   uint32_t gmap[16];
   uint32_t gb[4];              // per register group: its lowest local bit
-  uint4 gpos[4];               // and its qubits
+  uint4 gpos[4];               // its qubits
+  uint32_t gqub[4];            // and the same in bytes (chain_pending)
 };
+using PassShared = PassSharedT<true>;
 
 // One CTA's share of a pass: tiles first_tile .. first_tile + tiles_per_cta-1
 // (tile = sample * tiles_per_sample + tile within the sample). Ends with a
@@ -799,8 +805,8 @@ struct PassShared {
 // -> 659 adjoint; step of n = 20, d = 24, 64 samples 25.10 -> 23.00 ms, of n =
 // 12, d = 20, 256 samples 237 -> 222 us.
 // H: threads per column as a power of two (1: two threads of 8 registers each).
-template <bool BWD, bool ROUNDS, bool TC = false, bool RX = false, int KC = 0, int H = 0>
-__device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_tile, float2* smem, PassShared& sh,
+template <bool BWD, bool ROUNDS, bool TC = false, bool RX = false, int KC = 0, int H = 0, class Shared>
+__device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_tile, float2* smem, Shared& sh,
                                          const TcCtx* tc = nullptr, float (*acc_rows)[8][32] = nullptr) {
   uint32_t (&s_lg)[256] = sh.lg;
   float (&s_red)[2][kThreads / 32][kMaxStepSlots] = sh.red;
@@ -838,8 +844,11 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
     s_gmap[tid] = pd.gmap[tid];
     if (tid < 4) {
       sh.gb[tid] = pd.groups[tid][0];
-      sh.gpos[tid] = make_uint4(pd.gmap[pd.groups[tid][0] & 15], pd.gmap[pd.groups[tid][1] & 15],
-                                pd.gmap[pd.groups[tid][2] & 15], pd.gmap[pd.groups[tid][3] & 15]);
+      const uint4 q = make_uint4(pd.gmap[pd.groups[tid][0] & 15], pd.gmap[pd.groups[tid][1] & 15],
+                                 pd.gmap[pd.groups[tid][2] & 15], pd.gmap[pd.groups[tid][3] & 15]);
+      sh.gpos[tid] = q;
+      sh.gqub[tid] = q.x | q.y << 8 | q.z << 16 | q.w << 24 |
+                     (q.y == q.x + 1 && q.z == q.x + 2 && q.w == q.x + 3 ? kContig : 0u);
     }
     if (ROUNDS && tid < 8) sh.ident[tid] = make_float4(1.f, 0.f, 1.f, 0.f);
   }
@@ -1065,8 +1074,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
       const uint32_t base = (col & ((1u << lb) - 1u)) | ((col >> lb) << (lb + 4u));
       float2* const at = tp + loc(base) + (H && h ? loc(8u << lb) : 0u);
       const uint32_t gb = gidx(base);
-      const uint4 gp = sh.gpos[g];
-      const uint32_t pos[4] = {gp.x, gp.y, gp.z, gp.w};
+      const uint32_t qubits = sh.gqub[g];
       float2 r[NR];
       float2 l[NR];
       ld_group<KC, BWD>(lb, at, at + lam_at, r, l);
@@ -1075,10 +1083,11 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
       const uint32_t rgb = ((gb >> 1) | ((gb & 1u) << (nq - 1))) & nmask;
       const uint32_t lgb = ((gb << 1) | (gb >> (nq - 1))) & nmask;
       const uint32_t g12 = gb & rgb;
-      const bool contig = pos[1] == pos[0] + 1 && pos[2] == pos[0] + 2 && pos[3] == pos[0] + 3;
       uint32_t D = 0;
-      if (!TC) chain_pending(pend, rgb, lgb, g12, nq, pos, contig, D);
+      if (!TC) chain_pending(pend, rgb, lgb, g12, nq, qubits, D);
       if constexpr (TC) {
+        const uint4 gp = sh.gpos[g];
+        const uint32_t pos[4] = {gp.x, gp.y, gp.z, gp.w};
         tc_rounds(*tc, P, nr, tc->bsm + (size_t)sb * kMaxStepRounds * kTcBFloats, gb, pos, a.n_eff, r, ph, tid);
       } else {
       // a round whose rotations are steep runs twice (see rot_T): the forward
@@ -1096,7 +1105,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
           else rot_T<3, RX>(r, pend_q(P.v[k][3].x, (D >> 3) & 1u), (lk.z >> 3) & 1u);
           apply_diag(r, pre ? sh.ident : &P.v[k][4 + (H ? 4 * h : 0)]);
           if (!pre) {
-            chain_pending(lk.x, rgb, lgb, g12, nq, pos, contig, D);
+            chain_pending(lk.x, rgb, lgb, g12, nq, qubits, D);
             pend ^= lk.w;
             ++k;
           }
@@ -1104,7 +1113,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
         } else {
           const uint4 lk = P.rec[k * (kBwdRoundWords / 4) + 2];  // links, bbits, rx mask, leaving links
           if (!again) {
-            chain_pending(lk.x, rgb, lgb, g12, nq, pos, contig, D);
+            chain_pending(lk.x, rgb, lgb, g12, nq, qubits, D);
             pend ^= lk.w;
           }
           float v[8];
@@ -1398,7 +1407,8 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
 template <bool BWD, bool ROUNDS, bool RX = false, int MINB = 2, int KC = 0, int H = 0>
 __global__ void __launch_bounds__(kThreads, MINB) pass_kernel(const PassArgs a) {
   extern __shared__ __align__(16) float2 smem[];
-  __shared__ PassShared sh;
+  // (the forward leaves the rows' 8 KiB to L1: n = 16, d = 20, 500 samples 2.16 -> 2.13 ms)
+  __shared__ PassSharedT<BWD && ROUNDS> sh;
   const int64_t first = KC ? (int64_t)blockIdx.x : (int64_t)blockIdx.x * (blockDim.x >> (a.pd.K - kRegBits + H));
   if constexpr (BWD && !ROUNDS) {
     __shared__ float acc_rows[kThreads / 32][8][32];  // a generic step's terms waiting for their reduction
@@ -1413,7 +1423,7 @@ __global__ void __launch_bounds__(kThreads, MINB) pass_kernel(const PassArgs a) 
 // two B staging buffers of kMaxStepRounds rounds.
 __global__ void __launch_bounds__(kThreads, 2) tc_pass_kernel(const PassArgs a) {
   extern __shared__ __align__(16) float2 smem[];
-  __shared__ PassShared sh;
+  __shared__ PassSharedT<false> sh;
   __shared__ __align__(8) uint64_t mbar[2];
   __shared__ uint32_t tmem_slot;
   const int warp = threadIdx.x >> 5;

@@ -386,16 +386,17 @@ __device__ __forceinline__ void diag_bwd(float2 (&p)[16], float2 (&l)[16], const
   g[3] = T;
 }
 
-// The rotation of an adjoint item on register bit R (q un-applies it; RX where
-// rx, uniform over the CTA, else RY), after the round's diagonal; gy: the
-// thread's sum of Im<lambda|P|psi> taken before it. A pending Z_R negates q
-// and gy. The round's scale and the earlier items' rotations multiply gy by a
-// factor that is the same for every thread and sample; the owner lane of the
-// reduced sum undoes it (the table's factor).
+// The gradient value of an adjoint item's rotation on register bit R (RX where
+// rx, uniform over the CTA, else RY): the thread's sum of Im<lambda|P|psi>, after
+// the round's diagonal and before any of its rotations (they commute with P on
+// the other bits). A pending Z_R (a) negates it. The round's scale multiplies it
+// by a factor that is the same for every thread and sample; the owner lane of
+// the reduced sum undoes it (the table's factor). All four values before the
+// rotations, and psi's rotations before lambda's, need fewer registers at a time
+// than rotation by rotation: adjoint of n = 20, d = 24, 64 samples 1.258 -> 1.244
+// ms a launch.
 template <int R, bool RX, int NR>
-__device__ __forceinline__ void rot_bwd(float2 (&p)[NR], float2 (&l)[NR], float qt, uint32_t a, float& gy, bool rx) {
-  const int f = (int)(a << 31);
-  const float q = __int_as_float(__float_as_int(qt) ^ f);
+__device__ __forceinline__ float grad_T(const float2 (&p)[NR], const float2 (&l)[NR], uint32_t a, bool rx) {
   float g;
   if (RX && rx) {
     g = 0.f;
@@ -417,9 +418,27 @@ __device__ __forceinline__ void rot_bwd(float2 (&p)[NR], float2 (&l)[NR], float 
     }
     g = (accp.x + accp.y) - (accm.x + accm.y);
   }
-  rot_T<R, RX>(p, q, rx);
-  rot_T<R, RX>(l, q, rx);
-  gy = __int_as_float(__float_as_int(g) ^ f);
+  return pend_q(g, a);
+}
+// A round's rotations on register bits 0 .. 2 (a half column) or 0 .. 3 of one state.
+template <bool RX, int NR>
+__device__ __forceinline__ void rots(float2 (&z)[NR], const float4* v, uint32_t D, uint32_t rx) {
+  rot_T<0, RX>(z, pend_q(v[0].x, D & 1u), rx & 1u);
+  rot_T<1, RX>(z, pend_q(v[1].x, (D >> 1) & 1u), (rx >> 1) & 1u);
+  rot_T<2, RX>(z, pend_q(v[2].x, (D >> 2) & 1u), (rx >> 2) & 1u);
+  if constexpr (NR == 16) rot_T<3, RX>(z, pend_q(v[3].x, (D >> 3) & 1u), (rx >> 3) & 1u);
+}
+
+// The same item by item, where an item may be an RX: one branch per item takes
+// its value and rotates both states (value by value, then state by state, took
+// 1.28 ms a launch of 100 states of 20 qubits, this 1.25). The value then carries
+// the earlier items' rotations (the table's .z).
+template <int R>
+__device__ __forceinline__ void item_bwd(float2 (&p)[16], float2 (&l)[16], float qt, uint32_t a, float& gy, bool rx) {
+  const float q = pend_q(qt, a);
+  gy = grad_T<R, true>(p, l, a, rx);
+  rot_T<R, true>(p, q, rx);
+  rot_T<R, true>(l, q, rx);
 }
 
 // ---- two threads per column ------------------------------------------------------
@@ -452,7 +471,8 @@ __device__ __forceinline__ void rot_fwd_half(float2 (&r)[8], float q, uint32_t h
   partner(r, o);
   rot_half<RX>(r, o, q, h, rx);
 }
-// rot_bwd on bit 3; gy: the thread's share (l_1 . p_0 in thread 1, -l_0 . p_1 in thread 0).
+// The gradient value and the rotation of an adjoint item on bit 3; gy: the
+// thread's share (l_1 . p_0 in thread 1, -l_0 . p_1 in thread 0).
 template <bool RX>
 __device__ __forceinline__ void rot_bwd_half(float2 (&p)[8], float2 (&l)[8], float qt, uint32_t a, float& gy, uint32_t h,
                                              bool rx) {
@@ -1098,11 +1118,8 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
         if (!BWD) {
           const uint4 lk = P.rec[k * (kFwdRoundWords / 4) + 1];  // links, bbits, rx mask, leaving links
           const bool pre = P.v[k][0].y < 0.f && !again;
-          rot_T<0, RX>(r, pend_q(P.v[k][0].x, D & 1u), lk.z & 1u);
-          rot_T<1, RX>(r, pend_q(P.v[k][1].x, (D >> 1) & 1u), (lk.z >> 1) & 1u);
-          rot_T<2, RX>(r, pend_q(P.v[k][2].x, (D >> 2) & 1u), (lk.z >> 2) & 1u);
+          rots<RX>(r, P.v[k], D, lk.z);
           if constexpr (H) rot_fwd_half<RX>(r, pend_q(P.v[k][3].x, (D >> 3) & 1u), h, (lk.z >> 3) & 1u);
-          else rot_T<3, RX>(r, pend_q(P.v[k][3].x, (D >> 3) & 1u), (lk.z >> 3) & 1u);
           apply_diag(r, pre ? sh.ident : &P.v[k][4 + (H ? 4 * h : 0)]);
           if (!pre) {
             chain_pending(lk.x, rgb, lgb, g12, nq, qubits, D);
@@ -1119,24 +1136,45 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
           float v[8];
           if constexpr (H) diag_bwd(r, l, again ? sh.ident : &P.v[k][4 + 4 * h], v, h);
           else diag_bwd(r, l, again ? sh.ident : &P.v[k][4], v);
-          rot_bwd<0, RX>(r, l, P.v[k][0].x, D & 1u, v[4], lk.z & 1u);
-          rot_bwd<1, RX>(r, l, P.v[k][1].x, (D >> 1) & 1u, v[5], (lk.z >> 1) & 1u);
-          rot_bwd<2, RX>(r, l, P.v[k][2].x, (D >> 2) & 1u, v[6], (lk.z >> 2) & 1u);
-          if constexpr (H) rot_bwd_half<RX>(r, l, P.v[k][3].x, (D >> 3) & 1u, v[7], h, (lk.z >> 3) & 1u);
-          else rot_bwd<3, RX>(r, l, P.v[k][3].x, (D >> 3) & 1u, v[7], (lk.z >> 3) & 1u);
-          // lane holds value idx of its tile; the first 8 lanes of a tile keep theirs
-          const int idx = lane & 7;
-          float sum = rows8(v, lanes, lane, sh.rows[warp]);
-          const bool owner = (lane & (lanes - 1)) < 8 && !again;  // a round's first run has its values
+          if constexpr (RX && !H) {
+            item_bwd<0>(r, l, P.v[k][0].x, D & 1u, v[4], lk.z & 1u);
+            item_bwd<1>(r, l, P.v[k][1].x, (D >> 1) & 1u, v[5], (lk.z >> 1) & 1u);
+            item_bwd<2>(r, l, P.v[k][2].x, (D >> 2) & 1u, v[6], (lk.z >> 2) & 1u);
+            item_bwd<3>(r, l, P.v[k][3].x, (D >> 3) & 1u, v[7], (lk.z >> 3) & 1u);
+          } else {
+            v[4] = grad_T<0, RX>(r, l, D & 1u, lk.z & 1u);
+            v[5] = grad_T<1, RX>(r, l, (D >> 1) & 1u, (lk.z >> 1) & 1u);
+            v[6] = grad_T<2, RX>(r, l, (D >> 2) & 1u, (lk.z >> 2) & 1u);
+            if constexpr (H) rot_bwd_half<RX>(r, l, P.v[k][3].x, (D >> 3) & 1u, v[7], h, (lk.z >> 3) & 1u);
+            else v[7] = grad_T<3, RX>(r, l, (D >> 3) & 1u, (lk.z >> 3) & 1u);
+            rots<RX>(r, P.v[k], D, lk.z);
+            rots<RX>(l, P.v[k], D, lk.z);
+          }
+          int idx;
+          float sum;
+          bool owner;
+          if constexpr (RX && !H) {
+            // shuffles here: with the rows, whose registers this instance lacks and
+            // whose 8 KiB L1 then lacks, 100 states of 20 qubits took 1.27 ms a launch,
+            // this 1.25
+            sum = lanes == 32 ? butterfly8(v, 32, lane, idx) : butterfly8(v, lanes, lane, idx);
+            owner = (lane & ((lanes >> 3) - 1)) == 0;
+          } else {
+            // lane holds value idx of its tile; the first 8 lanes of a tile keep theirs
+            idx = lane & 7;
+            sum = rows8(v, lanes, lane, sh.rows[warp]);
+            owner = (lane & (lanes - 1)) < 8;
+          }
+          owner = owner && !again;  // a round's first run has its values
           if (owner) {
             const int32_t term =
                 reinterpret_cast<const int32_t*>(&P.rec[k * (kBwdRoundWords / 4)])[idx];
-            if (idx >= 4) sum *= fabsf(P.v[k][idx - 4].y);
+            if (idx >= 4) sum *= RX && !H ? P.v[k][idx - 4].z : fabsf(P.v[k][0].y);
             if (Tt >= 32) {
               s_red[buf][warp][k * 8 + idx] = sum;
               if (warp == 0) s_slot[buf][k * 8 + idx] = term;
             } else if (active && term >= 0) {
-              a.g_part[tile * a.n_slots + term] = 0.5 * (double)sum;
+              a.g_part[tile * a.n_slots + term] = (double)(0.5f * sum);
             }
           }
           again = P.v[k][0].y < 0.f && !again;
@@ -1269,13 +1307,13 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
               const uint32_t kk = (ks & ~7u) + (uint32_t)idx;
               if ((lane & ((lanes >> 3) - 1)) == 0 && kk <= ks) {
                 if (Tt >= 32) s_red[buf][warp][kk] = sum;
-                else if (active) a.g_part[tile * a.n_slots + s_slot[buf][kk]] = 0.5 * (double)sum;
+                else if (active) a.g_part[tile * a.n_slots + s_slot[buf][kk]] = (double)(0.5f * sum);
               }
               __syncwarp();
             }
           } else {
             for (int off = 1; off < lanes; off <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-            if (active && (lane & (Tt - 1)) == 0) a.g_part[tile * a.n_slots + o.y] = 0.5 * (double)acc;
+            if (active && (lane & (Tt - 1)) == 0) a.g_part[tile * a.n_slots + o.y] = (double)(0.5f * acc);
           }
         } else if (oc == OP_CNOT) {
           const bool creg = ((o.y >> 8) & 1u) != 0;
@@ -1408,7 +1446,7 @@ template <bool BWD, bool ROUNDS, bool RX = false, int MINB = 2, int KC = 0, int 
 __global__ void __launch_bounds__(kThreads, MINB) pass_kernel(const PassArgs a) {
   extern __shared__ __align__(16) float2 smem[];
   // (the forward leaves the rows' 8 KiB to L1: n = 16, d = 20, 500 samples 2.16 -> 2.13 ms)
-  __shared__ PassSharedT<BWD && ROUNDS> sh;
+  __shared__ PassSharedT<BWD && ROUNDS && (H || !RX)> sh;
   const int64_t first = KC ? (int64_t)blockIdx.x : (int64_t)blockIdx.x * (blockDim.x >> (a.pd.K - kRegBits + H));
   if constexpr (BWD && !ROUNDS) {
     __shared__ float acc_rows[kThreads / 32][8][32];  // a generic step's terms waiting for their reduction
@@ -1641,19 +1679,23 @@ __device__ void round_params(const PrepArgs& a, bool on, bool fwd, int64_t r, co
   float4* out = (fwd ? a.rpf : a.rpb) + r * kRoundPar;
   RoundPar64* out64 = (fwd ? a.rpf64 : a.rpb64) + r;
   if (e < 4) {
-    // the factor of rotation e's gradient value: 1 / (scale^2), less the rotations before it
-    double g = Q[3];
+    // the factors of the rotations' gradient values: 1 / scale^2 (S: the product
+    // of the Q), and, for kernels that take each after the rotations before it,
+    // less those (complex128's only one)
+    double g = Q[3], all = S;
 #pragma unroll
     for (int k = 2; k >= 0; --k)
       if (k >= e) g *= Q[k];
-    if (twice) g *= S;
+    if (twice) {
+      g *= S;
+      all *= S;
+    }
     if (!fwd) q = -q;
-    if (twice) g = -g;
     if (f64) {
       out64->q[e] = q;
-      out64->g[e] = g;
+      out64->g[e] = twice ? -g : g;
     } else {
-      out[e] = make_float4((float)q, (float)g, 0.f, 0.f);
+      out[e] = make_float4((float)q, (float)(twice ? -all : all), (float)g, 0.f);
     }
   } else if (e < 12) {
     const double sc = (neg ? -1.0 : 1.0) * (twice ? 1.0 / S : rsqrt(S));

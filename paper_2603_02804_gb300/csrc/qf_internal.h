@@ -58,8 +58,9 @@ constexpr int kFwdRoundWords = 16;
 constexpr int kBwdRoundWords = 12;
 constexpr int kMaxStepRounds = 4;   // 8 gradient values per round
 // Parameters of one round of a complex64 round program, in float4: [0, 4) the 4
-// items' rotations, x = q and y = the factor of the adjoint's gradient value of
-// the rotation (negative: the round runs twice); [4, 12) the round's diagonal,
+// items' rotations, x = q and y = the factor of the adjoint's gradient values of
+// the rotations (negative: the round runs twice), z = that of the item's own
+// where the values are taken item by item; [4, 12) the round's diagonal,
 // i.e. the 4 RZ runs (and the CZ links between register bits) merged into one
 // phase per register index, two per float4, times the scale and sign that the
 // rotations leave out. (The four q's in one float4 would be loaded together,

@@ -167,7 +167,9 @@ typedef struct {
 /* Summary of a plan (host-side numbers). */
 typedef struct {
   int32_t n_qubits;        /* as created                                       */
-  int32_t n_eff;           /* simulated qubits (>= 4: smaller circuits padded)  */
+  int32_t n_eff;           /* simulated qubits (>= 4: smaller circuits padded;
+                              7 where a smaller circuit's batch runs faster in
+                              round programs, with idle qubits)               */
   int32_t n_params;
   int32_t n_slots;         /* gradient slots = parametrised gates               */
   int32_t path;

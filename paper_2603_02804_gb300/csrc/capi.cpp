@@ -1117,7 +1117,25 @@ qf_status qf_circuit_destroy(qf_circuit* c) {
   return QF_OK;
 }
 
-qf_status qf_plan(qf_circuit* c, const qf_plan_opts* opts, int64_t batch, size_t* workspace_bytes) {
+// Whether a circuit of fewer than 7 qubits may be simulated on 7, where round
+// programs run it: 8 threads per sample in place of one to four, and a quarter
+// of the steps. 4 qubits, 20 layers, step of 8 / 2048 samples 156 / 203 ->
+// 43 / 66 us; 6 qubits, 64 samples 244 -> 78 us; complex128, 4 qubits, 2 layers,
+// 64 samples 213 -> 99 us. The state is up to 8 times as large, which shows in
+// batches that fill the GPU: at 8192 samples the forward of 4 qubits, 2 layers
+// takes 24.8 us against 21.7, complex128 steps 1.2 to 1.3 times as long (at 2048
+// half as long). A complex128 forward of one qubit is slower at every batch (114
+// us against 59).
+static bool may_pad(const qf_circuit* c, const qf_plan_opts& o, int64_t batch) {
+  if (o.tile_bits != 0 || o.ckpt_mode != 0) return false;
+  return c->f64 ? c->circ.n >= qf::kRegBits && batch <= 2048 : batch <= 4096;
+}
+// A padded plan's workspace and tables stay within half of the fixed scratch
+// block of qf_train_step_noalloc, so that a step which fits it unpadded is not
+// refused; qf_plan_fit, whose caller counts bytes, does not pad.
+static constexpr size_t kPadBytes = QF_NOALLOC_MAX_BYTES / 2;
+
+static qf_status plan_circuit(qf_circuit* c, const qf_plan_opts* opts, int64_t batch, bool pad, size_t* workspace_bytes) {
   if (!c) return fail(QF_ERR_INVALID_ARG, "null circuit");
   if (batch < 0) return fail(QF_ERR_INVALID_ARG, "negative batch");
   qf_plan_opts o{};
@@ -1169,6 +1187,7 @@ qf_status qf_plan(qf_circuit* c, const qf_plan_opts* opts, int64_t batch, size_t
     }
     c->tc = false;
     if (c->path == QF_PATH_FUSED) {
+      req.pad = pad && may_pad(c, o, batch);
       c->fp = qf::plan_fused(c->circ, req);
       c->lay_valid = true;
       c->lay_tile_bits = o.tile_bits;
@@ -1188,6 +1207,12 @@ qf_status qf_plan(qf_circuit* c, const qf_plan_opts* opts, int64_t batch, size_t
     }
     c->L = make_layout(c, batch);
     build_blob(c);
+    if (req.pad && c->fp.n_eff > std::max(c->circ.n, qf::kRegBits) && c->L.total + c->blob.size() > kPadBytes) {
+      req.pad = false;
+      c->fp = qf::plan_fused(c->circ, req);
+      c->L = make_layout(c, batch);
+      build_blob(c);
+    }
   } catch (const std::domain_error& e) {
     return fail(QF_ERR_UNSUPPORTED, e.what());
   } catch (const std::bad_alloc&) {
@@ -1202,6 +1227,10 @@ qf_status qf_plan(qf_circuit* c, const qf_plan_opts* opts, int64_t batch, size_t
   c->planned = true;
   if (workspace_bytes) *workspace_bytes = c->L.total;
   return QF_OK;
+}
+
+qf_status qf_plan(qf_circuit* c, const qf_plan_opts* opts, int64_t batch, size_t* workspace_bytes) {
+  return plan_circuit(c, opts, batch, true, workspace_bytes);
 }
 
 double qf_mem_model(double k, double d, double b, double* b_best) {
@@ -1222,7 +1251,7 @@ qf_status qf_plan_fit(qf_circuit* c, const qf_plan_opts* opts, int64_t batch, si
     qf_plan_opts t = o;
     t.ckpt_layers = cl;
     t.host_only = 1;
-    return qf_plan(c, &t, batch, ws);
+    return plan_circuit(c, &t, batch, false, ws);
   };
   size_t ws = 0;
   qf_status s;
@@ -1253,7 +1282,7 @@ qf_status qf_plan_fit(qf_circuit* c, const qf_plan_opts* opts, int64_t batch, si
     if (wsc(best) > mem_bytes) return fail(QF_ERR_WORKSPACE, "no checkpoint interval fits");
     qf_plan_opts fin = o;
     fin.ckpt_layers = best;
-    if ((s = qf_plan(c, &fin, batch, &ws)) != QF_OK) return s;
+    if ((s = plan_circuit(c, &fin, batch, false, &ws)) != QF_OK) return s;
     *ckpt_layers = best;
     if (workspace_bytes) *workspace_bytes = ws;
     return QF_OK;
@@ -1270,7 +1299,7 @@ qf_status qf_plan_fit(qf_circuit* c, const qf_plan_opts* opts, int64_t batch, si
   }
   qf_plan_opts fin = o;
   fin.ckpt_layers = hi;
-  if ((s = qf_plan(c, &fin, batch, &ws)) != QF_OK) return s;
+  if ((s = plan_circuit(c, &fin, batch, false, &ws)) != QF_OK) return s;
   *ckpt_layers = hi;
   if (workspace_bytes) *workspace_bytes = ws;
   return QF_OK;
@@ -1831,7 +1860,7 @@ qf_status qf_batch_create(int32_t n_circuits, qf_circuit* const* circuits, const
         throw std::invalid_argument("batched launches take RZ/RY round programs (no RX)" + at);
       if (c->path == QF_PATH_FUSED && (c->fp.ckpt_mode != 0 || c->tc))
         throw std::invalid_argument("batched launches use checkpoint mode 0 on the CUDA cores" + at);
-      if (c->path != QF_PATH_FUSED || !c->fp.rounds)
+      if (c->path != QF_PATH_FUSED || !c->fp.rounds || c->circ.n < qf::kRoundQubits)
         throw std::invalid_argument("batched launches need fused round programs (RZ/RY rotations, CZ on "
                                     "neighbouring qubits, at least 7 qubits per tile)" + at);
       if (b->B[i] < 1) throw std::invalid_argument("batch must be >= 1" + at);

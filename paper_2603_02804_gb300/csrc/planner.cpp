@@ -556,6 +556,15 @@ static bool round_eligible(const Circuit& c) {
   return true;
 }
 
+// Whether a circuit below the round programs' 7 qubits keeps its links when
+// padded to them (the ring's closing link would not be one of neighbours).
+static bool pads_to_rounds(const Circuit& c) {
+  if (c.n >= kRoundQubits || !round_eligible(c)) return false;
+  for (const Gate& g : c.gates)
+    if (g.kind == G_CZ && std::abs(g.q0 - g.q1) != 1) return false;
+  return true;
+}
+
 static void fill_slots(const Circuit& c, std::vector<int32_t>& slot_param, std::vector<int32_t>& slot_kind,
                        std::vector<int32_t>& slot_gate, std::vector<int32_t>& param_off,
                        std::vector<int32_t>& param_slots) {
@@ -771,15 +780,21 @@ namespace {
 FusedPlan plan_fused_with(const Circuit& c_in, const PlanRequest& req, bool strict_catch_up) {
   validate_circuit(c_in);
   FusedPlan P;
-  P.n_eff = std::max(c_in.n, kRegBits);
+  const bool padded = req.pad && !req.generic && req.tile_bits == 0 && pads_to_rounds(c_in);
+  P.n_eff = padded ? kRoundQubits : std::max(c_in.n, kRegBits);
   int K = req.tile_bits > 0 ? req.tile_bits : kMaxTileBits;
   if (K < kRegBits || K > kMaxTileBits) throw std::runtime_error("tile_bits must be in 4..12");
   K = std::min(K, P.n_eff);
   // a multi-pass tile needs at least one qubit beyond the low nibble
   if (P.n_eff > K && K < kRegBits + 1) K = kRegBits + 1;
   P.K = K;
-  P.rounds = !req.generic && K >= 7 && round_eligible(c_in);
-  const Circuit& c = c_in;
+  P.rounds = !req.generic && K >= kRoundQubits && round_eligible(c_in);
+  Circuit wide;
+  if (padded) {
+    wide = c_in;
+    wide.n = P.n_eff;
+  }
+  const Circuit& c = padded ? wide : c_in;
   // gradient terms: generic programs have one per rotation, in circuit order
   std::vector<int> term_of_gate(c.gates.size(), -1);
   P.term_off.assign(1, 0);
@@ -811,7 +826,7 @@ FusedPlan plan_fused_with(const Circuit& c_in, const PlanRequest& req, bool stri
   };
 
   // checkpoint boundaries in gate-sequence positions
-  const int G = ckpt_interval_gates(c, req.ckpt_layers);
+  const int G = ckpt_interval_gates(c_in, req.ckpt_layers);
   long next_ckpt = G;
   int prefix = 0;
   int n_ckpt_slots = 0;

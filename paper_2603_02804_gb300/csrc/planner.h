@@ -84,6 +84,7 @@ struct PlanRequest {
   int qshift = -1;       // layout to use (-1: choose), as FusedPlan::qshift
   int strict = -1;       // catch-up rule to use (-1: choose), as FusedPlan::strict
   int catch_up = -1;     // rule the layout search may choose (-1: either, 0: rising, 1: strict)
+  bool pad = false;      // circuits of fewer than 7 qubits may be simulated on 7 (round programs)
 };
 
 // Throws std::runtime_error with a message on invalid input.

@@ -15,6 +15,7 @@
 namespace qf {
 
 constexpr int kThreads = 256;          // threads per CTA of the pass kernels
+constexpr int kRoundQubits = 7;        // round programs' fewest qubits per tile (8 threads: the reductions' lanes)
 constexpr int kRegBits = 4;            // amplitudes per thread per step = 16
 constexpr int kMaxTileBits = 12;       // 4096 amplitudes = 32 KiB per state tile
 constexpr int kTileAmps = 1 << kMaxTileBits;

@@ -5,7 +5,7 @@ import pytest
 import torch
 
 from oracle import oracle as orc
-from paper_2603_02804_gb300 import build as qbuild
+from paper_2603_02804_gb300 import build as qbuild, workloads
 from paper_2603_02804_gb300.torch_api import Batch, Simulator
 
 pytestmark = pytest.mark.gpu
@@ -103,3 +103,39 @@ def test_observables_beyond_the_tile(n, kw, obs):
     """The adjoint seeded from another tile's amplitudes (X or Y on qubits
     outside the last pass's tile, on bit 0 and not), and E over half the state."""
     check(Simulator(n, 3, 3, obs=obs, **kw), orc.hea(n, 3), n, 9 * n, 3, obs, np.float32, 1e-5, n)
+
+
+@pytest.mark.parametrize("precision,real,tol", [("complex64", np.float32, 1e-5), ("complex128", np.float64, 1e-11)])
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 6])
+def test_few_qubits_on_seven(n, precision, real, tol):
+    """Chains of fewer than 7 qubits run as round programs on 7, up to the batch
+    where the larger state costs more, and up to a bounded workspace; observables
+    on the last qubits, given states and rings (whose closing link has no
+    neighbours there) keep their results."""
+    obs = "YX"[:n] if n < 3 else "I" * (n - 3) + "ZYX"
+    most = 2048 if precision == "complex128" else 4096
+    for B in (5, most, most + 1):
+        sim = Simulator(n, 2, B, obs=obs, precision=precision)
+        padded = B <= most and (precision == "complex64" or n >= 4)
+        assert sim.info()["n_eff"] == (7 if padded else max(n, 4))
+        check(sim, orc.hea(n, 2), n, 6 * n, B, obs, real, tol, 40 + n + B)
+    assert Simulator(n, 2000, 512, precision=precision).info()["n_eff"] == max(n, 4)  # 200 stored states
+    if n >= 3:
+        rows = workloads.xyz_ring_gates(n, 2)
+        sim = Simulator(n, 0, 5, gates=rows, n_params=6 * n, obs=obs, precision=precision)
+        assert sim.info()["n_eff"] == max(n, 4)
+        check(sim, orc.Circuit(n=n, gates=np.array(rows, np.int32), n_params=6 * n), n, 6 * n, 5, obs, real, tol, n)
+    if precision == "complex64":
+        rows = [r for r in workloads.xyz_ring_gates(n, 2) if r[0] != 3 or r[2] == r[1] + 1]
+        rng = np.random.default_rng(n)
+        psi = rng.normal(size=(3, 2 ** n, 2))
+        psi = np.ascontiguousarray((psi / np.linalg.norm(psi, axis=(1, 2), keepdims=True)).astype(np.float32))
+        states = torch.view_as_complex(torch.from_numpy(psi)).cuda()
+        theta = torch.from_numpy(rng.uniform(0, 2 * np.pi, 6 * n).astype(np.float32)).cuda()
+        out = []
+        for program in (0, 1):
+            sim = Simulator(n, 0, 3, gates=rows, n_params=6 * n, obs=obs, encoding="state", program=program)
+            assert sim.info()["n_eff"] == (7 if program == 0 else max(n, 4))
+            out.append([v.double().cpu().numpy() for v in sim.train_step(theta, states)])
+        for a, b in zip(*out):
+            assert np.max(np.abs(a - b)) < tol

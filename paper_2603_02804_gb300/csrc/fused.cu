@@ -860,6 +860,9 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
   const int wpt = Tt >= 32 ? Tt / 32 : 1;  // warps per tile
   const int lanes = Tt < 32 ? Tt : 32;
 
+  // (round programs: one op per step, read a step ahead; the first one here)
+  uint2 next = make_uint2(0u, 0u);
+  if (ROUNDS && pd.op_begin < pd.op_end) next = __ldg(a.ops + pd.op_begin);
   if (tid < 16) {
     s_gmap[tid] = pd.gmap[tid];
     if (tid < 4) {
@@ -934,8 +937,22 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
     cp_async_commit();
   };
 
+  // round programs: the first step's parameters, on their way while the tile
+  // loads (after them, they were two more trips to L2 in a row: a ring of 13
+  // qubits, 37 samples, adjoint 19.6 -> 18.8 us a pass and forward 10.5 -> 10.1; n
+  // = 16, d = 100, 64 samples 4.88 -> 4.80 ms a step). The tile's loads go first:
+  // waiting for the op word before them took n = 20 from 1.244 to 1.255 ms a pass.
+  auto stage_first = [&]() {
+    if (ROUNDS && warp == 0) {
+      uint32_t rb;
+      int nr;
+      if (next_step(pd.op_begin, rb, nr)) stage(0, rb, nr);
+    }
+  };
+
   // ---- bring psi (and lambda) in -------------------------------------------
   const int32_t psrc = pd.psi_src;
+  if (psrc == SRC_GENERATE || !active) stage_first();
   if (psrc == SRC_GENERATE && a.psi_in) {
     // given initial states [B][2^n_in]; padding qubits (n_in <= bit < n_eff) are |0>
     const int64_t din = 1ll << a.n_in;
@@ -1000,6 +1017,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
       else vp[it] = __ldcg(reinterpret_cast<const float4*>(src + g));
       if (two) vl[it] = __ldcg(reinterpret_cast<const float4*>(lsrc + (g ^ lx)));
     }
+    stage_first();
     if (far) {
       const float scale = (float)(2.0 * a.dLdE[b]);
 #pragma unroll
@@ -1025,14 +1043,8 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
 #pragma unroll
     for (int it = 0; it < NIT; ++it) st_pair(tl, p_it(it), __ldcg(reinterpret_cast<const float4*>(src + g_it(it))));
   }
-  // round programs: stage the first step's parameters
-  int sb = 0;
-  if (ROUNDS && warp == 0) {
-    uint32_t rb;
-    int nr;
-    if (next_step(pd.op_begin, rb, nr)) stage(0, rb, nr);
-    cp_async_wait_all();
-  }
+  int sb = 0;  // round programs: the step's staging buffer
+  if (ROUNDS && warp == 0) cp_async_wait_all();
   if (TC) {
     uint32_t rb;
     int nr;
@@ -1062,9 +1074,6 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
   uint32_t pend = 0;  // links whose CZ signs the tile's amplitudes still lack (round programs)
   int32_t pc = pd.op_begin;
   const uint2* ops = a.ops;
-  // (round programs: one op per step, read a step ahead)
-  uint2 next = make_uint2(0u, 0u);
-  if (ROUNDS && pc < pd.op_end) next = __ldg(ops + pc);
 #pragma unroll 1
   while (pc < pd.op_end) {
     const uint2 op = ROUNDS ? next : __ldg(ops + pc);

@@ -1,7 +1,8 @@
 // Fused forward / adjoint pass kernels for sm_103a.
 //
 // One CTA (256 threads) owns 4096 amplitudes of shared memory per state:
-// one tile of K = 12 tile bits, or 2^(12-K) tiles of a smaller circuit. A
+// one tile of K = 12 tile bits, or 2^(12-K) tiles of a smaller circuit (fewer
+// where a launch has few tiles, see the launch rule). A
 // pass loads its tiles from HBM once (or generates psi_0 in place), runs the
 // pass's step program on them in shared memory and registers, and stores them
 // once: the forward and backward gate fusion of Secs. 3.2-3.3.
@@ -1055,7 +1056,13 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
   __syncthreads();
   if (BWD && pd.lam_src == LAM_SEED) {
     // lambda_M = 2 (dL/dE_b) O psi_M (Eq. 4); (O psi)_x = i^{#Y} (-1)^{|(x^xm)&zm|} psi_{x^xm}
-    const float scale = active ? (float)(2.0 * a.dLdE[b]) : 0.f;
+    float scale = 0.f;
+    if (active) {
+      double dl = 1.0;
+      if (a.dLdE) dl = a.dLdE[b];
+      else if (a.loss_kind == 1) dl = a.loss_scale * (a.e_part[b] - (double)a.y[b]);  // one tile per sample
+      scale = (float)(2.0 * dl);
+    }
 #pragma unroll 1
     for (int it = 0; it < NR; ++it) {
       const uint32_t i = (uint32_t)it * Tt + tau;  // single amplitudes here
@@ -1533,7 +1540,7 @@ __global__ void tc_table_kernel(const uint4* fwd_rounds, int32_t n_rounds, const
 // Gate tables from theta in float64, rounded once to float32 (or kept in
 // float64 for complex128 plans): generic programs' fused 2x2 products
 // (forward) and (cos, sin) of theta/2 per term (backward); round programs'
-// per-round rotation shears and diagonal phases (both directions); (cos, sin)
+// per-round rotations and diagonal phases (both directions); (cos, sin)
 // of x/2 per sample and qubit (encoding). Element 0 also clears the forward
 // pass's CTA counter when a train step finishes its loss in that pass.
 __device__ void prep_one(const PrepArgs& a, int64_t i);
@@ -1820,6 +1827,16 @@ __global__ void g_partial_kernel(const double* g_part, int64_t rows_per_group, i
 // grad[p] (or grad[b][p]) = sum over tiles, then over the slots of p, in a
 // fixed order.
 __global__ void g_reduce_kernel(const GradReduceArgs a) {
+  // (a.loss: the last block does the step's loss beside the gradients)
+  if (a.loss && blockIdx.x == gridDim.x - 1) {
+    if (a.f64)
+      loss_block<double>(a.loss_kind, a.E, static_cast<const double*>(a.y), a.B, a.loss_scale, a.loss, a.dLdE, a.e_part, 1,
+                         threadIdx.x, 256);
+    else
+      loss_block<float>(a.loss_kind, a.E, static_cast<const float*>(a.y), a.B, a.loss_scale, a.loss, a.dLdE, a.e_part, 1,
+                        threadIdx.x, 256);
+    return;
+  }
   // one warp per output value; lane k sums rows k, k+32, ... and the warp
   // combines the 32 lane sums in a fixed butterfly (bitwise repeatable)
   const int64_t out = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -2387,7 +2404,7 @@ cudaError_t launch_g_reduce(const GradReduceArgs& a, cudaStream_t st) {
   if (g_reduce_stages(a.tps, a.slot_step) == 2) {
     // many rows per output: coalesced chunk sums first (groups: the samples
     // in per-sample mode, else all rows), then the fixed-order sum over chunks
-    if (a.scratch == nullptr || a.B == 0) return cudaErrorInvalidValue;
+    if (a.scratch == nullptr || a.B == 0 || a.loss) return cudaErrorInvalidValue;
     const int64_t groups = a.per_sample ? a.B : 1;
     const int64_t rows = a.per_sample ? a.tps : a.B * a.tps;
     const int64_t chunks = (rows + kGReduceChunk - 1) / kGReduceChunk;
@@ -2402,7 +2419,7 @@ cudaError_t launch_g_reduce(const GradReduceArgs& a, cudaStream_t st) {
     r.per_sample = a.per_sample;
   }
   const int64_t threads = n * 32;
-  g_reduce_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(r);
+  g_reduce_kernel<<<(unsigned)((threads + 255) / 256) + (r.loss ? 1u : 0u), 256, 0, st>>>(r);
   return cudaGetLastError();
 }
 

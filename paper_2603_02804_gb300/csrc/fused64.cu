@@ -474,7 +474,13 @@ __global__ void __launch_bounds__(kThreads, 1) pass64_kernel(const PassArgs64 a)
   barrier();
   if (BWD && pd.lam_src == LAM_SEED) {
     // lambda_M = 2 (dL/dE_b) O psi_M (Eq. 4); (O psi)_x = i^{#Y} (-1)^{|(x^xm)&zm|} psi_{x^xm}
-    const double scale = active ? 2.0 * a.dLdE[b] : 0.0;
+    double scale = 0.0;
+    if (active) {
+      double dl = 1.0;
+      if (a.dLdE) dl = a.dLdE[b];
+      else if (a.loss_kind == 1) dl = a.loss_scale * (a.e_part[b] - a.y[b]);  // one tile per sample
+      scale = 2.0 * dl;
+    }
 #pragma unroll 1
     for (int it = 0; it < 16; ++it) {
       const uint32_t i = (uint32_t)it * Tt + tau;

@@ -31,7 +31,7 @@ struct PassArgs {
   uint32_t x_mask;        // observable X/Y part (global bits; read for LAM_SEED_FAR)
   uint32_t z_mask;        // observable Z part (global bits)
   uint32_t y_count;       // number of Y factors (phase i^y_count)
-  const double* dLdE;     // [B]
+  const double* dLdE;     // [B]; null: a late loss (below), the seed's from the sample's own E
   double* e_part;         // [B * tiles per sample]
   double* g_part;         // [B * tiles per sample][n_slots], or [B][n_slots] when g_accum
   int32_t n_slots;
@@ -42,6 +42,9 @@ struct PassArgs {
   // The pass that computes the expectation may also finish the loss: with
   // done != null, the last CTA to finish sums E from e_part and writes E, the
   // loss and dL/dE as loss_kernel does (done: a CTA counter prep zeroes).
+  // A late loss (one tile per sample) needs no such pass: the adjoint's seed
+  // takes dL/dE from the sample's own partial, and the gradient reduction's
+  // launch finishes the loss.
   uint32_t* done;
   double* E;              // [B]
   const float* y;         // labels (MSE)
@@ -127,6 +130,14 @@ struct GradReduceArgs {
   int32_t per_sample;
   double* grad;
   double* scratch;      // stage-1 partials of a two-stage reduction (g_reduce_stages() == 2)
+  double* loss;         // non-null: one more block finishes a late loss (one stage, one tile per sample)
+  double* E;
+  double* dLdE;
+  const double* e_part;
+  const void* y;        // float64 labels where f64
+  int32_t f64;
+  int32_t loss_kind;
+  double loss_scale;    // 2 / B
 };
 
 // Launches of launch_g_reduce for partial rows per sample `tps` and slot
@@ -206,7 +217,10 @@ struct PassArgs64 {
   int64_t slot_stride;
   uint32_t z_mask;
   uint32_t y_count;
-  const double* dLdE;
+  const double* dLdE;     // [B]; null: a late loss (see PassArgs)
+  const double* y;        // labels of a late loss
+  int32_t loss_kind;
+  double loss_scale;
   double* e_part;         // [B * tiles per sample]
   double* g_part;         // [B * tiles per sample][n_slots]
   int32_t n_slots;

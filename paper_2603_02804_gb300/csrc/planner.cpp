@@ -986,7 +986,7 @@ FusedPlan plan_fused_with(const Circuit& c_in, const PlanRequest& req, bool stri
         if ((bbits >> r) & 1u) ext &= ~(1u << gq[r]);
       step_ext ^= ext;
       fw[7] = ext;
-      for (int r = 0; r < 8; ++r) fw[8 + r] = (uint32_t)bw[r];  // the items' terms (forward shears)
+      for (int r = 0; r < 8; ++r) fw[8 + r] = (uint32_t)bw[r];  // the items' terms (the forward's parameters)
       bw[8] = (int32_t)links;
       bw[9] = (int32_t)bbits;
       bw[10] = (int32_t)rx_mask;

@@ -3,8 +3,7 @@
 // A plan is a list of passes. A pass streams every tile of the batched state
 // once: a tile is the 2^K amplitudes whose indices differ only in K chosen
 // "tile bits" (always including global bits 0..3, so every tile is a set of
-// contiguous 128-byte runs). The tile sits in shared memory (XOR-swizzled)
-// while a program of steps runs on it. A step loads 16 amplitudes per thread
+// contiguous 128-byte runs). The tile sits in shared memory while a program of steps runs on it. A step loads 16 amplitudes per thread
 // whose indices differ in 4 tile bits (the step's register group), applies
 // every gate absorbed into the step to those registers, and stores them back.
 // This is the gate-fusion of Secs. 3.2-3.3 generalised from "one fused 2x2
@@ -66,8 +65,8 @@ constexpr int kMaxStepRounds = 4;   // 8 gradient values per round
 // phase per register index, two per float4, times the scale and sign that the
 // rotations leave out. (The four q's in one float4 would be loaded together,
 // and the adjoint has no registers for that: it spilled, 3 % slower.) Prep
-// fills them with 16 lanes per round; complex128 programs hold shears and
-// phases in float64 (RoundPar64).
+// fills them with 16 lanes per round; complex128 programs hold the same in
+// float64 (RoundPar64).
 constexpr int kRoundPar = 12;
 constexpr double kMaxTan = 256.0;   // largest |tan(w/2)| of a round that runs its rotations once
 

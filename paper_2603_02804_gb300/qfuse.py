@@ -127,10 +127,12 @@ def _ptr(t) -> int | None:
     """Device/host address of a tensor, numpy array or int (None stays NULL)."""
     if t is None:
         return None
+    try:
+        return t.data_ptr()
+    except AttributeError:
+        pass
     if isinstance(t, int):
         return t
-    if hasattr(t, "data_ptr"):
-        return t.data_ptr()
     if hasattr(t, "ctypes"):
         return t.ctypes.data
     raise TypeError(f"cannot take the address of {type(t)}")

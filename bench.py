@@ -122,16 +122,17 @@ def fp32_peak_tflops(peaks):
 def algorithmic_flops(n, d, B):
     """Arithmetic per step in flops (a multiply or an add = 1, FMA = 2) of the
     round programs, per qubit and layer and per pair of amplitudes.
-    Forward: the RY as three shears on (re, im) = 6 FMA = 12 flops, plus a
-    quarter of the round's merged diagonal (one complex multiply, 6 flops, per
-    amplitude for the 4 RZ runs of a round) = 3 flops; 15 in all.
-    Adjoint: the RY un-applied from psi and lambda (12 FMA) and its
-    Im<lambda|Y|psi> (4 FMA) = 32 flops, plus a quarter of the diagonal's
+    Forward: the RY as [[1, -q], [q, 1]] on (re, im) (its scale is in the
+    diagonal) = 4 FMA = 8 flops, plus a quarter of the round's merged diagonal
+    (one complex multiply, 6 flops, per amplitude for the 4 RZ runs of a round)
+    = 3 flops; 11 in all.
+    Adjoint: the RY un-applied from psi and lambda (8 FMA) and its
+    Im<lambda|Y|psi> (4 FMA) = 24 flops, plus a quarter of the diagonal's
     share (two complex multiplies and Im(conj(lambda) psi) per amplitude,
-    15 flops, and the signed sums) = 8 flops; 40 in all. Counting each gate
+    15 flops, and the signed sums) = 8 flops; 32 in all. Counting each gate
     separately, as a per-gate program must, gives 36 and 96."""
     pairs = B * (1 << (n - 1))
-    return n * d * pairs * 15, n * d * pairs * 40
+    return n * d * pairs * 11, n * d * pairs * 32
 
 
 def per_gate_model_flops(n, d, B):
@@ -523,7 +524,7 @@ def run_large(args, w):
         "traffic": traffic, "traffic_note": traffic_note,
         "kernel": "pass_kernel<true> (fused adjoint pass)", "peak_source": f"{peak_what} (derived: FP32 FMA peak)",
         "bwd_kernel_ms": bwd_launch_ms, "fwd_kernel_ms": fwd_launch_ms,
-        "flops_model": "executed arithmetic of the round programs: 15 (forward) and 40 (adjoint) flops per "
+        "flops_model": "executed arithmetic of the round programs: 11 (forward) and 32 (adjoint) flops per "
                        "amplitude pair, qubit and layer",
         "per_gate_flops_model": {"achieved": pg_bwd / passes / (bwd_launch_ms / 1e3) / 1e12,
                                  "frac": pg_bwd / passes / (bwd_launch_ms / 1e3) / 1e12 / fp32_peak,
@@ -1065,7 +1066,7 @@ def run_small(args, w):
                 "fwd_kernel": {"achieved": (fwd_fl / info["n_passes"]) / (fwd_launch_ms / 1e3) / 1e12,
                                "ms": fwd_launch_ms},
                 "bwd_kernel_ms": bwd_launch_ms,
-                "flops_model": "executed arithmetic of the round programs: 15 (forward) and 40 (adjoint) flops "
+                "flops_model": "executed arithmetic of the round programs: 11 (forward) and 32 (adjoint) flops "
                                "per amplitude pair, qubit and layer",
                 "timing": (f"CUDA events on the launching stream around every pass launch of {args.steps} "
                            f"steps run right after the timed ones (launched kernel by kernel: "

@@ -159,8 +159,9 @@ typedef struct {
   int32_t fwd_ctas;    /* fused forward round passes: CTAs per SM the pass kernel
                           is budgeted for (registers per thread): 0 = automatic
                           (3 when a pass has more tiles than two CTAs per SM
-                          hold, else 2), 2 or 3. Tuning knob; results do not
-                          depend on it                                          */
+                          hold, else 2), 2 or 3; without effect where two threads
+                          share a column (small launches). Tuning knob; results
+                          do not depend on it                                   */
   int32_t reserved[4];
 } qf_plan_opts;
 
@@ -402,16 +403,17 @@ qf_status qf_graph_stats(const qf_circuit* c, int64_t* recorded, int64_t* replay
 /* ---- batched launch over many circuits ----------------------------------
  * Many circuits of different widths, depths and batch sizes, trained in one
  * persistent kernel launch: each work item (one sample, or a group of small
- * samples, of one circuit) is taken by one CTA from a work queue ordered
- * largest first, and that CTA runs the item's fused forward passes, its
- * dL/dE and its fused adjoint passes (Secs. 3.2-3.3) with no waits on other
- * CTAs. The loss is summed over every circuit; each circuit gets its own
+ * samples, of one circuit) is taken from a work queue ordered largest first by
+ * a cluster of CTAs that shares its tiles (by one CTA where a sample is one
+ * tile), which runs the item's fused forward passes, its dL/dE and its fused
+ * adjoint passes (Secs. 3.2-3.3) with no waits on other items. Steps of one
+ * batch run one after another, on whatever streams they are issued. The loss is summed over every circuit; each circuit gets its own
  * gradient. Per step: 4 kernels and one memset; capturable in a CUDA graph. */
 typedef struct qf_batch qf_batch;
 
 /* Build a batched launch. circuits[i] must be planned with QF_PATH_FUSED as
- * round programs (qf_plan_info: tile_bits >= 7, RZ/RY rotations, CZ on
- * neighbouring qubits; host_only plans are fine); batch[i] >= 1 samples of
+ * round programs (at least 7 qubits and qf_plan_info: tile_bits >= 7, RZ/RY
+ * rotations, CZ on neighbouring qubits; host_only plans are fine); batch[i] >= 1 samples of
  * circuit i; obs[i] its observable; loss_kind QF_LOSS_SUM or QF_LOSS_MSE
  * (mean over each circuit's samples, summed over circuits). Allocates the
  * batch's device tables; the circuits must outlive the batch and not be

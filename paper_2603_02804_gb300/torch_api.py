@@ -98,7 +98,7 @@ class Simulator:
         return qfuse.qf_graph_stats(self.handle)
 
     def _stream(self):
-        # the handle alone: a Stream object of the device takes 3.4 us of a 37 us step (n = 4)
+        # the handle alone: a Stream object of the device takes 3.4 us of a 37 us step (n = 4; now 26)
         i = self.device.index
         return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device() if i is None else i)
 

@@ -2254,7 +2254,9 @@ cudaError_t launch_pass(bool bwd, const PassArgs& a, cudaStream_t st, int fwd_ct
   } while (0)
   // one CTA per SM at most: the adjoint's registers need not leave room for two
   // (the two-CTA instance of runtime tile sizes spills: n = 8, d = 20, 64 samples
-  // 102 us a step against 96)
+  // 102 us a step against 96; that of 12-qubit tiles does not, but with 144
+  // registers instead of 128 n = 12, 64 samples takes 81.9 us against 83.6 and a
+  // ring of 13, 37 samples 18.5 us a pass against 18.8)
   const bool alone = grid <= n_sm;
   if (half && bwd) {
     if (rx) QF_RUN(pass_kernel<true, true, true, 2, 0, 1>);
@@ -2271,6 +2273,7 @@ cudaError_t launch_pass(bool bwd, const PassArgs& a, cudaStream_t st, int fwd_ct
     if (alone && !k12 && !rx) QF_RUN(pass_kernel<true, true, false, 1>);
     if (rx && k12) QF_RUN(pass_kernel<true, true, true, 2, 12>);
     if (rx) QF_RUN(pass_kernel<true, true, true>);
+    if (k12 && alone) QF_RUN(pass_kernel<true, true, false, 1, 12>);
     if (k12) QF_RUN(pass_kernel<true, true, false, 2, 12>);
     QF_RUN(pass_kernel<true, true>);
   }

@@ -293,11 +293,15 @@ __device__ __forceinline__ void apply_pending(uint32_t D, float2 (&r)[NR], float
 // rotations are one scale of the state, multiplied into the 16 phases of the
 // round's diagonal, which the kernel applies anyway. q is rounded before the
 // scale is made from it, so that the norm is kept; a large q costs no accuracy,
-// as the scaled result is rounded once. Where any of the four has |tan(w/2)| >
-// kMaxTan, the round runs twice, by half the angles (|q| <= 1) and with the
-// diagonal once: 1 % of the rounds for uniform angles, and the scale of a round
-// stays above 2^-32 (a branch that repeats only the rotations made every round
-// 8 % slower: registers spill). Three shears (3 FMAs per component) need no scale and
+// as the scaled result is rounded once. The scale of a round stays above 2^-32:
+// where the four squared cosines multiply to less than kMinShrink = 2^-64 (a
+// round of four angles within 0.008 of pi, or of two that are pi in float32), the
+// rotations run twice, by half the angles (|q| <= 1). Their second run is a branch
+// at an edge of the round's block (before it in the forward, after it in the
+// adjoint): in the middle it cost every adjoint round 3 %. A step with every
+// angle at pi against uniform angles: n = 12, d = 20, 256 samples 267 us against
+// 211; ring of RX, RY, RZ, n = 12, d = 10, 256 samples 256 against 200 (a second run of the whole
+// round, where any |tan(w/2)| > 256: 339 against 216, 330 against 200). Three shears (3 FMAs per component) need no scale and
 // were slower: training step of n = 20, d = 24, 64 samples 28.35 -> 25.10 ms, of
 // n = 12, d = 20, 256 samples 268 -> 237 us (with the pending links below). A
 // pending Z_R turns the rotation by w into one by -w, i.e. q into -q.
@@ -395,7 +399,7 @@ __device__ __forceinline__ void diag_bwd(float2 (&p)[16], float2 (&l)[16], const
 // the reduced sum undoes it (the table's factor). All four values before the
 // rotations, and psi's rotations before lambda's, need fewer registers at a time
 // than rotation by rotation: adjoint of n = 20, d = 24, 64 samples 1.258 -> 1.244
-// ms a launch.
+// ms a launch. (A steep round takes them before its first run.)
 template <int R, bool RX, int NR>
 __device__ __forceinline__ float grad_T(const float2 (&p)[NR], const float2 (&l)[NR], uint32_t a, bool rx) {
   float g;
@@ -803,7 +807,6 @@ template <bool ROWS>
 struct PassSharedT {
   StepPar par[2];
   float rows[ROWS ? kThreads / 32 : 1][32][8];  // round adjoints: a round's values of each lane
-  float4 ident[8];             // the diagonal of a round's run that has none
   uint32_t ticket;             // the CTA's finishing order (loss on the last CTA)
   uint32_t lg[256];
   float red[2][kThreads / 32][kMaxStepSlots];
@@ -874,7 +877,6 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
       sh.gqub[tid] = q.x | q.y << 8 | q.z << 16 | q.w << 24 |
                      (q.y == q.x + 1 && q.z == q.x + 2 && q.w == q.x + 3 ? kContig : 0u);
     }
-    if (ROUNDS && tid < 8) sh.ident[tid] = make_float4(1.f, 0.f, 1.f, 0.f);
   }
   __syncthreads();
   for (int i = tid; i < (1 << (K - kRegBits)); i += nthr) {
@@ -1126,37 +1128,37 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
         const uint32_t pos[4] = {gp.x, gp.y, gp.z, gp.w};
         tc_rounds(*tc, P, nr, tc->bsm + (size_t)sb * kMaxStepRounds * kTcBFloats, gb, pos, a.n_eff, r, ph, tid);
       } else {
-      // a round whose rotations are steep runs twice (see rot_T): the forward
-      // with its diagonal and links the second time, the adjoint the first
-      bool again = false;
+      // a round of steep rotations runs them twice (see rot_T)
 #pragma unroll 1
-      for (int k = 0; k < nr;) {
+      for (int k = 0; k < nr; ++k) {
+        const bool steep = P.v[k][0].y < 0.f;
         if (!BWD) {
           const uint4 lk = P.rec[k * (kFwdRoundWords / 4) + 1];  // links, bbits, rx mask, leaving links
-          const bool pre = P.v[k][0].y < 0.f && !again;
+          if (steep) {
+            rots<RX>(r, P.v[k], D, lk.z);
+            if constexpr (H) rot_fwd_half<RX>(r, pend_q(P.v[k][3].x, (D >> 3) & 1u), h, (lk.z >> 3) & 1u);
+          }
           rots<RX>(r, P.v[k], D, lk.z);
           if constexpr (H) rot_fwd_half<RX>(r, pend_q(P.v[k][3].x, (D >> 3) & 1u), h, (lk.z >> 3) & 1u);
-          apply_diag(r, pre ? sh.ident : &P.v[k][4 + (H ? 4 * h : 0)]);
-          if (!pre) {
-            chain_pending(lk.x, rgb, lgb, g12, nq, qubits, D);
-            pend ^= lk.w;
-            ++k;
-          }
-          again = pre;
+          apply_diag(r, &P.v[k][4 + (H ? 4 * h : 0)]);
+          chain_pending(lk.x, rgb, lgb, g12, nq, qubits, D);
+          pend ^= lk.w;
         } else {
           const uint4 lk = P.rec[k * (kBwdRoundWords / 4) + 2];  // links, bbits, rx mask, leaving links
-          if (!again) {
-            chain_pending(lk.x, rgb, lgb, g12, nq, qubits, D);
-            pend ^= lk.w;
-          }
+          chain_pending(lk.x, rgb, lgb, g12, nq, qubits, D);
+          pend ^= lk.w;
           float v[8];
-          if constexpr (H) diag_bwd(r, l, again ? sh.ident : &P.v[k][4 + 4 * h], v, h);
-          else diag_bwd(r, l, again ? sh.ident : &P.v[k][4], v);
+          if constexpr (H) diag_bwd(r, l, &P.v[k][4 + 4 * h], v, h);
+          else diag_bwd(r, l, &P.v[k][4], v);
           if constexpr (RX && !H) {
             item_bwd<0>(r, l, P.v[k][0].x, D & 1u, v[4], lk.z & 1u);
             item_bwd<1>(r, l, P.v[k][1].x, (D >> 1) & 1u, v[5], (lk.z >> 1) & 1u);
             item_bwd<2>(r, l, P.v[k][2].x, (D >> 2) & 1u, v[6], (lk.z >> 2) & 1u);
             item_bwd<3>(r, l, P.v[k][3].x, (D >> 3) & 1u, v[7], (lk.z >> 3) & 1u);
+            if (steep) {  // (here it spills 24 bytes, after the reduction 48)
+              rots<RX>(r, P.v[k], D, lk.z);
+              rots<RX>(l, P.v[k], D, lk.z);
+            }
           } else {
             v[4] = grad_T<0, RX>(r, l, D & 1u, lk.z & 1u);
             v[5] = grad_T<1, RX>(r, l, (D >> 1) & 1u, (lk.z >> 1) & 1u);
@@ -1181,7 +1183,6 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
             sum = rows8(v, lanes, lane, sh.rows[warp]);
             owner = (lane & (lanes - 1)) < 8;
           }
-          owner = owner && !again;  // a round's first run has its values
           if (owner) {
             const int32_t term =
                 reinterpret_cast<const int32_t*>(&P.rec[k * (kBwdRoundWords / 4)])[idx];
@@ -1193,8 +1194,15 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
               a.g_part[tile * a.n_slots + term] = (double)(0.5f * sum);
             }
           }
-          again = P.v[k][0].y < 0.f && !again;
-          k += again ? 0 : 1;
+          if ((H || !RX) && steep) {
+            if constexpr (H) {
+              const float q3 = pend_q(P.v[k][3].x, (D >> 3) & 1u);
+              rot_fwd_half<RX>(r, q3, h, (lk.z >> 3) & 1u);
+              rot_fwd_half<RX>(l, q3, h, (lk.z >> 3) & 1u);
+            }
+            rots<RX>(r, P.v[k], D, lk.z);
+            rots<RX>(l, P.v[k], D, lk.z);
+          }
         }
       }
       if ((op.x >> kStepFlushBit) & 1u) {
@@ -1659,7 +1667,8 @@ __device__ double diag_angle(const double (&phi)[4], uint32_t bbits, int m, bool
 
 // One round's parameters by a half-warp (e: lane in it), float32 or (complex128
 // plans) float64: lanes 0..3 take the 4 rotations, lanes 4..11 two phases of
-// the diagonal each, one sincos per lane (see rot_T).
+// the diagonal each, one sincos per lane (see rot_T). Float64 has the exponents
+// for any four tangents (at most 2^54 each), so only complex64 rounds run twice.
 __device__ void round_params(const PrepArgs& a, bool on, bool fwd, int64_t r, const int32_t* rec,
                              const RoundTerm* rt, int e, int lane) {
   double ang = 0.0;
@@ -1678,11 +1687,15 @@ __device__ void round_params(const PrepArgs& a, bool on, bool fwd, int64_t r, co
   double c, s;
   sincos_prep(ang, &s, &c);
   const int half = lane & 16;
-  const bool steep = e < 4 && fabs(s) > kMaxTan * fabs(c);
+  const bool f64 = a.rpf64 || a.rpb64;
+  // the rotations shrink the norm by the product of their cosines
+  float shrink = e < 4 ? (float)(c * c) : 1.f;
+  shrink *= __shfl_xor_sync(0xffffffffu, shrink, 1);
+  shrink *= __shfl_xor_sync(0xffffffffu, shrink, 2);
+  const bool steep = !f64 && e < 4 && shrink < kMinShrink;
   const bool twice = ((__ballot_sync(0xffffffffu, steep) >> half) & 15u) != 0;
   const uint32_t neg = __popc((__ballot_sync(0xffffffffu, odd) >> half) & 15u) & 1u;
   double q = e < 4 ? s / (twice ? 1.0 + c : c) : 0.0;  // tan(w/4) = sin(w/2) / (1 + cos(w/2))
-  const bool f64 = a.rpf64 || a.rpb64;
   if (!f64) q = (double)(float)q;
   double Q[4], S = 1.0;
 #pragma unroll
@@ -1709,7 +1722,7 @@ __device__ void round_params(const PrepArgs& a, bool on, bool fwd, int64_t r, co
     if (!fwd) q = -q;
     if (f64) {
       out64->q[e] = q;
-      out64->g[e] = twice ? -g : g;
+      out64->g[e] = g;
     } else {
       out[e] = make_float4((float)q, (float)(twice ? -all : all), (float)g, 0.f);
     }

@@ -194,8 +194,9 @@ __device__ __forceinline__ void pending64(uint32_t D, double2 (&r)[16], double2 
 
 // One rotation on register bit R, two FMAs per real component: the rotation by
 // w over cos(w/2), q = tan(w/2) (see fused.cu's rot_T). The cosines are a scale
-// of the round's diagonal; a round with a steep rotation runs twice by half
-// the angles. Against three shears, and with the diagonal's terms from
+// of the round's diagonal; |q| <= 2^54, whose products float64 holds (running
+// rounds with |q| > 256 twice by half the angles took a step with every angle at
+// pi, n = 12, d = 10, 256 samples, from 3,270 to 5,280 us). Against three shears, and with the diagonal's terms from
 // complement differences: step of n = 12, d = 10, 256 samples 4,296 -> 3,328 us,
 // as these kernels are bound by FP64 issue.
 template <int R>
@@ -541,14 +542,10 @@ __global__ void __launch_bounds__(kThreads, 1) pass64_kernel(const PassArgs64 a)
         }
       }
       uint32_t D = 0;
-      // a round with a steep rotation runs twice: the forward with its diagonal
-      // and links the second time, the adjoint the first
-      bool again = false;
 #pragma unroll 1
-      for (int k = 0; k < nr;) {
+      for (int k = 0; k < nr; ++k) {
         const size_t rr = (size_t)op.y + k;
         const RoundPar64& v = a.rpar[rr];
-        const bool steep = v.g[0] < 0.0;
         if (!BWD) {
           const uint4 lk = __ldg(a.rounds + rr * (kFwdRoundWords / 4) + 1);
           // the items' rotation terms (-1: absent) in words 12..15
@@ -557,34 +554,23 @@ __global__ void __launch_bounds__(kThreads, 1) pass64_kernel(const PassArgs64 a)
           rot_fwd64<1>(r, v.q[1], (D >> 1) & 1u, (int)ty.y >= 0, RX && ((lk.z >> 1) & 1u));
           rot_fwd64<2>(r, v.q[2], (D >> 2) & 1u, (int)ty.z >= 0, RX && ((lk.z >> 2) & 1u));
           rot_fwd64<3>(r, v.q[3], (D >> 3) & 1u, (int)ty.w >= 0, RX && ((lk.z >> 3) & 1u));
-          again = steep && !again;
-          if (!again) {
-            diag64(r, v.ph);
-            chain64(lk.x, gb, pos, a.n_eff, D);
-            ++k;
-          }
+          diag64(r, v.ph);
+          chain64(lk.x, gb, pos, a.n_eff, D);
         } else {
           const uint4 lk = __ldg(a.rounds + rr * (kBwdRoundWords / 4) + 2);
           const uint4 ty = __ldg(a.rounds + rr * (kBwdRoundWords / 4) + 1);
+          chain64(lk.x, gb, pos, a.n_eff, D);
           double gv[8];
-          if (!again) {
-            chain64(lk.x, gb, pos, a.n_eff, D);
-            diag_terms64(r, l, gv);
-            diag64(r, v.ph);
-            diag64(l, v.ph);
-          }
+          diag_terms64(r, l, gv);
+          diag64(r, v.ph);
+          diag64(l, v.ph);
           rot_bwd64<0>(r, l, v.q[0], D & 1u, gv[4], (int)ty.x >= 0, RX && (lk.z & 1u));
           rot_bwd64<1>(r, l, v.q[1], (D >> 1) & 1u, gv[5], (int)ty.y >= 0, RX && ((lk.z >> 1) & 1u));
           rot_bwd64<2>(r, l, v.q[2], (D >> 2) & 1u, gv[6], (int)ty.z >= 0, RX && ((lk.z >> 2) & 1u));
           rot_bwd64<3>(r, l, v.q[3], (D >> 3) & 1u, gv[7], (int)ty.w >= 0, RX && ((lk.z >> 3) & 1u));
-          if (again) {  // the first run has the round's values
-            again = false;
-            ++k;
-            continue;
-          }
           int idx;
           double sum = butterfly8_64(gv, lanes, lane, idx);
-          if (idx >= 4) sum *= fabs(v.g[idx - 4]);
+          if (idx >= 4) sum *= v.g[idx - 4];
           const bool owner = (lane & ((lanes >> 3) - 1)) == 0;
           const int32_t term = __ldg(reinterpret_cast<const int32_t*>(a.rounds + rr * (kBwdRoundWords / 4)) + idx);
           if (Tt >= 32) {
@@ -595,8 +581,6 @@ __global__ void __launch_bounds__(kThreads, 1) pass64_kernel(const PassArgs64 a)
           } else if (owner && active && term >= 0) {
             a.g_part[tile * a.n_slots + term] = 0.5 * sum;
           }
-          again = steep;
-          if (!again) ++k;
         }
       }
       pending64<BWD>(D, r, l);

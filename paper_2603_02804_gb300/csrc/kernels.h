@@ -56,8 +56,8 @@ struct PassArgs {
 
 // Parameters of one round of a complex128 round program, as the complex64 ones
 // (kRoundPar): the 4 items' rotations q, the factors of their gradient values
-// (negative: the round runs twice) and the diagonal as a phase per register
-// index, times the scale and sign that the rotations leave out.
+// and the diagonal as a phase per register index, times the scale and sign that
+// the rotations leave out.
 struct RoundPar64 {
   double q[4];
   double g[4];

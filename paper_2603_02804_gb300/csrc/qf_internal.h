@@ -59,7 +59,7 @@ constexpr int kBwdRoundWords = 12;
 constexpr int kMaxStepRounds = 4;   // 8 gradient values per round
 // Parameters of one round of a complex64 round program, in float4: [0, 4) the 4
 // items' rotations, x = q and y = the factor of the adjoint's gradient values of
-// the rotations (negative: the round runs twice), z = that of the item's own
+// the rotations (negative: they run twice), z = that of the item's own
 // where the values are taken item by item; [4, 12) the round's diagonal,
 // i.e. the 4 RZ runs (and the CZ links between register bits) merged into one
 // phase per register index, two per float4, times the scale and sign that the
@@ -68,7 +68,7 @@ constexpr int kMaxStepRounds = 4;   // 8 gradient values per round
 // fills them with 16 lanes per round; complex128 programs hold the same in
 // float64 (RoundPar64).
 constexpr int kRoundPar = 12;
-constexpr double kMaxTan = 256.0;   // largest |tan(w/2)| of a round that runs its rotations once
+constexpr float kMinShrink = 0x1p-64f;  // product of cos^2(w/2) below which a complex64 round's rotations run twice
 
 // Source / destination codes of a pass.
 enum : int32_t {

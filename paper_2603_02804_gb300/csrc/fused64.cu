@@ -16,7 +16,8 @@
 // adjoint (psi and lambda) takes 128 KiB. One CTA per SM (8 warps) keeps the
 // FP64 pipe busy; the launch bound lets the 16 + 16 double2 registers of the
 // adjoint step stay in registers. A launch of few tiles gets smaller CTAs, and
-// below one tile per SM a cluster of two CTAs shares a tile (launch_pass64).
+// a cluster of two CTAs shares a 12-qubit tile where that evens out the SMs
+// (launch_pass64).
 //
 // Shared-memory layout: amplitude with local index i lives at
 // i ^ ((i >> 4) & 7). Eight 16-byte amplitudes fill the 32 banks, and a
@@ -841,14 +842,20 @@ cudaError_t launch_pass64(bool bwd, const PassArgs64& a, cudaStream_t st) {
   // Each of an SM's four schedulers has its own FP64 lanes and a warp keeps them
   // busy alone, so the work should sit on all schedulers: CTAs shrink to one tile
   // (one warp at least) while that leaves SMs without one, and two CTAs share a
-  // 12-qubit tile where the busiest SM's part of a tile, ceil(CTAs / SMs) /
-  // 2^split, falls by it. n = 12, d = 10: step of 64 samples (split) 980 us, of
-  // 128 (one CTA per tile and SM) 1,690 us. (Four or eight CTAs per tile gave
-  // nothing more: that leaves schedulers idle.)
+  // 12-qubit tile. Up to one tile per two SMs both directions gain (152 SMs, n =
+  // 12, d = 10, 64 samples: forward 462 -> 304 us, step 1,657 -> 981). Beyond, an
+  // adjoint launch gains wherever the busiest SM's part of a tile, ceil(CTAs / SMs)
+  // / 2^split, falls by it (adjoint of 160 to 228 samples 2,385 -> 1,845 us, of 500
+  // 4,772 -> 4,203, of 2,048 16,718 -> 16,037; where it does not fall, 0.5 % slower).
+  // A forward launch gains with one tile too many only (153 samples 891 -> 750 us);
+  // its last wave's halves sit two on an SM, and everywhere else it loses 4 % (160
+  // to 228 samples 892 -> 923, 500 1,756 -> 1,825, 2,048 6,083 -> 6,342): not split.
+  // (Four or eight CTAs per tile gave nothing more: that leaves schedulers idle.)
   int thr = kThreads;
   while (thr > 32 && thr > (1 << tl2) && (total_tiles << tl2) < (int64_t)thr * n_sm) thr >>= 1;
   const int64_t whole = (total_tiles + n_sm - 1) / n_sm, halves = (2 * total_tiles + n_sm - 1) / n_sm;
-  const int split = thr == kThreads && thr == 1 << tl2 && halves < 2 * whole ? 1 : 0;
+  const bool evens = bwd ? halves < 2 * whole : 2 * total_tiles <= n_sm;
+  const int split = thr == kThreads && thr == 1 << tl2 && evens ? 1 : 0;
   PassArgs64 arg = a;
   arg.split = split;
   thr >>= split;

@@ -407,8 +407,12 @@ qf_status qf_graph_stats(const qf_circuit* c, int64_t* recorded, int64_t* replay
  * a cluster of CTAs that shares its tiles (by one CTA where a sample is one
  * tile), which runs the item's fused forward passes, its dL/dE and its fused
  * adjoint passes (Secs. 3.2-3.3) with no waits on other items. Steps of one
- * batch run one after another, on whatever streams they are issued. The loss is summed over every circuit; each circuit gets its own
- * gradient. Per step: 4 kernels and one memset; capturable in a CUDA graph. */
+ * batch, issued directly or by qf_batch_graph_launch, run one after another, on
+ * whatever streams and from whatever threads they are issued. A step that the
+ * caller captures into a graph of its own is not part of that order: the caller
+ * orders its replays against other steps on the same workspace. The loss is
+ * summed over every circuit; each circuit gets its own gradient. Per step: 4
+ * kernels and one memset; capturable in a CUDA graph. */
 typedef struct qf_batch qf_batch;
 
 /* Build a batched launch. circuits[i] must be planned with QF_PATH_FUSED as

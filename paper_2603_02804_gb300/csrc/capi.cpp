@@ -10,6 +10,7 @@
 #include <cstdint>
 #include <exception>
 #include <map>
+#include <mutex>
 #include <new>
 #include <stdexcept>
 #include <string>
@@ -1827,16 +1828,19 @@ struct qf_batch {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   // the last step's end: every step of a batch writes the same workspace, so
-  // one issued on another stream waits for it
+  // the next one waits for it
   cudaEvent_t done = nullptr;
-  cudaStream_t last = nullptr;
   bool stepped = false;
+  std::mutex mu;  // held over a step's wait, launches and record
 };
 
 namespace {
 
-// Order a step on st after the batch's previous one (on another stream), and
-// mark its end. Steps under capture are ordered by whoever replays them.
+// Order a step on st after the batch's previous one, and mark its end. The wait
+// is made whatever the stream's handle: the same one may name another stream (a
+// new one in the place of a destroyed one, or another thread's per-thread
+// stream), and on the stream itself it costs nothing. Steps under capture are
+// ordered by whoever replays them.
 bool batch_capturing(cudaStream_t st) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
@@ -1846,13 +1850,12 @@ bool batch_capturing(cudaStream_t st) {
   return cs != cudaStreamCaptureStatusNone;
 }
 cudaError_t batch_begin(qf_batch* b, cudaStream_t st) {
-  if (!b->stepped || b->last == st || batch_capturing(st)) return cudaSuccess;
+  if (!b->stepped || batch_capturing(st)) return cudaSuccess;
   return cudaStreamWaitEvent(st, b->done, 0);
 }
 cudaError_t batch_end(qf_batch* b, cudaStream_t st) {
   if (batch_capturing(st)) return cudaSuccess;
   const cudaError_t e = cudaEventRecord(b->done, st);
-  b->last = st;
   b->stepped = e == cudaSuccess;
   return e;
 }
@@ -2188,6 +2191,7 @@ qf_status qf_batch_train_step(qf_batch* b, const float* theta_d, const float* x_
   a.lterm = reinterpret_cast<double*>(a.ws + b->lterm_off);
   a.queue = reinterpret_cast<int32_t*>(a.ws + b->queue_off);
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
+  const std::lock_guard<std::mutex> lock(b->mu);
   QF_CU(batch_begin(b, st));
   QF_CU(qf::launch_batch(a, b->clusters, b->cluster_size, b->prep_total, b->n_grad_out, st));
   QF_CU(batch_end(b, st));
@@ -2224,6 +2228,7 @@ qf_status qf_batch_graph_capture(qf_batch* b, const float* theta_d, const float*
 qf_status qf_batch_graph_launch(qf_batch* b, void* stream) {
   if (!b || !b->exec) return fail(QF_ERR_INVALID_ARG, "no captured graph (call qf_batch_graph_capture)");
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
+  const std::lock_guard<std::mutex> lock(b->mu);
   QF_CU(batch_begin(b, st));
   QF_CU(cudaGraphLaunch(b->exec, st));
   QF_CU(batch_end(b, st));

@@ -407,8 +407,10 @@ qf_status qf_graph_stats(const qf_circuit* c, int64_t* recorded, int64_t* replay
  * a cluster of CTAs that shares its tiles (by one CTA where a sample is one
  * tile), which runs the item's fused forward passes, its dL/dE and its fused
  * adjoint passes (Secs. 3.2-3.3) with no waits on other items. Steps of one
- * batch, issued directly or by qf_batch_graph_launch, run one after another, on
- * whatever streams and from whatever threads they are issued. A step that the
+ * batch on one workspace, issued directly or by qf_batch_graph_launch, run one
+ * after another, on whatever streams and from whatever threads they are issued;
+ * steps on workspaces of their own may overlap (on up to four; with more, all
+ * are ordered). A step that the
  * caller captures into a graph of its own is not part of that order: the caller
  * orders its replays against other steps on the same workspace. The loss is
  * summed over every circuit; each circuit gets its own gradient. Per step: 4

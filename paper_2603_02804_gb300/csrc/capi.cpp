@@ -1827,20 +1827,29 @@ struct qf_batch {
   int clusters = 0, cluster_size = 0;  // of the persistent kernel
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
-  // the last step's end: every step of a batch writes the same workspace, so
-  // the next one waits for it
-  cudaEvent_t done = nullptr;
-  bool stepped = false;
-  std::mutex mu;  // held over a step's wait, launches and record
+  void* graph_ws = nullptr;  // the captured step's workspace
+  // The end of the last step on each workspace: the next step on the same memory
+  // waits for it. Once there are more workspaces than entries, the oldest entry
+  // is taken over and every step waits for all of them (`full`), so that a step
+  // that lost its entry lies before one that has one.
+  struct Step {
+    const char* ws = nullptr;
+    cudaEvent_t done = nullptr;
+  };
+  std::array<Step, 4> steps;
+  size_t oldest = 0;
+  bool full = false;
+  std::mutex mu;  // held over a step's waits, launches and record
 };
 
 namespace {
 
-// Order a step on st after the batch's previous one, and mark its end. The wait
-// is made whatever the stream's handle: the same one may name another stream (a
-// new one in the place of a destroyed one, or another thread's per-thread
-// stream), and on the stream itself it costs nothing. Steps under capture are
-// ordered by whoever replays them.
+// Order a step on st after those on the same memory, and mark its end. Steps on
+// workspaces of their own share nothing and may overlap. The wait is made
+// whatever the stream's handle: the same one may name another stream (a new one
+// in the place of a destroyed one, or another thread's per-thread stream), and
+// on the stream itself it costs nothing. Steps under capture are ordered by
+// whoever replays them.
 bool batch_capturing(cudaStream_t st) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
@@ -1849,14 +1858,33 @@ bool batch_capturing(cudaStream_t st) {
   }
   return cs != cudaStreamCaptureStatusNone;
 }
-cudaError_t batch_begin(qf_batch* b, cudaStream_t st) {
-  if (!b->stepped || batch_capturing(st)) return cudaSuccess;
-  return cudaStreamWaitEvent(st, b->done, 0);
-}
-cudaError_t batch_end(qf_batch* b, cudaStream_t st) {
+cudaError_t batch_begin(qf_batch* b, const void* ws, cudaStream_t st) {
   if (batch_capturing(st)) return cudaSuccess;
-  const cudaError_t e = cudaEventRecord(b->done, st);
-  b->stepped = e == cudaSuccess;
+  const char* w = static_cast<const char*>(ws);
+  bool entry = false;
+  for (const qf_batch::Step& s : b->steps) entry = entry || s.ws == w || !s.ws;
+  b->full = b->full || !entry;
+  for (const qf_batch::Step& s : b->steps) {
+    const bool shares = s.ws && s.ws < w + b->ws_total && w < s.ws + b->ws_total;
+    if (!shares && !(s.ws && b->full)) continue;
+    const cudaError_t e = cudaStreamWaitEvent(st, s.done, 0);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+cudaError_t batch_end(qf_batch* b, const void* ws, cudaStream_t st) {
+  if (batch_capturing(st)) return cudaSuccess;
+  qf_batch::Step* to = nullptr;
+  for (qf_batch::Step& s : b->steps)
+    if (s.ws == ws) to = &s;
+  for (qf_batch::Step& s : b->steps)
+    if (!to && !s.ws) to = &s;
+  if (!to) {
+    to = &b->steps[b->oldest];
+    b->oldest = (b->oldest + 1) % b->steps.size();
+  }
+  const cudaError_t e = cudaEventRecord(to->done, st);
+  if (e == cudaSuccess) to->ws = static_cast<const char*>(ws);
   return e;
 }
 
@@ -1869,8 +1897,10 @@ void batch_free(qf_batch* b) {
   if (b->exec) cudaGraphExecDestroy(b->exec);
   if (b->graph) cudaGraphDestroy(b->graph);
   if (b->d_tables) cudaFree(b->d_tables);
-  if (b->done) cudaEventDestroy(b->done);
-  b->done = nullptr;
+  for (qf_batch::Step& s : b->steps) {
+    if (s.done) cudaEventDestroy(s.done);
+    s.done = nullptr;
+  }
   b->exec = nullptr;
   b->graph = nullptr;
   b->d_tables = nullptr;
@@ -1976,7 +2006,10 @@ qf_status qf_batch_create(int32_t n_circuits, qf_circuit* const* circuits, const
         b->cluster_size = cs;
       }
     }
-    if (b->clusters <= 0 || cudaEventCreateWithFlags(&b->done, cudaEventDisableTiming) != cudaSuccess) {
+    bool holds = b->clusters > 0;
+    for (qf_batch::Step& s : b->steps)
+      holds = holds && cudaEventCreateWithFlags(&s.done, cudaEventDisableTiming) == cudaSuccess;
+    if (!holds) {
       cudaGetLastError();
       batch_free(b);
       delete b;
@@ -2192,9 +2225,9 @@ qf_status qf_batch_train_step(qf_batch* b, const float* theta_d, const float* x_
   a.queue = reinterpret_cast<int32_t*>(a.ws + b->queue_off);
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
   const std::lock_guard<std::mutex> lock(b->mu);
-  QF_CU(batch_begin(b, st));
+  QF_CU(batch_begin(b, ws_d, st));
   QF_CU(qf::launch_batch(a, b->clusters, b->cluster_size, b->prep_total, b->n_grad_out, st));
-  QF_CU(batch_end(b, st));
+  QF_CU(batch_end(b, ws_d, st));
   return QF_OK;
 }
 
@@ -2221,6 +2254,7 @@ qf_status qf_batch_graph_capture(qf_batch* b, const float* theta_d, const float*
   }
   if (e != cudaSuccess) return fail(QF_ERR_CUDA, std::string("stream capture failed: ") + cudaGetErrorString(e));
   b->graph = g;
+  b->graph_ws = ws_d;
   QF_CU(cudaGraphInstantiate(&b->exec, g, 0));
   return QF_OK;
 }
@@ -2229,9 +2263,9 @@ qf_status qf_batch_graph_launch(qf_batch* b, void* stream) {
   if (!b || !b->exec) return fail(QF_ERR_INVALID_ARG, "no captured graph (call qf_batch_graph_capture)");
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
   const std::lock_guard<std::mutex> lock(b->mu);
-  QF_CU(batch_begin(b, st));
+  QF_CU(batch_begin(b, b->graph_ws, st));
   QF_CU(cudaGraphLaunch(b->exec, st));
-  QF_CU(batch_end(b, st));
+  QF_CU(batch_end(b, b->graph_ws, st));
   return QF_OK;
 }
 

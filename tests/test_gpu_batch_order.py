@@ -49,3 +49,44 @@ def test_threads_on_their_own_per_thread_stream(batch):
     torch.cuda.synchronize()
     for out in outs:
         assert all(torch.equal(a, b) for a, b in zip(out, ref))
+
+
+def test_steps_with_workspaces_of_their_own_overlap(batch):
+    """A step on another stream and workspace does not wait for one that is
+    still queued behind 0.5 s of other work."""
+    bt, inputs, ref = batch
+    ws2 = torch.empty_like(bt.ws)
+    outs = [bt.outputs(), bt.outputs()]
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    step(bt, inputs, outs[1], ws2, s2)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s1):
+        torch.cuda._sleep(1_000_000_000)  # cycles
+    step(bt, inputs, outs[0], bt.ws, s1)
+    step(bt, inputs, outs[1], ws2, s2)
+    s2.synchronize()
+    assert not s1.query()
+    torch.cuda.synchronize()
+    for out in outs:
+        assert all(torch.equal(a, b) for a, b in zip(out, ref))
+
+
+def test_more_workspaces_than_the_order_remembers(batch):
+    """Seven workspaces in turn on three streams, each used again later on
+    another stream behind other work, one of them reached by overlapping ranges."""
+    bt, inputs, ref = batch
+    size = bt.ws.numel() + 256
+    spaces = [torch.empty(size, dtype=torch.uint8, device="cuda") for _ in range(7)]
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    outs = [bt.outputs() for _ in range(21)]
+    torch.cuda.synchronize()
+    for k, out in enumerate(outs):
+        s = streams[k % 3]
+        if k % 4 == 0:
+            with torch.cuda.stream(s):
+                torch.cuda._sleep(2_000_000)
+        w = spaces[(k * 5) % 7]
+        step(bt, inputs, out, w[256:] if k % 2 else w, s)
+    torch.cuda.synchronize()
+    for out in outs:
+        assert all(torch.equal(a, b) for a, b in zip(out, ref))

@@ -98,9 +98,13 @@ class Simulator:
         return qfuse.qf_graph_stats(self.handle)
 
     def _stream(self):
-        # the handle alone: a Stream object of the device takes 3.4 us of a 37 us step (n = 4; now 26)
+        # the handle alone, where this PyTorch has the call: a Stream object of the device takes 3.4 us of a
+        # 37 us step (n = 4; now 26)
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is None:
+            return torch.cuda.current_stream(self.device)
         i = self.device.index
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device() if i is None else i)
+        return raw(torch.cuda.current_device() if i is None else i)
 
     def _check(self, theta, x):
         if self.encoding == "state":

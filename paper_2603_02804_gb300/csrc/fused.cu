@@ -2265,11 +2265,11 @@ cudaError_t launch_pass(bool bwd, const PassArgs& a, cudaStream_t st, int fwd_ct
     __VA_ARGS__<<<(unsigned)grid, thr, smem, st>>>(a);                                       \
     return cudaGetLastError();                                                               \
   } while (0)
-  // one CTA per SM at most: the adjoint's registers need not leave room for two
-  // (the two-CTA instance of runtime tile sizes spills: n = 8, d = 20, 64 samples
-  // 102 us a step against 96; that of 12-qubit tiles does not, but with 144
-  // registers instead of 128 n = 12, 64 samples takes 81.9 us against 83.6 and a
-  // ring of 13, 37 samples 18.5 us a pass against 18.8)
+  // one CTA per SM at most: the adjoint's registers need not leave room for two (150
+  // instead of 109: a step of n = 12, d = 20, 64 samples 135 us against 138; a ring
+  // of 13 qubits, d = 31, 37 samples 354 against 362). Rounds on smaller tiles have
+  // no such launches but those of exactly 256 threads per SM: below 128 two threads
+  // share a column, from there on CTAs of 128 outnumber the SMs
   const bool alone = grid <= n_sm;
   if (half && bwd) {
     if (rx) QF_RUN(pass_kernel<true, true, true, 2, 0, 1>);
@@ -2282,8 +2282,6 @@ cudaError_t launch_pass(bool bwd, const PassArgs& a, cudaStream_t st, int fwd_ct
   if (bwd) {
     if (!rounds && alone) QF_RUN(pass_kernel<true, false, false, 1>);
     if (!rounds) QF_RUN(pass_kernel<true, false>);
-    if (rx && alone && !k12) QF_RUN(pass_kernel<true, true, true, 1>);
-    if (alone && !k12 && !rx) QF_RUN(pass_kernel<true, true, false, 1>);
     if (rx && k12) QF_RUN(pass_kernel<true, true, true, 2, 12>);
     if (rx) QF_RUN(pass_kernel<true, true, true>);
     if (k12 && alone) QF_RUN(pass_kernel<true, true, false, 1, 12>);

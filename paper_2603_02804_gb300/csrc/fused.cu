@@ -79,8 +79,8 @@ __device__ __forceinline__ void st_regs(float2* at, const float2 (&r)[NR]) {
 #pragma unroll
   for (int j = 0; j < NR; ++j) at[group_off<B>(j)] = r[j];
 }
-// The group's lowest local bit b is one of these in round programs (K = 7 .. 12:
-// 0, 4, 8 and K - 4; KC = 12: 0, 4, 8). at2: lambda's place (adjoint).
+// The group's lowest local bit b is one of these in round programs (K = 7 .. 11:
+// 0, 4 and K - 4; KC = 12: 0, 4, 8). at2: lambda's place (adjoint).
 template <int KC, bool BWD, int NR>
 __device__ __forceinline__ void ld_group(uint32_t b, const float2* at, const float2* at2, float2 (&r)[NR],
                                          float2 (&l)[NR]) {
@@ -91,11 +91,10 @@ __device__ __forceinline__ void ld_group(uint32_t b, const float2* at, const flo
     switch (b) {
       case 0: QF_LD(0) break;
       case 3: QF_LD(3) break;
-      case 4: QF_LD(4) break;
       case 5: QF_LD(5) break;
       case 6: QF_LD(6) break;
       case 7: QF_LD(7) break;
-      default: QF_LD(8) break;
+      default: QF_LD(4) break;
     }
   }
 #undef QF_LD
@@ -110,11 +109,10 @@ __device__ __forceinline__ void st_group(uint32_t b, float2* at, float2* at2, co
     switch (b) {
       case 0: QF_ST(0) break;
       case 3: QF_ST(3) break;
-      case 4: QF_ST(4) break;
       case 5: QF_ST(5) break;
       case 6: QF_ST(6) break;
       case 7: QF_ST(7) break;
-      default: QF_ST(8) break;
+      default: QF_ST(4) break;
     }
   }
 #undef QF_ST

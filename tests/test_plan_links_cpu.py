@@ -52,7 +52,11 @@ def check_plan(h):
                 if w0 & 15 != pi.OP_STEP:
                     assert pend == 0, "a checkpoint is stored or read with signs pending"
                     continue
-                regs = [pd["gmap"][q] for q in pd["groups"][(w0 >> 4) & 3]]
+                group = pd["groups"][(w0 >> 4) & 3]
+                # the kernels' constant offsets: four consecutive local bits from one of these
+                assert group[0] in ((0, 4, 8) if pd["K"] == 12 else (0, 3, 4, 5, 6, 7))
+                assert group == [group[0] + r for r in range(4)] and group[3] < pd["K"]
+                regs = [pd["gmap"][q] for q in group]
                 check_linear(pend, regs, n, rng)
                 for k in range((w0 >> 8) & 0xFFFF):
                     rec = prog.round_words[(w1 + k) * words:(w1 + k + 1) * words]

@@ -801,10 +801,39 @@ template <class Y>
 __device__ void loss_block(int kind, double* E, const Y* y, int64_t B, double scale, double* loss, double* dLdE,
                            const double* e_part, int tps, int tid, int nthr);
 
+// dL/dE of sample b (a late loss: from the sample's own E, one tile per sample).
+__device__ __forceinline__ double seed_dl(const PassArgs& a, int64_t b) {
+  if (a.dLdE) return a.dLdE[b];
+  return a.loss_kind == 1 ? a.loss_scale * (a.e_part[b] - (double)a.y[b]) : 1.0;
+}
+
+// Round programs seed lambda with dL/dE / 2^e, e its exponent, and multiply the
+// gradient partials by 2^e in float64 (exact, both): a round's scale (rot_T) takes
+// up to 2^64 off the products of lambda and psi, and with a small dL/dE they left
+// float32's range (1e-24 and angles 0.009 from pi: gradients 36 % off).
+__device__ __forceinline__ int grad_exponent(double dl) {
+  const int e = ((__double2hiint(dl) >> 20) & 0x7ff) - 1023;
+  return e > -800 && e < 800 ? e : 0;  // (zero, infinities and NaN go as they are)
+}
+__device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+// A partial v / 2 times 2^e. A float64 product is a latency that the summing warp
+// brings to the step's next barrier: small tiles, whose steps are short, add to the
+// exponent's bits instead (n = 7, d = 20, 64 samples 75.6 -> 74.3 us a step; 12-qubit
+// tiles are slower by it, n = 20, d = 8, 64 samples 8.40 -> 8.46 ms).
+template <bool BITS>
+__device__ __forceinline__ double partial(float v, int e) {
+  if (!BITS) return (double)v * pow2(e - 1);
+  const double d = (double)(0.5f * v);
+  const int hi = __double2hiint(d);
+  const bool number = (uint32_t)(hi & 0x7ff00000) - 0x00100000u < 0x7fe00000u;  // not 0, infinite or NaN
+  return __hiloint2double(number ? hi + e * (1 << 20) : hi, __double2loint(d));
+}
+
 template <bool ROWS>
 struct PassSharedT {
   StepPar par[2];
   float rows[ROWS ? kThreads / 32 : 1][32][8];  // round adjoints: a round's values of each lane
+  int32_t gexp[kThreads >> (kRoundQubits - kRegBits)];  // round adjoints: grad_exponent per tile of the CTA
   uint32_t ticket;             // the CTA's finishing order (loss on the last CTA)
   uint32_t lg[256];
   float red[2][kThreads / 32][kMaxStepSlots];
@@ -862,6 +891,9 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
   const int wpt = Tt >= 32 ? Tt / 32 : 1;  // warps per tile
   const int lanes = Tt < 32 ? Tt : 32;
 
+  // (read here, used after the tile's loads)
+  const bool seeds = BWD && (pd.lam_src == LAM_SEED || pd.lam_src == LAM_SEED_FAR);
+  const double dl = active && (seeds || (BWD && ROUNDS)) ? seed_dl(a, b) : 0.0;
   // (round programs: one op per step, read a step ahead; the first one here)
   uint2 next = make_uint2(0u, 0u);
   if (ROUNDS && pd.op_begin < pd.op_end) next = __ldg(a.ops + pd.op_begin);
@@ -1020,7 +1052,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
     }
     stage_first();
     if (far) {
-      const float scale = (float)(2.0 * a.dLdE[b]);
+      const float scale = (float)(2.0 * dl * (ROUNDS ? pow2(-grad_exponent(dl)) : 1.0));
 #pragma unroll
       for (int it = 0; it < NIT; ++it) {
         const uint32_t xp = g_it(it) ^ a.x_mask;  // the pair's partners: xp and xp ^ 1
@@ -1044,6 +1076,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
 #pragma unroll
     for (int it = 0; it < NIT; ++it) st_pair(tl, p_it(it), __ldcg(reinterpret_cast<const float4*>(src + g_it(it))));
   }
+  if (BWD && ROUNDS && tau == 0) sh.gexp[tile_in_cta] = grad_exponent(dl);
   int sb = 0;  // round programs: the step's staging buffer
   if (ROUNDS && warp == 0) cp_async_wait_all();
   if (TC) {
@@ -1056,13 +1089,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
   __syncthreads();
   if (BWD && pd.lam_src == LAM_SEED) {
     // lambda_M = 2 (dL/dE_b) O psi_M (Eq. 4); (O psi)_x = i^{#Y} (-1)^{|(x^xm)&zm|} psi_{x^xm}
-    float scale = 0.f;
-    if (active) {
-      double dl = 1.0;
-      if (a.dLdE) dl = a.dLdE[b];
-      else if (a.loss_kind == 1) dl = a.loss_scale * (a.e_part[b] - (double)a.y[b]);  // one tile per sample
-      scale = (float)(2.0 * dl);
-    }
+    const float scale = (float)(2.0 * dl * (ROUNDS ? pow2(-grad_exponent(dl)) : 1.0));
 #pragma unroll 1
     for (int it = 0; it < NR; ++it) {
       const uint32_t i = (uint32_t)it * Tt + tau;  // single amplitudes here
@@ -1189,7 +1216,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
               s_red[buf][warp][k * 8 + idx] = sum;
               if (warp == 0) s_slot[buf][k * 8 + idx] = term;
             } else if (active && term >= 0) {
-              a.g_part[tile * a.n_slots + term] = (double)(0.5f * sum);
+              a.g_part[tile * a.n_slots + term] = partial<KC == 0>(sum, sh.gexp[tile_in_cta]);
             }
           }
           if ((H || !RX) && steep) {
@@ -1225,6 +1252,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
         // do, then float64 across tiles
         const int nk = nr * 8;
         const bool first = a.g_first != 0;
+        const double half = pow2(sh.gexp[0] - 1);
         for (int kk = nthr - 1 - tid; kk < nk; kk += nthr) {  // the last warp (warp 0 stages)
           const int32_t term = s_slot[buf][kk];
           if (term < 0) continue;
@@ -1236,7 +1264,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
               sum += (double)sf;
             }
           double* dst = a.g_part + a.g_row * a.n_slots + term;
-          *dst = first ? 0.5 * sum : *dst + 0.5 * sum;
+          *dst = first ? half * sum : *dst + half * sum;
         }
         buf ^= 1;
       } else if (BWD && Tt >= 32) {
@@ -1249,7 +1277,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs& a, const int64_t first_
           if (t2 < total_tiles && term >= 0) {
             float sf = 0.f;
             for (int w = 0; w < wpt; ++w) sf += s_red[buf][tc * wpt + w][kk];
-            a.g_part[t2 * a.n_slots + term] = (double)(0.5f * sf);
+            a.g_part[t2 * a.n_slots + term] = partial<KC == 0>(sf, sh.gexp[KC ? 0 : tc]);
           }
         }
         buf ^= 1;

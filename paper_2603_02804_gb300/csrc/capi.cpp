@@ -1980,8 +1980,8 @@ qf_status qf_batch_create(int32_t n_circuits, qf_circuit* const* circuits, const
     // The persistent kernel's cluster size: a larger one shortens the longest
     // item (which has to end well before the launch, hence the 1.2), a smaller
     // one fits the GPU's SM groups with fewer SMs left over. Units: a round of a
-    // CTA's tiles. 32 circuits of 8 to 16 qubits: 7.73 ms with
-    // clusters of 8, 7.26 with 4 (chosen), 7.45 with 2.
+    // CTA's tiles. 32 circuits of 8 to 16 qubits, up to 60 layers: 7.47 ms with
+    // clusters of 8, 6.97 with 4 (chosen), 7.22 with 2, 13.81 with 1.
     auto tiles_of = [&](int i, int64_t* tps, int64_t* tpc) {
       const qf::FusedPlan& P = b->circ[i]->fp;
       *tps = 1ll << (P.n_eff - P.K);

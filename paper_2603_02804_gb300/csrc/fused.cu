@@ -2057,8 +2057,8 @@ __global__ void batch_prep_kernel(const BatchArgs a, int64_t total) {
 // of CTAs: each pass's tiles are dealt to the CTAs, with a cluster barrier
 // between passes (it also orders their writes to the states). One CTA per
 // sample made the longest item the length of the launch: 32 circuits of 8 to
-// 16 qubits 14.57 -> 7.65 ms. Items of single-tile circuits are then taken by the
-// CTAs one by one. Items never wait on each other.
+// 16 qubits, up to 60 layers, 13.81 ms with clusters of one CTA, 6.97 with four.
+// Items of single-tile circuits are then taken by the CTAs one by one. Items never wait on each other.
 __device__ void run_item(const BatchArgs& a, const BatchItem item, bool wide) {
   namespace cg = cooperative_groups;
   const BatchCircuit& C = a.circ[item.c];

@@ -32,8 +32,10 @@ struct PassArgs {
   uint32_t z_mask;        // observable Z part (global bits)
   uint32_t y_count;       // number of Y factors (phase i^y_count)
   const double* dLdE;     // [B]; null: a late loss (below), the seed's from the sample's own E
+                          // (round programs divide lambda by its power of two and the partials make it good)
   double* e_part;         // [B * tiles per sample]
-  double* g_part;         // [B * tiles per sample][n_slots], or [B][n_slots] when g_accum
+  double* g_part;         // [B * tiles per sample][n_slots]; g_accum: [B * g_ranks][n_slots], a row per sample
+                          // and CTA that takes tiles of it (BatchCircuit::g_ranks <= tiles per sample)
   int32_t n_slots;
   int32_t g_accum;        // round programs: a call's tiles are of one sample, its partials add into row g_row
   int32_t g_first;        // the row's first call stores instead
@@ -152,7 +154,8 @@ inline int64_t g_reduce_scratch(int64_t B, int64_t tps, int64_t n_slots) {
 
 cudaError_t launch_prep(const PrepArgs& a, cudaStream_t st);
 // fwd_ctas: CTAs per SM of the forward round-pass instance (0: 3 when the
-// grid exceeds two CTAs per SM, else 2); the adjoint always runs two.
+// grid exceeds two CTAs per SM, else 2); the adjoint runs two, or one where the
+// launch has no more (12-qubit tiles, generic programs).
 cudaError_t launch_pass(bool bwd, const PassArgs& a, cudaStream_t st, int fwd_ctas = 0);
 // Forward pass on the tensor cores (round programs, 12-qubit tiles).
 cudaError_t launch_pass_tc(const PassArgs& a, cudaStream_t st);

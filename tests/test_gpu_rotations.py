@@ -1,5 +1,5 @@
 """Round programs at the angles where a rotation's reduced form changes: the
-wrap to [-pi, pi], the bit flip beyond pi / 2 and the poles of tan and cot."""
+wrap to [-pi, pi], a tangent of 1 and its poles (steep rounds)."""
 import numpy as np
 import pytest
 import torch
